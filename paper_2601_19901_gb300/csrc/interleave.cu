@@ -192,7 +192,8 @@ __global__ void __launch_bounds__(256) k_interleave(DispConst c, const uint8_t* 
 // Rendered view nearest a on the display-view axis (positions pos[], ties to
 // the later view), from the window of four views around it.
 __device__ __forceinline__ int nearest_view(const float* pos, int nr, float r, float a) {
-    int lo = int(floorf(r * a)) - 2;
+    // clamped as binary32: an offset of any size converts to an index
+    int lo = int(fminf(fmaxf(floorf(r * a), 0.0f), float(nr))) - 2;
     lo = lo > nr - 4 ? nr - 4 : lo;
     lo = lo < 0 ? 0 : lo;
     const int hi = lo + 3 < nr - 1 ? lo + 3 : nr - 1;
