@@ -14,9 +14,14 @@
 // k_interleave_gauss is the Gaussian reconstruction of Sec. 4 (recon 2, 3):
 // per subpixel the mean of the caller's samples, each the nearest rendered
 // view to the subpixel's phase plus the sample's angular offset at the view
-// pixel holding its spatially offset position. It is bound by its nearest-view
-// searches (72 per pixel with crosstalk), not by the gathers (L1 / L2 hits):
-// staging bands of views in shared memory measured slower.
+// pixel holding its spatially offset position: up to 72 view searches and
+// gathers a pixel with crosstalk and eight samples. The searches go through a
+// table of thresholds in shared memory, and a warp's lanes take panel columns
+// a stride apart at which the lens phase repeats, so that they mostly gather
+// from the same view (see there).
+#include <algorithm>
+#include <cmath>
+
 #include "lfdpr_internal.cuh"
 
 namespace lfdpr {
@@ -267,25 +272,245 @@ __device__ __forceinline__ uint32_t gauss_pixel(const DispConst& c, const uint32
     return o;
 }
 
-__global__ void __launch_bounds__(256) k_interleave_gauss(DispConst c, const uint8_t* __restrict__ views,
-                                                          const float* __restrict__ pos,
-                                                          const float* __restrict__ samples, int ns,
-                                                          uint8_t* __restrict__ panel) {
+// The nearest view by a table. On the axis of a = phase + angular offset the
+// nearest view changes at the midpoints of neighbouring positions, which lie
+// at least a quarter of a view apart (a view stays in its interval of half a
+// display view), so a bin an eighth of a view wide holds at most one change:
+// view v below a threshold, v + 1 from it on. A search is then one 8-byte
+// shared load, a comparison and an addition, instead of four positions loaded
+// and compared.
+//
+// The table gives what nearest_view gives, bit for bit. Its thresholds are
+// found with nearest_view itself: the smallest a at which it returns the
+// later view, a few floats around the rounded midpoint (near a midpoint the
+// rounded distances still move one way each, so the answer changes once).
+// That needs neighbouring positions further apart than rounding can confuse:
+// where two views around a bin are less than kGaussApart apart (views placed
+// on the same border of their intervals), or the few steps do not settle a
+// threshold, the block keeps to nearest_view for every pixel.
+constexpr int kGaussBins = 8;          // bins per display view
+constexpr int kGaussMargin = 4;        // display views covered on either side of [0, N]
+constexpr float kGaussApart = 0x1p-12f;
+constexpr int kGaussSteps = 16;
+constexpr int kGaussMaxStride = 64;    // largest column stride between a warp's lanes
+
+struct GaussBin {
+    float from;       // the next view's bytes start here (+inf: not in this bin)
+    uint32_t off;     // byte offset of the bin's first view
+};
+
+__host__ __device__ __forceinline__ int gauss_bins(int n_views) { return kGaussBins * (n_views + 2 * kGaussMargin) + 1; }
+
+// Bin b: a in [b / 8 - 4, (b + 1) / 8 - 4). False if it has no single threshold.
+__device__ __forceinline__ bool gauss_bin(const float* pos, int nr, float r, int b, uint32_t view_bytes, GaussBin& o) {
+    const float lo = float(b) * (1.0f / kGaussBins) - float(kGaussMargin), hi = lo + 1.0f / kGaussBins;
+    int m0 = nearest_view(pos, nr, r, lo);
+    const int m1 = nearest_view(pos, nr, r, hi);
+    if (!LFDPR_IN_BOUNDS(uint32_t(m0), uint32_t(nr), 23) || !LFDPR_IN_BOUNDS(uint32_t(m1), uint32_t(nr), 23)) m0 = m1;
+    o.from = INFINITY;
+    o.off = uint32_t(m0) * view_bytes;
+    bool ok = m1 == m0 || m1 == m0 + 1;
+    for (int m = max(m0 - 1, 0); m <= min(m1, nr - 2); m++) ok &= pos[m + 1] - pos[m] >= kGaussApart;
+    if (!ok || m1 == m0) return ok;
+    float t = 0.5f * (pos[m0] + pos[m1]);   // positive: the positions are apart and not negative
+    int step = 0;
+    if (nearest_view(pos, nr, r, t) >= m1) {
+        for (; step < kGaussSteps; step++) {
+            const float q = __uint_as_float(__float_as_uint(t) - 1u);
+            if (nearest_view(pos, nr, r, q) < m1) break;
+            t = q;
+        }
+    } else {
+        for (; step < kGaussSteps; step++) {
+            t = __uint_as_float(__float_as_uint(t) + 1u);
+            if (nearest_view(pos, nr, r, t) >= m1) break;
+        }
+    }
+    o.from = t;
+    return step < kGaussSteps;
+}
+
+// Panel pixel (x, y) as gauss_pixel, its views found in the table at shared
+// address bins (less the bias of the bin number below): the same view bytes,
+// summed as integers (exact, as the sums of at most 32 bytes are in binary32).
+// The bin number is floor(8 a) + 32, the low bits of one fma rounded down
+// onto 1.5 2^23. mean: 1 / ns where ns is a power of two (the product is then
+// the quotient), else 0.
+constexpr float kGaussMagic = 12582912.0f;              // 1.5 2^23
+constexpr uint32_t kGaussMagicBits = 0x4b400000u;
+template <bool XT>
+__device__ __forceinline__ uint32_t gauss_pixel_table(const DispConst& c, const uint8_t* __restrict__ views,
+                                                      uint32_t bins, uint32_t view_bytes, const float4* smp, int ns,
+                                                      float mean, int x, int y, float sxw, float syh) {
+    constexpr int K = XT ? 3 : 1;
+    const int W = c.W, H = c.H;
+    const float N = float(c.n_views);
+    const float vx = (float(x) + 0.5f) * sxw, vy = (float(y) + 0.5f) * syh;
+    float phi[3][K];   // [channel][own, -1, +1]
+#pragma unroll
+    for (int ch = 0; ch < 3; ch++) {
+        const float p0 = subpixel_phase(c, x, y, ch);
+        phi[ch][0] = p0;
+        if constexpr (XT) {
+            float pm = p0 - 1.0f, pp = p0 + 1.0f;
+            if (pm < 0.0f) pm += N;
+            if (pp >= N) pp -= N;
+            phi[ch][1] = pm;
+            phi[ch][2] = pp;
+        }
+    }
+    uint32_t acc[3][K];
+#pragma unroll
+    for (int ch = 0; ch < 3; ch++)
+#pragma unroll
+        for (int k = 0; k < K; k++) acc[ch][k] = 0u;
+    for (int s = 0; s < ns; s++) {
+        const float4 q = smp[s];
+        int px = int(floorf(vx + q.x)), py = int(floorf(vy + q.y));
+        px = px < 0 ? 0 : (px >= W ? W - 1 : px);
+        py = py < 0 ? 0 : (py >= H ? H - 1 : py);
+        const uint8_t* at = views + 4u * (uint32_t(py) * uint32_t(W) + uint32_t(px));
+#pragma unroll
+        for (int ch = 0; ch < 3; ch++)
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                const float a = phi[ch][k] + q.z;
+                const uint32_t n = __float_as_uint(__fmaf_rd(a, float(kGaussBins), kGaussMagic + float(kGaussBins * kGaussMargin)));
+                float from;
+                uint32_t off;
+                asm("ld.shared.v2.b32 {%0, %1}, [%2];" : "=f"(from), "=r"(off) : "r"(bins + 8u * n));
+                if (a >= from) off += view_bytes;
+                uint64_t p;   // at + off in one instruction
+                asm("mad.wide.u32 %0, %1, 1, %2;" : "=l"(p) : "r"(off), "l"(at));
+                acc[ch][k] += __ldg(reinterpret_cast<const uint8_t*>(p) + ch);
+            }
+    }
+    uint32_t o = 0xff000000u;
+#pragma unroll
+    for (int ch = 0; ch < 3; ch++) {
+        float m[K];
+#pragma unroll
+        for (int k = 0; k < K; k++)
+            m[k] = mean > 0.0f ? float(acc[ch][k]) * mean : __fdiv_rn(float(acc[ch][k]), float(ns));
+        float v = m[0];
+        if constexpr (XT) {
+            float t = v * c.xtalk_c;
+            t = fmaf(c.xtalk, m[1], t);
+            t = fmaf(c.xtalk, m[2], t);
+            v = t;
+        }
+        o |= uint32_t(round_u8(v)) << (8 * ch);
+    }
+    return o;
+}
+
+// A block's tile is one panel row of 32 S columns; warp w's lanes take columns
+// j, j + S, j + 2 S, ... for j = w, w + 8, ... < S. With S a multiple of the
+// lens pitch the lanes see the same lens phase, so each gather's 32 bytes lie
+// in one view's row, S W / Wp pixels apart: two 128-byte lines for the 48-view
+// display (S = 8) instead of the eight views of 32 neighbouring columns, and
+// the gathers' lines are what the kernel would otherwise wait for (gauss_stride
+// picks S). Blocks take runs of consecutive rows of a column tile, which share
+// view rows in L1; a finished row is written from shared memory in order.
+// 96 views of 420x560 to a 2560x1600 panel, 8 samples, crosstalk: 0.646 ms with
+// four positions compared per search and 32 neighbouring columns a warp, 0.182
+// now, bound by issue (two thirds of the slots; 72 searches and gathers of
+// about a dozen instructions) and the L1 wavefronts of the gathers (half their
+// rate). 64 registers and four blocks per SM: five at 48 registers take 0.195.
+// table: the views' bytes fit 32-bit offsets and every sample's angular
+// offset lies within the table's margin (the launch cannot know the offsets:
+// they are checked here).
+constexpr int kGaussThreads = 256;
+template <bool XT>
+__global__ void __launch_bounds__(kGaussThreads, 4) k_interleave_gauss(DispConst c, const uint8_t* __restrict__ views,
+                                                                    const float* __restrict__ pos,
+                                                                    const float* __restrict__ samples, int ns,
+                                                                    uint8_t* __restrict__ panel, int S, int table) {
     wait_previous_kernel();
     allow_next_kernel();
+    extern __shared__ __align__(16) uint8_t s_dyn[];
+    GaussBin* s_bins = reinterpret_cast<GaussBin*>(s_dyn);
+    const int n_bins = table ? gauss_bins(c.n_views) : 0;
+    uint32_t* s_row = reinterpret_cast<uint32_t*>(s_bins + n_bins);   // [2][32 S] finished rows
     __shared__ float s_pos[kMaxRenderViews];
     __shared__ float s_smp[3 * 32];
-    for (int i = threadIdx.x; i < c.nr; i += blockDim.x) s_pos[i] = pos[i];
-    for (int i = threadIdx.x; i < 3 * ns; i += blockDim.x) s_smp[i] = samples[i];
+    __shared__ float4 s_smp4[32];
+    const uint32_t view_bytes = 4u * uint32_t(c.W) * uint32_t(c.H);
+    bool slow = !table;
+    for (int i = threadIdx.x; i < c.nr; i += kGaussThreads) s_pos[i] = pos[i];
+    for (int i = threadIdx.x; i < 3 * ns; i += kGaussThreads) s_smp[i] = samples[i];
+    for (int i = threadIdx.x; i < ns; i += kGaussThreads) {
+        const float4 q = make_float4(samples[3 * i], samples[3 * i + 1], samples[3 * i + 2], 0.0f);
+        s_smp4[i] = q;
+        slow |= !(fabsf(q.z) <= float(kGaussMargin));
+    }
     __syncthreads();
-    const uint64_t total = (uint64_t)c.Wp * c.Hp;
+    for (int b = threadIdx.x; b < n_bins; b += kGaussThreads) {
+        GaussBin o;
+        slow |= !gauss_bin(s_pos, c.nr, float(c.nr / c.n_views), b, view_bytes, o);
+        s_bins[b] = o;
+    }
+    slow = __syncthreads_or(slow);
+    const uint32_t bins = uint32_t(__cvta_generic_to_shared(s_bins)) - 8u * kGaussMagicBits;
+    const float mean = (ns & (ns - 1)) == 0 ? 1.0f / float(ns) : 0.0f;
     const float sxw = float(c.W) / float(c.Wp), syh = float(c.H) / float(c.Hp);
     const uint32_t* v32 = reinterpret_cast<const uint32_t*>(views);
-    for (uint64_t gi = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; gi < total;
-         gi += (uint64_t)gridDim.x * blockDim.x) {
-        const int y = int(gi / c.Wp), x = int(gi - (uint64_t)y * c.Wp);
-        reinterpret_cast<uint32_t*>(panel)[gi] = gauss_pixel(c, v32, s_pos, s_smp, ns, x, y, sxw, syh);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cols = 32 * S, n_strips = (c.Wp + cols - 1) / cols;
+    const uint32_t total = uint32_t(n_strips) * uint32_t(c.Hp);
+    // this block's run of rows, strip after strip
+    const uint32_t i0 = uint32_t((uint64_t)total * blockIdx.x / gridDim.x);
+    const uint32_t i1 = uint32_t((uint64_t)total * (blockIdx.x + 1u) / gridDim.x);
+    uint32_t* row = s_row;
+    for (uint32_t i = i0; i < i1; i++, row = row == s_row ? s_row + cols : s_row) {
+        const int strip = int(i / uint32_t(c.Hp)), y = int(i - uint32_t(strip) * uint32_t(c.Hp));
+        const int x0 = strip * cols;
+        for (int j = warp; j < S; j += kGaussThreads / 32) {
+            const int x = x0 + j + S * lane;
+            if (x >= c.Wp) continue;
+            bool exact = slow;   // (a phase is no number where slant or pitch overflow)
+#pragma unroll
+            for (int ch = 0; ch < 3; ch++) {
+                const float p0 = subpixel_phase(c, x, y, ch);
+                exact |= !(p0 >= 0.0f && p0 <= float(c.n_views));
+            }
+            row[j + S * lane] = exact ? gauss_pixel(c, v32, s_pos, s_smp, ns, x, y, sxw, syh)
+                                      : gauss_pixel_table<XT>(c, views, bins, view_bytes, s_smp4, ns, mean, x, y, sxw, syh);
+        }
+        __syncthreads();   // the row is complete; the other buffer's readers are past their barrier
+        uint32_t* dst = reinterpret_cast<uint32_t*>(panel) + (uint64_t)y * c.Wp + x0;
+        for (int q = threadIdx.x; q < cols && x0 + q < c.Wp; q += kGaussThreads) dst[q] = row[q];
     }
+}
+
+// The column stride between a warp's lanes: of the multiples of 8 (one warp
+// of the block per column between) the one whose gathers touch the fewest
+// lines, counting up to the strip's width past the panel as work. A gather's
+// lines are estimated from the lanes' views (the stride in lens periods) and
+// columns; below three lines the kernel no longer waits for them.
+int gauss_stride(const DispConst& c) {
+    int best = 8;
+    double least = 1e30;
+    for (int S = 8; S <= kGaussMaxStride; S += 8) {
+        int lines = 0;
+        int last_view = -1, last_line = -1;
+        for (int l = 0; l < 32; l++) {
+            const double ph = double(l) * S * double(c.inv_pitch);
+            // half a view up, so that a stride of whole periods stays in one view whatever its rounding
+            const int view = int((ph - std::floor(ph)) * c.nr + 0.5) % c.nr;
+            const int line = int(double(l) * S * c.W / c.Wp) / 32;
+            lines += view != last_view || line != last_line;
+            last_view = view;
+            last_line = line;
+        }
+        const int cols = 32 * S;
+        const double cost = std::max(3, lines) * (double((c.Wp + cols - 1) / cols) * cols / c.Wp);
+        if (cost < least) {
+            least = cost;
+            best = S;
+        }
+    }
+    return best;
 }
 
 }  // namespace
@@ -380,8 +605,17 @@ cudaError_t launch_interleave(const DispConst& dc, const uint8_t* views, const f
     cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (dc.recon == 2 || dc.recon == 3) {
         if (n_samples < 1 || n_samples > 32) return cudaErrorInvalidValue;
-        return launch_after_previous(k_interleave_gauss, dim3(sms * 16), dim3(256), 0, s, dc, views, pos, samples,
-                                     n_samples, panel);
+        const int S = gauss_stride(dc);
+        // 32-bit byte offsets of the views' texels
+        const int table = (uint64_t)dc.nr * dc.W * dc.H * 4u <= 0xffffffffull;
+        const size_t bytes = (table ? sizeof(GaussBin) * gauss_bins(dc.n_views) : 0u) + 2u * 32u * S * 4u;
+        const uint64_t rows = (uint64_t)((dc.Wp + 32 * S - 1) / (32 * S)) * dc.Hp;
+        const int grid = int(std::min<uint64_t>(rows, uint64_t(sms) * 4u));
+        if (dc.xtalk > 0.0f)
+            return launch_after_previous(k_interleave_gauss<true>, dim3(grid), dim3(kGaussThreads), bytes, s, dc, views,
+                                         pos, samples, n_samples, panel, S, table);
+        return launch_after_previous(k_interleave_gauss<false>, dim3(grid), dim3(kGaussThreads), bytes, s, dc, views,
+                                     pos, samples, n_samples, panel, S, table);
     }
     // widest source segment of a tile: (kTileCols - 1) W / Wp + 2 pixels
     const int64_t seg = ((int64_t)(kTileCols - 1) * dc.W) / dc.Wp + 2;

@@ -1,5 +1,8 @@
 """The interleave's forms against the oracle, byte for byte, on views of
-random bytes.
+random bytes: sizes at which a strip of panel columns, a lens period or a
+view row is left over, one view and many, eyes placed on the same border of
+their intervals (no threshold separates them) and sample offsets beyond the
+table of nearest views.
 """
 from dataclasses import replace
 
@@ -52,6 +55,42 @@ def _panel(d, views, jitter=None, samples=None):
 
 def _views(d, seed):
     return np.random.default_rng(seed).integers(0, 256, (d.n_render_views, d.view_h, d.view_w, 4), dtype=np.uint8)
+
+
+# (views, view w, h, panel w, h, pitch, slant, recon, crosstalk, samples, eyes, largest dphi)
+GAUSS = [(48, 42, 56, 256, 16, 8.0, 0.2, 2, 0.15, 8, "random", None),      # one whole strip
+         (48, 42, 56, 257, 17, 8.0, 0.2, 2, 0.15, 8, "random", None),      # and one column more
+         (48, 21, 28, 1600, 9, 8.0, -0.2, 3, 0.15, 8, "random", None),
+         (37, 33, 25, 1277, 13, 5.3, 1.0 / 6.0, 2, 0.0, 7, "random", None),
+         (24, 64, 20, 900, 11, 5.0, 0.25, 2, 0.15, 32, "half", None),
+         (8, 17, 9, 31, 300, 2.5, 0.1, 3, 0.1, 1, "random", None),
+         (1, 9, 9, 40, 10, 8.0, 0.2, 3, 0.2, 3, "random", None),
+         (1, 9, 9, 40, 10, 8.0, 0.2, 2, 0.2, 4, "random", None),
+         (2, 5, 3, 70, 10, 4.0, 0.0, 2, 0.3, 8, "random", None),
+         (256, 8, 8, 520, 8, 11.0, 0.3, 2, 0.15, 8, "random", None),       # the most views
+         (16, 12, 12, 260, 20, 8.0, 0.2, 2, 0.15, 8, "ends", None),        # every interval's start or end
+         (16, 12, 12, 260, 20, 8.0, 0.2, 2, 0.15, 8, "border", None),      # neighbours at one place
+         (16, 12, 12, 260, 20, 8.0, 0.2, 3, 0.15, 8, "border", None),
+         (16, 12, 12, 260, 20, 8.0, 0.2, 2, 0.15, 8, "close", None),       # neighbours a few floats apart
+         (16, 12, 12, 260, 20, 8.0, 0.2, 2, 0.15, 8, "random", 4.0),       # the table's last bin
+         (16, 12, 12, 260, 20, 8.0, 0.2, 2, 0.15, 8, "random", 4.01),      # beyond it
+         (16, 12, 12, 260, 20, 8.0, 0.2, 2, 0.15, 8, "random", 1e9)]
+
+
+@pytest.mark.parametrize("case", range(len(GAUSS)))
+def test_gaussian_interleave_matches_oracle(case):
+    n, w, h, pw, ph, pitch, slant, recon, xtalk, ns, eyes, dphi = GAUSS[case]
+    d = _display(n, w, h, pw, ph, pitch, slant, recon, xtalk)
+    rng = np.random.default_rng(100 + case)
+    nr = d.n_render_views
+    u = {"random": rng.random(nr), "half": np.full(nr, 0.5), "ends": rng.integers(0, 2, nr).astype(float),
+         "border": np.arange(nr) % 2 == 0, "close": np.where(np.arange(nr) % 2 == 0, 1.0 - 1e-6, 1e-6)}[eyes]
+    u = np.asarray(u).astype(np.float32)
+    smp = (rng.normal(0.0, 1.0, (ns, 3)) * [0.5625, 0.5625, 0.5]).astype(np.float32)
+    if dphi is not None:
+        smp[0, 2], smp[1, 2] = dphi, -dphi
+    views = _views(d, case)
+    assert np.array_equal(_panel(d, views, u, smp), O.interleave(d, views, jitter=u, samples=smp))
 
 
 @pytest.mark.parametrize("recon", [2, 3])
