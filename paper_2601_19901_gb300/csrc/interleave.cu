@@ -10,6 +10,7 @@
 // segment of that row for every rendered view in shared memory with
 // coalesced loads, then forms every panel row that samples that view row,
 // one thread per 4 adjacent panel pixels and one 16-byte store per row.
+// k_interleave_tent stages the tent's display views instead.
 // k_interleave (the direct gather) serves displays whose tile would not fit.
 // k_interleave_gauss is the Gaussian reconstruction of Sec. 4 (recon 2, 3):
 // per subpixel the mean of the caller's samples, each the nearest rendered
@@ -73,10 +74,13 @@ __device__ __forceinline__ float subpixel_phase(const DispConst& c, int x, int y
     return fr * float(c.n_views);
 }
 
+// floor of the phase, below N (one addition rounded down onto 2^23: the
+// conversion instruction runs at a quarter of the rate); 0 where the phase is
+// no number (slant or pitch overflow).
 __device__ __forceinline__ int view_of_subpixel(const DispConst& c, int x, int y, int ch) {
-    int k = int(subpixel_phase(c, x, y, ch));
-    k = k >= c.n_views ? c.n_views - 1 : (k < 0 ? 0 : k);
-    return k;
+    const uint32_t N = uint32_t(c.n_views);
+    const uint32_t k = __float_as_uint(__fadd_rd(subpixel_phase(c, x, y, ch), 8388608.0f)) - 0x4b000000u;
+    return int(k > N ? 0u : min(k, N - 1u));
 }
 
 // Panel pixel (x, y) as RGBA8 (alpha 255) from its view pixel's texels.
@@ -129,33 +133,45 @@ __device__ __forceinline__ void store4(const DispConst& c, uint8_t* __restrict__
     }
 }
 
-constexpr int kTileThreads = 256;
+constexpr int kTileThreads = 256, kTentThreads = 128;
 constexpr int kTileCols = 4 * kTileThreads;   // panel columns per tile
+constexpr int kTentCols = 4 * kTentThreads;
+constexpr int kStageCols = 4;                 // 32-column runs of a row segment loaded together
+
+// The first panel row sampling view row sy; false if none does.
+__device__ __forceinline__ bool first_row_of(const DispConst& c, int sy, int& y) {
+    y = max(0, int(uint32_t(sy) * uint32_t(c.Hp) / uint32_t(c.H)) - 1);
+    while (y < c.Hp && source_y(c, y) < sy) y++;
+    return y < c.Hp && source_y(c, y) == sy;
+}
 
 // Block (strip bx, view row sy): view pixels sx_lo..sx_lo + n - 1 of row sy
 // for every rendered view, then the panel rows whose source row is sy.
 __global__ void __launch_bounds__(kTileThreads) k_interleave_tile(DispConst c, const uint8_t* __restrict__ views,
-                                                                  uint8_t* __restrict__ panel, int stride) {
+                                                                  uint8_t* __restrict__ panel, int cols, int stride) {
     wait_previous_kernel();
     allow_next_kernel();
     extern __shared__ uint32_t s_row[];
     const int sy = blockIdx.y;
-    const int x0 = blockIdx.x * kTileCols;
-    const int x1 = min(x0 + kTileCols, c.Wp);   // exclusive
-    // panel rows sampling view row sy: y_first.. while source_y(y) == sy
-    int y = max(0, int(uint32_t(sy) * uint32_t(c.Hp) / uint32_t(c.H)) - 1);
-    while (y < c.Hp && source_y(c, y) < sy) y++;
-    if (y >= c.Hp || source_y(c, y) != sy) return;
+    const int x0 = blockIdx.x * cols;
+    const int x1 = min(x0 + cols, c.Wp);   // exclusive
+    int y;
+    if (!first_row_of(c, sy, y)) return;
     const int sx_lo = source_x(c, x0), n = source_x(c, x1 - 1) - sx_lo + 1;
     const uint64_t npix = (uint64_t)c.W * c.H;
     const uint32_t* v32 = reinterpret_cast<const uint32_t*>(views);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int m = warp; m < c.nr; m += kTileThreads / 32) {
-        const uint32_t* src = v32 + (uint64_t)m * npix + (uint64_t)sy * c.W + sx_lo;
-        for (int i = lane; i < n; i += 32)
-            if (LFDPR_IN_BOUNDS(uint32_t(sx_lo + i), uint32_t(c.W), 20) && LFDPR_IN_BOUNDS(i, stride, 20))
-                s_row[m * stride + i] = __ldg(src + i);
-    }
+    for (int i0 = lane; i0 < n; i0 += 32 * kStageCols)
+#pragma unroll 2
+        for (int m = warp; m < c.nr; m += kTileThreads / 32) {
+            const uint32_t* src = v32 + (uint64_t)m * npix + (uint64_t)sy * c.W + sx_lo;
+#pragma unroll
+            for (int q = 0; q < kStageCols; q++) {
+                const int i = i0 + 32 * q;
+                if (i < n && LFDPR_IN_BOUNDS(uint32_t(sx_lo + i), uint32_t(c.W), 20) && LFDPR_IN_BOUNDS(i, stride, 20))
+                    s_row[m * stride + i] = __ldg(src + i);
+            }
+        }
     __syncthreads();
     const int xg = x0 + 4 * threadIdx.x;
     if (xg >= x1) return;
@@ -166,6 +182,127 @@ __global__ void __launch_bounds__(kTileThreads) k_interleave_tile(DispConst c, c
         uint32_t px[4];
 #pragma unroll
         for (int e = 0; e < 4; e++) px[e] = panel_pixel(c, SharedTexels{s_row, stride, sxi[e]}, xg + e, y);
+        store4(c, panel, xg, y, px);
+    }
+}
+
+// The same for tent reconstruction (recon 1). The block stages the display
+// views instead of the rendered ones: four times display view k is
+// r[2k-1] + 2 r[2k] + r[2k+1], a 10-bit sum per channel, so a pixel's three
+// channels fit one word and a subpixel reads one word per display view (three
+// with crosstalk) where it read three times as many rendered views and divided
+// each sum by its weight. The values are the specified ones exactly: the
+// weights 1/4 and 1/2 times bytes add without rounding, a sum of weights of 1
+// divides to the sum itself, and the factor 4 is taken back from the crosstalk
+// weights (a power of two). Display view 0 has no view before it, so its
+// weights sum to 3/4: its quotients are staged as binary32 (4 times each).
+// 96 views of 420x560 to a 2560x1600 panel with crosstalk: 0.222 ms reading the
+// rendered views' bytes and dividing, 0.049 now (90 MB of views read: 0.014 at
+// the copy rate); bound by issue, some 45 instructions a subpixel, and by the
+// staging's loads. Blocks of 128 threads: 256 leave fewer blocks to cover each
+// other's staging (0.057). Six registers spill to keep ten blocks per SM
+// (0.055 without).
+__device__ __forceinline__ uint32_t tent_word(uint32_t a, uint32_t b, uint32_t d) {
+    const uint32_t m = 0x00ff00ffu;
+    const uint32_t e = (a & m) + 2u * (b & m) + (d & m);                                        // channels 0 and 2
+    const uint32_t o = ((a >> 8) & 255u) + 2u * ((b >> 8) & 255u) + ((d >> 8) & 255u);   // channel 1
+    return (e & 0x3ffu) | (o << 10) | ((e >> 16) << 20);
+}
+template <bool XT>
+__global__ void __launch_bounds__(kTentThreads, 10) k_interleave_tent(DispConst c, const uint8_t* __restrict__ views,
+                                                                  uint8_t* __restrict__ panel, int cols, int stride) {
+    wait_previous_kernel();
+    allow_next_kernel();
+    // [1 + n_views + 1][stride] words (view N - 1 again before view 0, and view
+    // 0 after view N - 1, as crosstalk wraps), then [3][stride] view 0
+    extern __shared__ uint32_t s_tent[];
+    const int N = c.n_views;
+    float* s_view0 = reinterpret_cast<float*>(s_tent + (N + 2) * stride);
+    const int sy = blockIdx.y;
+    const int x0 = blockIdx.x * cols;
+    const int x1 = min(x0 + cols, c.Wp);   // exclusive
+    int y;
+    if (!first_row_of(c, sy, y)) return;
+    const int sx_lo = source_x(c, x0), n = source_x(c, x1 - 1) - sx_lo + 1;
+    const uint64_t npix = (uint64_t)c.W * c.H;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(views) + (uint64_t)sy * c.W + sx_lo;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // a warp takes a run of display views, so that view 2k + 1 serves k + 1 too
+    const int k0 = N * warp / (kTentThreads / 32), k1 = N * (warp + 1) / (kTentThreads / 32);
+    for (int i0 = lane; i0 < n && k0 < k1; i0 += 32 * kStageCols) {
+        const uint32_t* p = src + i0 + (uint64_t)(2 * k0) * npix;
+        uint32_t a[kStageCols];
+        bool on[kStageCols];
+#pragma unroll
+        for (int q = 0; q < kStageCols; q++) {
+            const int i = i0 + 32 * q;
+            on[q] = i < n && LFDPR_IN_BOUNDS(uint32_t(sx_lo + i), uint32_t(c.W), 20) && LFDPR_IN_BOUNDS(i, stride, 20);
+            a[q] = on[q] && k0 > 0 ? __ldg(p + 32 * q - npix) : 0u;
+        }
+#pragma unroll 2
+        for (int k = k0; k < k1; k++, p += 2 * npix) {
+            uint32_t b[kStageCols], d[kStageCols];
+#pragma unroll
+            for (int q = 0; q < kStageCols; q++) {
+                b[q] = on[q] ? __ldg(p + 32 * q) : 0u;
+                d[q] = on[q] ? __ldg(p + 32 * q + npix) : 0u;
+            }
+#pragma unroll
+            for (int q = 0; q < kStageCols; q++) {
+                const int i = i0 + 32 * q;
+                const uint32_t w = tent_word(a[q], b[q], d[q]);
+                if (on[q]) s_tent[(k + 1) * stride + i] = w;
+                if (XT && k == N - 1 && on[q]) s_tent[i] = w;
+                if (XT && k == 0 && on[q]) s_tent[(N + 1) * stride + i] = w;
+                if (k == 0 && on[q])
+#pragma unroll
+                    for (int ch = 0; ch < 3; ch++)
+                        s_view0[ch * stride + i] = 4.0f * __fdiv_rn(0.25f * float((w >> (10 * ch)) & 0x3ffu), 0.75f);
+                a[q] = d[q];
+            }
+        }
+    }
+    __syncthreads();
+    const int xg = x0 + 4 * threadIdx.x;
+    if (xg >= x1) return;
+    const float xc4 = 0.25f * c.xtalk_c, x4 = 0.25f * c.xtalk;
+    const uint32_t pitch = 4u * uint32_t(stride), s0 = uint32_t(__cvta_generic_to_shared(s_tent));
+    const uint32_t view0 = s0 + uint32_t(N + 2) * pitch;
+    // four times the display view in row `at` of the words (column and channel
+    // as given); view 0's are the binary32 ones
+    auto value4 = [&](uint32_t at, uint32_t col, int ch, bool first) -> float {
+        const uint32_t addr = first ? view0 + uint32_t(ch) * pitch + col : at;
+        uint32_t w;
+        asm("ld.shared.u32 %0, [%1];" : "=r"(w) : "r"(addr));
+        // 2^23 + the sum, by its bits
+        const float t = __uint_as_float(((w >> (10 * ch)) & 0x3ffu) | 0x4b000000u) - 8388608.0f;
+        return first ? __uint_as_float(w) : t;
+    };
+    uint32_t col[4];
+#pragma unroll
+    for (int e = 0; e < 4; e++) col[e] = 4u * uint32_t(min(source_x(c, min(xg + e, x1 - 1)) - sx_lo, n - 1));
+    for (; y < c.Hp && source_y(c, y) == sy; y++) {
+        uint32_t px[4];
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            uint32_t o = 0xff000000u;
+#pragma unroll
+            for (int ch = 0; ch < 3; ch++) {
+                const int k = view_of_subpixel(c, xg + e, y, ch);
+                const uint32_t at = s0 + col[e] + uint32_t(k) * pitch;   // view k - 1's row
+                float val;
+                if constexpr (XT) {
+                    val = value4(at + pitch, col[e], ch, k == 0) * xc4;
+                    val = fmaf(x4, value4(at, col[e], ch, k == (N > 1 ? 1 : 0)), val);
+                    val = fmaf(x4, value4(at + 2u * pitch, col[e], ch, k == N - 1), val);
+                } else {
+                    val = 0.25f * value4(at + pitch, col[e], ch, k == 0);
+                }
+                // round half to even (0 <= val < 255.5): the low byte of 1.5 2^23 + val
+                o |= (__float_as_uint(val + 12582912.0f) & 255u) << (8 * ch);
+            }
+            px[e] = o;
+        }
         store4(c, panel, xg, y, px);
     }
 }
@@ -617,16 +754,19 @@ cudaError_t launch_interleave(const DispConst& dc, const uint8_t* views, const f
         return launch_after_previous(k_interleave_gauss<false>, dim3(grid), dim3(kGaussThreads), bytes, s, dc, views,
                                      pos, samples, n_samples, panel, S, table);
     }
-    // widest source segment of a tile: (kTileCols - 1) W / Wp + 2 pixels
-    const int64_t seg = ((int64_t)(kTileCols - 1) * dc.W) / dc.Wp + 2;
-    const int64_t bytes = (int64_t)dc.nr * seg * 4;
+    // the widest source segment of a strip: (cols - 1) W / Wp + 2 pixels
+    const bool tent = dc.recon == 1;
+    const int cols = tent ? kTentCols : kTileCols;
+    const int64_t seg = ((int64_t)(cols - 1) * dc.W) / dc.Wp + 2;
+    const int64_t words = tent ? dc.n_views + 5 : dc.nr, bytes = words * seg * 4;
     if (bytes <= smem_max / 2) {
-        cudaError_t e = cudaFuncSetAttribute(k_interleave_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             int(bytes));
+        const auto kernel = !tent ? k_interleave_tile
+                            : dc.xtalk > 0.0f ? k_interleave_tent<true> : k_interleave_tent<false>;
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
         if (e != cudaSuccess) return e;
-        const dim3 grid((dc.Wp + kTileCols - 1) / kTileCols, dc.H);
-        return launch_after_previous(k_interleave_tile, grid, dim3(kTileThreads), size_t(bytes), s, dc, views, panel,
-                                     int(seg));
+        return launch_after_previous(kernel, dim3((dc.Wp + cols - 1) / cols, dc.H), dim3(tent ? kTentThreads : kTileThreads),
+                                     size_t(bytes), s,
+                                     dc, views, panel, cols, int(seg));
     }
     return launch_after_previous(k_interleave, dim3(sms * 8), dim3(256), 0, s, dc, views, panel);
 }

@@ -105,3 +105,26 @@ def test_sample_offsets_of_any_size(recon):
     far = smp.copy()
     far[:, 2] = [0.0, 0.25, 1e9, -1e9]
     assert np.array_equal(_panel(d, views, u, smp), O.interleave(d, views, jitter=u, samples=far))
+
+
+# (views, view w, h, panel w, h, pitch, slant, recon, crosstalk)
+TILED = [(48, 42, 56, 512, 33, 8.0, 0.2, 1, 0.15),        # one whole strip of panel columns
+         (48, 42, 56, 513, 33, 8.0, 0.2, 1, 0.15),        # two, uneven
+         (48, 42, 56, 2560, 12, 8.0, 0.2, 1, 0.0),
+         (37, 33, 25, 1277, 13, 5.3, 1.0 / 6.0, 1, 0.2),
+         (37, 33, 25, 1277, 13, 5.3, 1.0 / 6.0, 0, 0.2),
+         (37, 33, 25, 1278, 130, 5.3, -0.3, 0, 0.0),
+         (3, 40, 30, 77, 20, 2.5, 0.1, 1, 0.4),
+         (2, 40, 30, 77, 20, 2.5, 0.1, 1, 0.4),
+         (1, 40, 30, 77, 20, 2.5, 0.1, 1, 0.4),
+         (1, 1, 1, 1, 1, 1.0, 0.0, 1, 0.1),
+         (5, 300, 200, 30, 20, 6.0, 0.1, 1, 0.1),         # more view pixels than panel pixels
+         (40, 2000, 4, 100, 40, 8.0, 0.2, 1, 0.15),       # no tile fits: the direct gather
+         (256, 12, 9, 260, 20, 9.0, 0.2, 1, 0.15)]
+
+
+@pytest.mark.parametrize("case", range(len(TILED)))
+def test_tiled_interleave_matches_oracle(case):
+    d = _display(*TILED[case])
+    views = _views(d, 50 + case)
+    assert np.array_equal(_panel(d, views), O.interleave(d, views))
