@@ -206,6 +206,7 @@ struct TcGeom {
     int rows, span;           // TMA box rows of 32 positions per chunk; span = 32 rows positions in shared memory
     int Qp;                   // positions per chunk in memory (Q rounded up to 32)
     int stages;               // pipeline depth
+    int beside;               // whether the stages leave the reserved shared memory of each SM free
     uint32_t a_bytes, b_bytes, stage_bytes;
     uint32_t tmem_cols;       // power of two >= 2 R NT (two accumulator buffers)
     int m_tiles, n_tiles;     // tiles: ceil(Q / 128 R) position tiles x output-channel tiles
@@ -601,6 +602,8 @@ __global__ void k_from_chunked(const __nv_bfloat16* __restrict__ in, int H, int 
 // ---------------------------------------------------------------------------
 
 constexpr uint32_t kTcSmemMax = 227 * 1024;
+constexpr int kWarpsBeside = 2; // blocks of the warp an SM holds beside a layer's block
+constexpr int kMinStages = 2;   // below this a layer does not make room for another kernel's blocks
 
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -641,7 +644,8 @@ uint32_t pow2_cols(int n) {
 // Geometry of a layer over the bordered level image Hl x Wl: cin = cin_a +
 // cin_b input channels (map a, then map b), NT output channels per block, R
 // row groups of 128 positions per block.
-TcGeom tc_geom(int Hl, int Wl, int cin_a, int cin_b, int taps, int NT, int R, int n_tiles, int cout) {
+TcGeom tc_geom(int Hl, int Wl, int cin_a, int cin_b, int taps, int NT, int R, int n_tiles, int cout,
+               uint32_t reserve) {
     TcGeom g{};
     g.Hb = Hl + 2;
     g.Wb = Wl + 2;
@@ -659,8 +663,11 @@ TcGeom tc_geom(int Hl, int Wl, int cin_a, int cin_b, int taps, int NT, int R, in
     g.a_bytes = uint32_t(2 * g.span * 16);
     g.b_bytes = uint32_t(taps * 2 * NT * 16);
     g.stage_bytes = (g.a_bytes + g.b_bytes + 1023u) & ~1023u;
-    // one block per SM, as many stages as fit
-    g.stages = int(std::min<uint32_t>(uint32_t(kMaxStages), (kTcSmemMax - 3072u) / g.stage_bytes));
+    // one block per SM, as many stages as fit beside `reserve` bytes; wide
+    // views whose stages leave no room for them take the whole SM
+    const uint32_t room = kTcSmemMax - 3072u;
+    g.beside = room >= reserve && (room - reserve) / g.stage_bytes >= uint32_t(kMinStages);
+    g.stages = int(std::min<uint32_t>(uint32_t(kMaxStages), (g.beside ? room - reserve : room) / g.stage_bytes));
     g.tmem_cols = pow2_cols(2 * R * NT);
     g.m_tiles = (g.Q + 128 * R - 1) / (128 * R);
     g.n_tiles = n_tiles;
@@ -792,6 +799,7 @@ struct lfdpr_recon {
     int64_t w_off[14] = {}, b_off[14] = {};
     TcGeom geom[14] = {}, geom_out = {};
     CUtensorMap in_map[14], in_map_b[14], out_d0;
+    int warp_grid = 1;                // blocks of the warp
     uint8_t* warp = nullptr;          // [nout][H][W][4] the input views warped to the output eyes (RGBA8)
     cudaStream_t side = nullptr;      // the warp runs here, beside the network's layers
     cudaEvent_t fork = nullptr, join = nullptr;
@@ -914,7 +922,10 @@ lfdpr_status lfdpr_create_recon(int32_t view_w, int32_t view_h, int32_t in_views
         for (int k = 0; k < 32; k++) wout[size_t(o) * ko + k] = weights_bf16[nw3 + int64_t(o) * 32 + k];
     std::vector<float> bout(ntout, 0.0f);
     for (int o = 0; o < no3; o++) bout[o] = biases[nb3 + o];
-    // layer geometry and packed weights
+    // layer geometry and packed weights; the layers leave each SM the shared
+    // memory of two blocks of the warp (and 1 KB of the system's for each),
+    // which runs beside them
+    const uint32_t reserve = kWarpsBeside * (uint32_t(warp_smem(r->nin, r->nout, r->W)) + 1024u);
     for (int l = 0; l < 14; l++) {
         const ConvSpec& L = kLayers[l];
         const int Hl = r->Hp >> L.level, Wl = r->Wp >> L.level;
@@ -922,14 +933,19 @@ lfdpr_status lfdpr_create_recon(int32_t view_w, int32_t view_h, int32_t in_views
         pick_tile(Hl, Wl, L.cout, r->sm_count, NT, R);
         // layers 8, 10, 12 read [upsampled (map a) | skip (map b)]
         const int cin_b = (l == 8 || l == 10 || l == 12) ? L.cin / 3 : 0;
-        r->geom[l] = tc_geom(Hl, Wl, L.cin - cin_b, cin_b, 9, NT, R, L.cout / NT, L.cout);
+        r->geom[l] = tc_geom(Hl, Wl, L.cin - cin_b, cin_b, 9, NT, R, L.cout / NT, L.cout, reserve);
         if (l == 7 || l == 9 || l == 11) {   // write 2x upsampled into the next level's tensor
             r->geom[l].up = 1;
             r->geom[l].Wbo = 2 * Wl + 2;
             r->geom[l].Qpo = int(qpad(2 * Hl, 2 * Wl));
         }
     }
-    r->geom_out = tc_geom(r->Hp, r->Wp, 32, 0, 1, ntout, 1, 1, 0);
+    // as many blocks of the warp as the layers leave room for; where one does
+    // not, a block per row and interval
+    r->warp_grid = kWarpsBeside * r->sm_count;
+    for (const TcGeom& g : r->geom)
+        if (!g.beside) r->warp_grid = r->H * (r->nin - 1);
+    r->geom_out = tc_geom(r->Hp, r->Wp, 32, 0, 1, ntout, 1, 1, 0, 0);
     r->geom_out.base = reinterpret_cast<const uint32_t*>(r->warp);
     r->geom_out.nout = r->nout;
     r->geom_out.H = r->H;
@@ -1016,15 +1032,15 @@ lfdpr_status lfdpr_recon_forward(lfdpr_recon* r, const uint8_t* in_views, const 
     k_recon_in<<<sm * 8, 256, 0, s>>>(in_views, r->nin, r->H, r->W, H0, W0, r->x0);
     CKR(cudaGetLastError(), "launch k_recon_in");
     // the residual's base: the input views warped to the output eyes, on the
-    // side stream while the layers run (SMs the layers leave idle take it)
+    // side stream beside the layers. The first layer is launched before it, so
+    // that its blocks have their SMs when the warp's take what is left of them.
     CKR(cudaEventRecord(r->fork, s), "recon_forward: fork");
+    CKR(conv(0), "conv 0");
     CKR(cudaStreamWaitEvent(r->side, r->fork, 0), "recon_forward: fork");
     CKR(launch_warp_views(in_views, in_keys, in_eyes, r->nin, out_eyes, r->nout, r->W, r->H, pixels_per_unit,
-                          r->warp, r->side),
+                          r->warp, r->warp_grid, r->side),
         "launch k_warp_views");
     CKR(cudaEventRecord(r->join, r->side), "recon_forward: join");
-
-    CKR(conv(0), "conv 0");
     CKR(conv(1), "conv 1");
     CKR(pool(r->e0, H0, W0, 32, r->p1), "pool 1");
     CKR(conv(2), "conv 2");
@@ -1084,7 +1100,7 @@ lfdpr_status lfdpr_conv3x3_bf16(const void* in, int32_t H, int32_t W, int32_t ci
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int NT, R;
     pick_tile(H, W, cout, sms, NT, R);
-    const TcGeom g = tc_geom(H, W, cin, 0, 9, NT, R, cout / NT, cout);
+    const TcGeom g = tc_geom(H, W, cin, 0, 9, NT, R, cout / NT, cout, 0);
     if (!tc_valid(g)) return fail(LFDPR_EINVAL, "conv3x3: no tensor-core layout for a %d-wide image", W);
     // chunked bordered copies of the input and output, and the packed weights
     const size_t qp = qpad(H, W);
