@@ -14,7 +14,7 @@
 // core-matrix layout (8 positions x 8 channels = 128 contiguous bytes) the
 // MMAs read, copied by TMA as one box of 512-byte rows (32 positions each).
 //
-//   k_conv_tc<0>  3x3 convolution + bias + ReLU as an implicit GEMM
+//   k_conv_tc     3x3 convolution + bias + ReLU as an implicit GEMM
 //                 (M = positions, N = output channels, K = 9 x input
 //                 channels). A block takes R x 128 positions and NT output
 //                 channels. Per K step of 16 input channels one thread issues
@@ -24,10 +24,10 @@
 //                 issues tcgen05.mma (M 128, N NT, K 16) for the nine taps x R
 //                 row groups with shared-memory descriptors offset by the tap's
 //                 shift; tcgen05.commit frees the stage when its MMAs are
-//                 done. The four warps then read the accumulators back
+//                 done. The epilogue warps then read the accumulators back
 //                 (tcgen05.ld), add the bias, apply ReLU and store bf16, with
 //                 zeros on the border ring, one 16-byte store per chunk.
-//   k_conv_tc<1>  the output layer: the 1x1 convolution of d0 (32
+//   k_out_tc      the output layer: the 1x1 convolution of d0 (32
 //                 channels), plus the base (the input views warped to the
 //                 output eyes by warp.cu's k_warp_views, RGB / 255)
 //                 and the bias, clamped, scaled to 255, rounded half to even,
@@ -53,7 +53,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
+#include <set>
 #include <utility>
 #include <vector>
 
@@ -196,10 +198,9 @@ __device__ __forceinline__ void ld48(uint32_t taddr, float* v) {
 constexpr int kTcThreads = 320;
 constexpr int kEpiWarps = 8;
 
-// Geometry of one tensor-core layer launch (host-computed).
+// Geometry of one 3x3 layer launch (host-computed).
 struct TcGeom {
     int Hb, Wb, Q;            // bordered rows, columns, positions Hb Wb
-    int taps;                 // 9 (3x3) or 1 (1x1)
     int NT, R;                // output channels per tile; 128-position row groups per tile
     int ksteps;               // K steps of 16 input channels
     int split;                // 8-channel chunks read through map a (the rest through map b)
@@ -210,12 +211,10 @@ struct TcGeom {
     uint32_t a_bytes, b_bytes, stage_bytes;
     uint32_t tmem_cols;       // power of two >= 2 R NT (two accumulator buffers)
     int m_tiles, n_tiles;     // tiles: ceil(Q / 128 R) position tiles x output-channel tiles
-    int cout;                 // channels of the bf16 output tensor (3x3 layers)
-    int up;                   // 3x3 layers: write the output 2x upsampled (nearest) into a tensor of twice the size
+    int cout;                 // channels of the bf16 output tensor
+    int up;                   // write the output 2x upsampled (nearest) into a tensor of twice the size
     int Wbo, Qpo;             // that tensor's bordered width and positions per chunk
-    int nout, H, W;           // output layer: views written, view size
     int bias_n;               // biases staged in shared memory (<= 256)
-    const uint32_t* base;     // output layer: the residual's base, RGBA8 views laid out as the output
 };
 
 // A wait that also gives up as soon as another role of the block has given
@@ -248,7 +247,7 @@ constexpr int kMaxStages = 8;
 // Tile t (t = blockIdx.x, + gridDim.x, ...) covers positions (t % m_tiles) 128 R
 // .. + 128 R - 1 and output channels (t / m_tiles) NT .. + NT - 1; its
 // accumulators live in tensor-memory buffer (local tile index) % 2.
-template <int EPI, int TAPS, int R>
+template <int R>
 __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant__ CUtensorMap ma,
                                                            const __grid_constant__ CUtensorMap mb,
                                                            const uint8_t* __restrict__ wpk,
@@ -299,7 +298,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
             bool ok = true;
             for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
                 const int q0 = (t % g.m_tiles) * 128 * R, nt = t / g.m_tiles;
-                const int qs = q0 - (TAPS == 9 ? g.Wb + 1 : 0);
+                const int qs = q0 - (g.Wb + 1);
                 const int y0 = (qs >= 0 ? qs : qs - 31) / 32;   // the 32-position row holding the span's start
                 const uint8_t* wsrc = wpk + size_t(nt) * g.ksteps * g.b_bytes;
                 for (int ks = 0; ks < g.ksteps; ks++, kc++) {
@@ -328,9 +327,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
             // the 14-bit address field (shared addresses stay below 256 KB, so the
             // field never carries).
             const uint32_t idesc = tc::idesc_bf16(128, g.NT);
-            uint32_t toff[TAPS];
+            uint32_t toff[9];
 #pragma unroll
-            for (int tp = 0; tp < TAPS; tp++) toff[tp] = TAPS == 9 ? uint32_t((tp / 3) * g.Wb + (tp % 3)) : 0u;
+            for (int tp = 0; tp < 9; tp++) toff[tp] = uint32_t((tp / 3) * g.Wb + (tp % 3));
             const uint64_t a_desc0 = tc::sdesc(s0, uint32_t(g.span * 16), 128);
             const uint64_t b_desc0 = tc::sdesc(s0 + g.a_bytes, uint32_t(g.NT * 16), 128);
             const uint32_t b_tap = uint32_t(2 * g.NT);   // 16-byte units between taps' weights
@@ -338,7 +337,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
             bool ok = true;
             for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, it++) {
                 const int q0 = (t % g.m_tiles) * 128 * R;
-                const int qs = q0 - (TAPS == 9 ? g.Wb + 1 : 0);
+                const int qs = q0 - (g.Wb + 1);
                 const uint32_t delta = uint32_t(qs - 32 * ((qs >= 0 ? qs : qs - 31) / 32));   // span start in its first row
                 const int buf = it & 1;
                 // the epilogue has drained this buffer (its use two tiles ago)
@@ -358,7 +357,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
                     const uint32_t st16 = (uint32_t(s) * g.stage_bytes) >> 4;
                     const uint64_t ad = a_desc0 + st16 + delta, bd = b_desc0 + st16;
 #pragma unroll
-                    for (int tp = 0; tp < TAPS; tp++)
+                    for (int tp = 0; tp < 9; tp++)
 #pragma unroll
                         for (int r = 0; r < R; r++)
                             tc::mma(dacc + uint32_t(r * g.NT), ad + toff[tp] + uint32_t(r * 128), bd + tp * b_tap, idesc,
@@ -391,79 +390,40 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
             for (int r = 0; r < R; r++) {
                 const int q = q0 + r * 128 + lq * 32 + lane;
                 const int y = q / g.Wb, x = q - y * g.Wb;
-                if (EPI == 0) {
-                    const bool border = y == 0 || y >= g.Hb - 1 || x == 0 || x == g.Wb - 1;
-                    const int half = g.NT >> 1;
-                    for (int j = cg * half; j < (cg + 1) * half; j += 16) {
-                        float v[16], bv[16];
-                        tc::ld16(trow + uint32_t(r * g.NT + j), v);
+                const bool border = y == 0 || y >= g.Hb - 1 || x == 0 || x == g.Wb - 1;
+                const int half = g.NT >> 1;
+                for (int j = cg * half; j < (cg + 1) * half; j += 16) {
+                    float v[16], bv[16];
+                    tc::ld16(trow + uint32_t(r * g.NT + j), v);
 #pragma unroll
-                        for (int i = 0; i < 4; i++)
-                            *reinterpret_cast<float4*>(bv + 4 * i) = reinterpret_cast<const float4*>(s_bias + n0 + j)[i];
-                        uint4 pk[2];
-                        __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(pk);
+                    for (int i = 0; i < 4; i++)
+                        *reinterpret_cast<float4*>(bv + 4 * i) = reinterpret_cast<const float4*>(s_bias + n0 + j)[i];
+                    uint4 pk[2];
+                    __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(pk);
 #pragma unroll
-                        for (int i = 0; i < 8; i++) {
-                            const float a0 = border ? 0.0f : fmaxf(v[2 * i] + bv[2 * i], 0.0f);
-                            const float a1 = border ? 0.0f : fmaxf(v[2 * i + 1] + bv[2 * i + 1], 0.0f);
-                            h[i] = __floats2bfloat162_rn(a0, a1);
-                        }
-                        const int c8 = (n0 + j) / 8;
-                        if (!g.up) {
-                            if (q < g.Q) {
-                                __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out) + (size_t(c8) * g.Qp + q) * 8;
-                                *reinterpret_cast<uint4*>(o) = pk[0];
-                                *reinterpret_cast<uint4*>(o + size_t(g.Qp) * 8) = pk[1];
-                            }
-                        } else if (q < g.Q && !border) {
-                            // nearest 2x: pixel (y - 1, x - 1) -> the 2x2 block at (2 y - 2, 2 x - 2) of the larger image
-                            const size_t qh = size_t(2 * y - 1) * g.Wbo + size_t(2 * x - 1);
-                            __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out) + (size_t(c8) * g.Qpo + qh) * 8;
-#pragma unroll
-                            for (int k = 0; k < 2; k++) {
-                                __nv_bfloat16* ok_ = o + size_t(k) * g.Qpo * 8;
-                                *reinterpret_cast<uint4*>(ok_) = pk[k];
-                                *reinterpret_cast<uint4*>(ok_ + 8) = pk[k];
-                                *reinterpret_cast<uint4*>(ok_ + size_t(g.Wbo) * 8) = pk[k];
-                                *reinterpret_cast<uint4*>(ok_ + size_t(g.Wbo) * 8 + 8) = pk[k];
-                            }
-                        }
+                    for (int i = 0; i < 8; i++) {
+                        const float a0 = border ? 0.0f : fmaxf(v[2 * i] + bv[2 * i], 0.0f);
+                        const float a1 = border ? 0.0f : fmaxf(v[2 * i + 1] + bv[2 * i + 1], 0.0f);
+                        h[i] = __floats2bfloat162_rn(a0, a1);
                     }
-                } else {
-                    // output views: column o = 3 view + channel; 48-column steps alternate between the groups
-                    const int vy = y - 1, vx = x - 1;
-                    const bool inside = q < g.Q && vy >= 0 && vy < g.H && vx >= 0 && vx < g.W;
-                    uint32_t* views = static_cast<uint32_t*>(out);
-                    const size_t npix = size_t(g.H) * g.W, pix = size_t(vy) * g.W + vx;
-                    for (int j = cg * 48; j < g.NT; j += 96) {
-                        float v[48], bv[48];
-                        tc::ld48(trow + uint32_t(r * g.NT + j), v);
-#pragma unroll
-                        for (int i = 0; i < 12; i++)
-                            *reinterpret_cast<float4*>(bv + 4 * i) = reinterpret_cast<const float4*>(s_bias + j)[i];
-                        // the base's 16 views at this position, all loads in flight first
-                        uint32_t bws[16];
-#pragma unroll
-                        for (int k = 0; k < 16; k++) {
-                            const int view = j / 3 + k;
-                            bws[k] = inside && view < g.nout ? __ldg(g.base + size_t(view) * npix + pix) : 0u;
+                    const int c8 = (n0 + j) / 8;
+                    if (!g.up) {
+                        if (q < g.Q) {
+                            __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out) + (size_t(c8) * g.Qp + q) * 8;
+                            *reinterpret_cast<uint4*>(o) = pk[0];
+                            *reinterpret_cast<uint4*>(o + size_t(g.Qp) * 8) = pk[1];
                         }
+                    } else if (q < g.Q && !border) {
+                        // nearest 2x: pixel (y - 1, x - 1) -> the 2x2 block at (2 y - 2, 2 x - 2) of the larger image
+                        const size_t qh = size_t(2 * y - 1) * g.Wbo + size_t(2 * x - 1);
+                        __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out) + (size_t(c8) * g.Qpo + qh) * 8;
 #pragma unroll
-                        for (int k = 0; k < 16; k++) {
-                            const int view = j / 3 + k;
-                            if (!(inside && view < g.nout)) continue;
-                            // the base's RGB / 255, added to the product
-                            const uint32_t bw = bws[k];
-                            float base[3];
-#pragma unroll
-                            for (int c = 0; c < 3; c++) base[c] = float((bw >> (8 * c)) & 255u) * (1.0f / 255.0f);
-                            // round(clamp(x + base + b, 0, 1) 255), half to even: saturating add, scale, convert
-                            const uint32_t r0 = __float2uint_rn(__saturatef((v[3 * k] + base[0]) + bv[3 * k]) * 255.0f);
-                            const uint32_t g0 =
-                                __float2uint_rn(__saturatef((v[3 * k + 1] + base[1]) + bv[3 * k + 1]) * 255.0f);
-                            const uint32_t b0 =
-                                __float2uint_rn(__saturatef((v[3 * k + 2] + base[2]) + bv[3 * k + 2]) * 255.0f);
-                            views[size_t(view) * npix + pix] = 0xff000000u | r0 | (g0 << 8) | (b0 << 16);
+                        for (int k = 0; k < 2; k++) {
+                            __nv_bfloat16* ok_ = o + size_t(k) * g.Qpo * 8;
+                            *reinterpret_cast<uint4*>(ok_) = pk[k];
+                            *reinterpret_cast<uint4*>(ok_ + 8) = pk[k];
+                            *reinterpret_cast<uint4*>(ok_ + size_t(g.Wbo) * 8) = pk[k];
+                            *reinterpret_cast<uint4*>(ok_ + size_t(g.Wbo) * 8 + 8) = pk[k];
                         }
                     }
                 }
@@ -480,6 +440,195 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.tmem_cols));
+}
+
+// ---------------------------------------------------------------------------
+// The output layer
+// ---------------------------------------------------------------------------
+
+struct OutGeom {
+    int Wb, tiles;            // bordered columns of d0; tiles of 128 positions
+    int NT;                   // 3 nout padded to a multiple of 48
+    int nout, H, W;           // views written, view size
+};
+
+// The 1x1 convolution of d0 (32 channels) to 3 nout colours per position, plus
+// the base's RGB / 255 and the bias, clamped, times 255, rounded half to even.
+//
+// Bound by memory: d0, the base and the views are 105 MB at 48 views of
+// 420x560 (0.016 ms at the copy rate). The product is two MMAs per tile of 128
+// positions, so what counts is that enough warps keep base reads and view
+// writes in flight: a group of four epilogue warps for every 16 views (a group
+// covers a tile's 128 rows, 32 per warp), each warp reading its next tile's
+// base words before it works on this tile's. The weights stay in shared memory; bytes become binary32 and colours become bytes by their bits, not by
+// conversions (a quarter of the rate). 0.065 ms with eight epilogue warps on three
+// uneven column steps and the base read after the product, 0.035 now.
+//
+// Shared memory: [kOutStages x d0 tile (4 chunks x 128 positions x 16 B)], the
+// weights, the barriers: full[4] +0, empty[4] +32, acc_full[2] +64, acc_empty[2]
+// +80, weights +96, drain +104, tensor-memory address +112, abort word +116; the biases at
+// +128. Every wait is bounded as the 3x3 layers' are.
+constexpr int kOutStages = 4;
+__host__ __device__ constexpr int out_threads(int groups) { return 64 + 128 * groups; }
+constexpr uint32_t kOutTile = 4 * 128 * 16;
+template <int GROUPS>
+__global__ void __launch_bounds__(out_threads(GROUPS), 1) k_out_tc(const __grid_constant__ CUtensorMap m,
+                                                           const uint8_t* __restrict__ wpk,
+                                                           const float* __restrict__ bias,
+                                                           const uint32_t* __restrict__ base, uint32_t* __restrict__ out,
+                                                           const OutGeom g, int* __restrict__ status) {
+    constexpr int NT = 48 * GROUPS;
+    constexpr uint32_t b_bytes = 2u * 2u * NT * 16u;   // two K steps of 16 channels
+    constexpr uint32_t cols = 2 * NT <= 128 ? 128 : 2 * NT <= 256 ? 256 : 512;   // two accumulators
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t s0 = (tc::smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t wts = s0 + kOutStages * kOutTile, bars = wts + b_bytes;
+    const uint32_t empty = bars + 32, acc_full = bars + 64, acc_empty = bars + 80, wfull = bars + 96, drain = bars + 104,
+                   slot = bars + 112, abort_w = bars + 116;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        for (int s = 0; s < kOutStages; s++) {
+            tc::init(bars + 8 * s, 1);
+            tc::init(empty + 8 * s, 1);
+        }
+        for (int b = 0; b < 2; b++) {
+            tc::init(acc_full + 8 * b, 1);
+            tc::init(acc_empty + 8 * b, 4 * GROUPS);   // one arrival per epilogue warp
+        }
+        tc::init(wfull, 1);
+        tc::init(drain, 1);
+        asm volatile("st.shared.u32 [%0], %1;" ::"r"(abort_w), "r"(0u));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    float* s_bias = reinterpret_cast<float*>(smem_raw + (bars + 128 - tc::smem_u32(smem_raw)));
+    for (int i = tid; i < NT; i += out_threads(GROUPS)) s_bias[i] = bias[i];
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(cols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    uint32_t tmem;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem) : "r"(slot));
+    wait_previous_kernel();
+    allow_next_kernel();
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // producer: the weights once, then a tile's four 8-channel chunks per stage
+            tc::expect_tx(wfull, b_bytes);
+            tc::load_bulk(wts, wpk, b_bytes, wfull);
+            int k = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; t < g.tiles; t += gridDim.x, k++) {
+                const int s = k % kOutStages;
+                if (k >= kOutStages && !wait_or_abort(empty + 8 * s, uint32_t((k / kOutStages - 1) & 1), abort_w)) {
+                    ok = false;
+                    break;
+                }
+                tc::expect_tx(bars + 8 * s, kOutTile);
+                tc::load_box(s0 + s * kOutTile, &m, 0, 4 * t, 0, bars + 8 * s);
+                tc::load_box(s0 + s * kOutTile + kOutTile / 2, &m, 0, 4 * t, 2, bars + 8 * s);
+            }
+            // the copies issued last on each stage have landed before the block moves on
+            for (int q = max(0, k - kOutStages); q < k; q++)
+                tc::wait(bars + 8 * (q % kOutStages), uint32_t((q / kOutStages) & 1));
+            tc::wait(wfull, 0);
+            if (!ok) atomicOr(status, 1);
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t idesc = tc::idesc_bf16(128, NT);
+            bool ok = wait_or_abort(wfull, 0, abort_w);
+            int it = 0;
+            for (int t = blockIdx.x; t < g.tiles && ok; t += gridDim.x, it++) {
+                const int buf = it & 1, s = it % kOutStages;
+                // the epilogue has drained this buffer (its use two tiles ago)
+                if (it >= 2 && !wait_or_abort(acc_empty + 8 * buf, uint32_t((it / 2 - 1) & 1), abort_w)) {
+                    ok = false;
+                    break;
+                }
+                if (!wait_or_abort(bars + 8 * s, uint32_t((it / kOutStages) & 1), abort_w)) {
+                    ok = false;
+                    break;
+                }
+                tc::fence_after();
+#pragma unroll
+                for (int ks = 0; ks < 2; ks++)
+                    tc::mma(tmem + uint32_t(buf * NT), tc::sdesc(s0 + s * kOutTile + ks * (kOutTile / 2), 128 * 16, 128),
+                            tc::sdesc(wts + ks * (b_bytes / 2), NT * 16, 128), idesc, uint32_t(ks));
+                tc::commit(empty + 8 * s);
+                tc::commit(acc_full + 8 * buf);
+            }
+            // every MMA issued has completed before the block moves on
+            tc::commit(drain);
+            tc::wait(drain, 0);
+            if (!ok) atomicOr(status, 2);
+        }
+    } else {
+        const int lq = warp & 3, cg = (warp - 2) >> 2;   // lane quarter, group
+        const size_t npix = size_t(g.H) * g.W;
+        // this lane's position of tile t as a view pixel (false: border, padding or past the end)
+        auto pixel = [&](int t, size_t& pix) -> bool {
+            const int q = t * 128 + lq * 32 + lane, y = q / g.Wb, vy = y - 1, vx = q - y * g.Wb - 1;
+            pix = size_t(vy) * g.W + vx;
+            return t < g.tiles && vy >= 0 && vy < g.H && vx >= 0 && vx < g.W;
+        };
+        uint32_t next[16];   // the base's 16 views of this group at the next tile's position
+        size_t npx;
+        bool nin = pixel(blockIdx.x, npx);
+        auto fetch = [&]() {
+#pragma unroll
+            for (int k = 0; k < 16; k++)
+                next[k] = nin && 16 * cg + k < g.nout ? __ldg(base + size_t(16 * cg + k) * npix + npx) : 0u;
+        };
+        fetch();
+        int it = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < g.tiles; t += gridDim.x, it++) {
+            const int buf = it & 1;
+            const bool inside = nin;
+            uint32_t* dst = out + npx;
+            uint32_t bw[16];
+#pragma unroll
+            for (int k = 0; k < 16; k++) bw[k] = next[k];
+            nin = pixel(t + gridDim.x, npx);
+            fetch();
+            // one lane per warp polls (with backoff); the others wait at the shuffle
+            int got = 0;
+            if (lane == 0) got = wait_or_abort(acc_full + 8 * buf, uint32_t((it / 2) & 1), abort_w, 64) ? 1 : 0;
+            ok = __shfl_sync(0xffffffffu, got, 0) != 0;
+            if (!ok) break;
+            tc::fence_after();
+            float v[48];
+            tc::ld48(tmem + (uint32_t(lq * 32) << 16) + uint32_t(buf * NT + 48 * cg), v);
+#pragma unroll
+            for (int k = 0; k < 16; k++) {
+                const int view = 16 * cg + k;
+                if (!(inside && view < g.nout)) continue;
+                uint32_t o = 0xff000000u;
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    // the base's colour / 255, added to the product: round(clamp(x + base + b, 0, 1) 255)
+                    const float byte = __uint_as_float(0x4b000000u | ((bw[k] >> (8 * c)) & 255u)) - 8388608.0f;
+                    const float x = __saturatef((v[3 * k + c] + byte * (1.0f / 255.0f)) + s_bias[3 * view + c]) * 255.0f;
+                    o |= (__float_as_uint(x + 12582912.0f) & 255u) << (8 * c);
+                }
+                dst[size_t(view) * npix] = o;
+            }
+            // this warp's reads of the buffer are done
+            tc::fence_before();
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty + 8 * buf) : "memory");
+        }
+        if (!ok && lane == 0) atomicOr(status, 4);
+    }
+    __syncwarp();
+    tc::fence_before();
+    __syncthreads();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols));
 }
 
 // dst [n_tiles][ksteps][taps][2][NT][8] from src [cout][taps][cin]; rows co >=
@@ -644,24 +793,23 @@ uint32_t pow2_cols(int n) {
 // Geometry of a layer over the bordered level image Hl x Wl: cin = cin_a +
 // cin_b input channels (map a, then map b), NT output channels per block, R
 // row groups of 128 positions per block.
-TcGeom tc_geom(int Hl, int Wl, int cin_a, int cin_b, int taps, int NT, int R, int n_tiles, int cout,
+TcGeom tc_geom(int Hl, int Wl, int cin_a, int cin_b, int NT, int R, int n_tiles, int cout,
                uint32_t reserve) {
     TcGeom g{};
     g.Hb = Hl + 2;
     g.Wb = Wl + 2;
     g.Q = g.Hb * g.Wb;
-    g.taps = taps;
     g.NT = NT;
     g.R = R;
     g.ksteps = (cin_a + cin_b) / 16;
     g.split = cin_a / 8;
     g.Qp = (g.Q + 31) / 32 * 32;
     // the span plus up to 31 positions before it in its first 32-position row
-    const int L = 128 * R + (taps == 9 ? 2 * g.Wb + 2 : 0);
+    const int L = 128 * R + 2 * g.Wb + 2;
     g.rows = (L + 31 + 31) / 32;
     g.span = 32 * g.rows;
     g.a_bytes = uint32_t(2 * g.span * 16);
-    g.b_bytes = uint32_t(taps * 2 * NT * 16);
+    g.b_bytes = uint32_t(9 * 2 * NT * 16);
     g.stage_bytes = (g.a_bytes + g.b_bytes + 1023u) & ~1023u;
     // one block per SM, as many stages as fit beside `reserve` bytes; wide
     // views whose stages leave no room for them take the whole SM
@@ -673,6 +821,17 @@ TcGeom tc_geom(int Hl, int Wl, int cin_a, int cin_b, int taps, int NT, int R, in
     g.n_tiles = n_tiles;
     g.cout = cout;
     g.bias_n = n_tiles * NT;
+    return g;
+}
+
+OutGeom out_geom(int Hl, int Wl, int H, int W, int nout, int NT) {
+    OutGeom g{};
+    g.Wb = Wl + 2;
+    g.tiles = ((Hl + 2) * (Wl + 2) + 127) / 128;
+    g.NT = NT;
+    g.nout = nout;
+    g.H = H;
+    g.W = W;
     return g;
 }
 
@@ -707,41 +866,52 @@ int sm_count_cached() {
 
 bool tc_valid(const TcGeom& g) {
     return g.stages >= 2 && g.ksteps >= 1 && g.NT % 16 == 0 && g.NT >= 16 && g.NT <= 256 && g.tmem_cols <= 512 &&
-           (g.taps == 9 || g.taps == 1) && g.split % 2 == 0 && g.rows <= 256 && g.m_tiles >= 1 && g.n_tiles >= 1 &&
-           g.bias_n >= 1 && g.bias_n <= 256 && (g.taps == 1 || (g.NT / 2) % 16 == 0) && tc_smem(g) <= kTcSmemMax;
+           g.split % 2 == 0 && g.rows <= 256 && g.m_tiles >= 1 && g.n_tiles >= 1 && g.bias_n >= 1 && g.bias_n <= 256 &&
+           (g.NT / 2) % 16 == 0 && tc_smem(g) <= kTcSmemMax;
+}
+
+// The largest dynamic shared memory for a kernel of this file, asked for once
+// per kernel and device.
+cudaError_t allow_smem(const void* kernel) {
+    static std::mutex mu;
+    static std::set<std::pair<const void*, int>> done;
+    int dev = 0;
+    const cudaError_t d = cudaGetDevice(&dev);
+    if (d != cudaSuccess) return d;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done.count({kernel, dev})) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTcSmemMax));
+    if (e == cudaSuccess) done.insert({kernel, dev});
+    return e;
 }
 
 // Each layer is launched as a programmatic dependent of the kernel before it
 // (launch_after_previous): its blocks set up their barriers, tensor memory
 // and biases, then wait for that kernel in wait_previous_kernel().
-cudaError_t launch_tc(int epi, const TcGeom& g, const CUtensorMap& ma, const CUtensorMap& mb, const void* wpk,
-                      const float* bias, void* out, int* status, cudaStream_t s) {
+cudaError_t launch_tc(const TcGeom& g, const CUtensorMap& ma, const CUtensorMap& mb, const void* wpk, const float* bias,
+                      void* out, int* status, cudaStream_t s) {
     if (!tc_valid(g)) return cudaErrorInvalidValue;
-    static bool attrs[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!attrs[dev]) {
-        const void* fns[4] = {reinterpret_cast<const void*>(k_conv_tc<1, 1, 1>), reinterpret_cast<const void*>(k_conv_tc<0, 9, 1>),
-                              reinterpret_cast<const void*>(k_conv_tc<0, 9, 2>), reinterpret_cast<const void*>(k_conv_tc<0, 9, 4>)};
-        for (const void* f : fns) {
-            const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTcSmemMax));
-            if (e != cudaSuccess) return e;
-        }
-        attrs[dev] = true;
-    }
+    const auto kernel = g.R == 1 ? k_conv_tc<1> : g.R == 2 ? k_conv_tc<2> : g.R == 4 ? k_conv_tc<4> : nullptr;
+    if (!kernel) return cudaErrorInvalidValue;
+    const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kernel));
+    if (e != cudaSuccess) return e;
     const int grid = std::min(g.m_tiles * g.n_tiles, sm_count_cached());
-    const size_t smem = tc_smem(g);
-    const uint8_t* w = static_cast<const uint8_t*>(wpk);
-    if (epi == 1 && g.taps == 1 && g.R == 1)
-        return launch_after_previous(k_conv_tc<1, 1, 1>, grid, kTcThreads, smem, s, ma, mb, w, bias, out, g, status);
-    if (epi == 0 && g.taps == 9 && g.R == 1)
-        return launch_after_previous(k_conv_tc<0, 9, 1>, grid, kTcThreads, smem, s, ma, mb, w, bias, out, g, status);
-    if (epi == 0 && g.taps == 9 && g.R == 2)
-        return launch_after_previous(k_conv_tc<0, 9, 2>, grid, kTcThreads, smem, s, ma, mb, w, bias, out, g, status);
-    if (epi == 0 && g.taps == 9 && g.R == 4)
-        return launch_after_previous(k_conv_tc<0, 9, 4>, grid, kTcThreads, smem, s, ma, mb, w, bias, out, g, status);
-    return cudaErrorInvalidValue;
+    return launch_after_previous(kernel, grid, kTcThreads, tc_smem(g), s, ma, mb, static_cast<const uint8_t*>(wpk), bias, out,
+                                 g, status);
+}
+
+// The output layer, launched as the others.
+cudaError_t launch_out(const OutGeom& g, const CUtensorMap& m, const void* wpk, const float* bias, const uint32_t* base,
+                       uint32_t* out, int* status, cudaStream_t s) {
+    const int groups = g.NT / 48;
+    const auto kernel = groups == 1 ? k_out_tc<1> : groups == 2 ? k_out_tc<2> : groups == 3 ? k_out_tc<3>
+                        : groups == 4 ? k_out_tc<4> : nullptr;
+    if (!kernel || g.NT % 48) return cudaErrorInvalidValue;
+    const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kernel));
+    if (e != cudaSuccess) return e;
+    // more than half of the SM's shared memory: one block holds an SM and its tensor memory
+    return launch_after_previous(kernel, std::min(g.tiles, sm_count_cached()), out_threads(groups), smem_per_sm() / 2 + 1024, s, m,
+                                 static_cast<const uint8_t*>(wpk), bias, base, out, g, status);
 }
 
 cudaError_t launch_pack(const __nv_bfloat16* src, int cout, int taps, int cin, int NT, int n_tiles, __nv_bfloat16* dst,
@@ -797,7 +967,8 @@ struct lfdpr_recon {
     float* b_out = nullptr;           // [NT_out] (zero past 3 nout)
     int* status = nullptr;            // device: failed waits (bit 0 copies, 1 MMA, 2 epilogue)
     int64_t w_off[14] = {}, b_off[14] = {};
-    TcGeom geom[14] = {}, geom_out = {};
+    TcGeom geom[14] = {};
+    OutGeom geom_out = {};
     CUtensorMap in_map[14], in_map_b[14], out_d0;
     int warp_grid = 1;                // blocks of the warp
     uint8_t* warp = nullptr;          // [nout][H][W][4] the input views warped to the output eyes (RGBA8)
@@ -933,7 +1104,7 @@ lfdpr_status lfdpr_create_recon(int32_t view_w, int32_t view_h, int32_t in_views
         pick_tile(Hl, Wl, L.cout, r->sm_count, NT, R);
         // layers 8, 10, 12 read [upsampled (map a) | skip (map b)]
         const int cin_b = (l == 8 || l == 10 || l == 12) ? L.cin / 3 : 0;
-        r->geom[l] = tc_geom(Hl, Wl, L.cin - cin_b, cin_b, 9, NT, R, L.cout / NT, L.cout, reserve);
+        r->geom[l] = tc_geom(Hl, Wl, L.cin - cin_b, cin_b, NT, R, L.cout / NT, L.cout, reserve);
         if (l == 7 || l == 9 || l == 11) {   // write 2x upsampled into the next level's tensor
             r->geom[l].up = 1;
             r->geom[l].Wbo = 2 * Wl + 2;
@@ -945,11 +1116,7 @@ lfdpr_status lfdpr_create_recon(int32_t view_w, int32_t view_h, int32_t in_views
     r->warp_grid = kWarpsBeside * r->sm_count;
     for (const TcGeom& g : r->geom)
         if (!g.beside) r->warp_grid = r->H * (r->nin - 1);
-    r->geom_out = tc_geom(r->Hp, r->Wp, 32, 0, 1, ntout, 1, 1, 0, 0);
-    r->geom_out.base = reinterpret_cast<const uint32_t*>(r->warp);
-    r->geom_out.nout = r->nout;
-    r->geom_out.H = r->H;
-    r->geom_out.W = r->W;
+    r->geom_out = out_geom(r->Hp, r->Wp, r->H, r->W, r->nout, ntout);
     const __nv_bfloat16* conv_in[14] = {r->x0, r->e0a, r->p1, r->e1a, r->p2, r->e2a, r->p3,
                                         r->ba, r->U2,  r->d2a, r->U1, r->d1a, r->U0, r->d0a};
     const __nv_bfloat16* conv_skip[14] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
@@ -964,8 +1131,7 @@ lfdpr_status lfdpr_create_recon(int32_t view_w, int32_t view_h, int32_t in_views
         else
             r->in_map_b[l] = r->in_map[l];
     }
-    maps_ok = maps_ok && tc_valid(r->geom_out) &&
-              make_map(&r->out_d0, r->d0, 32, r->geom_out.Qp, r->geom_out.rows) == cudaSuccess;
+    maps_ok = maps_ok && make_map(&r->out_d0, r->d0, 32, qpad(r->Hp, r->Wp), 4) == cudaSuccess;
     if (!maps_ok) {
         dev_free(w_raw);
         dev_free(wout_raw);
@@ -1018,7 +1184,7 @@ lfdpr_status lfdpr_recon_forward(lfdpr_recon* r, const uint8_t* in_views, const 
     __nv_bfloat16* conv_out[14] = {r->e0a, r->e0, r->e1a, r->e1, r->e2a, r->e2, r->ba,
                                    r->U2,  r->d2a, r->U1, r->d1a, r->U0, r->d0a, r->d0};
     auto conv = [&](int l) {
-        return launch_tc(0, r->geom[l], r->in_map[l], r->in_map_b[l], r->w + r->w_off[l], r->b + r->b_off[l],
+        return launch_tc(r->geom[l], r->in_map[l], r->in_map_b[l], r->w + r->w_off[l], r->b + r->b_off[l],
                          conv_out[l], r->status, s);
     };
     auto pool = [&](const __nv_bfloat16* in, int H, int W, int C, __nv_bfloat16* o) {
@@ -1058,7 +1224,8 @@ lfdpr_status lfdpr_recon_forward(lfdpr_recon* r, const uint8_t* in_views, const 
     CKR(conv(12), "conv 12");
     CKR(conv(13), "conv 13");
     CKR(cudaStreamWaitEvent(s, r->join, 0), "recon_forward: join");
-    CKR(launch_tc(1, r->geom_out, r->out_d0, r->out_d0, r->w_out, r->b_out, out_views, r->status, s),
+    CKR(launch_out(r->geom_out, r->out_d0, r->w_out, r->b_out, reinterpret_cast<const uint32_t*>(r->warp),
+                   reinterpret_cast<uint32_t*>(out_views), r->status, s),
         "output layer");
 #undef CKR
     return LFDPR_OK;
@@ -1100,7 +1267,7 @@ lfdpr_status lfdpr_conv3x3_bf16(const void* in, int32_t H, int32_t W, int32_t ci
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int NT, R;
     pick_tile(H, W, cout, sms, NT, R);
-    const TcGeom g = tc_geom(H, W, cin, 0, 9, NT, R, cout / NT, cout, 0);
+    const TcGeom g = tc_geom(H, W, cin, 0, NT, R, cout / NT, cout, 0);
     if (!tc_valid(g)) return fail(LFDPR_EINVAL, "conv3x3: no tensor-core layout for a %d-wide image", W);
     // chunked bordered copies of the input and output, and the packed weights
     const size_t qp = qpad(H, W);
@@ -1116,7 +1283,7 @@ lfdpr_status lfdpr_conv3x3_bf16(const void* in, int32_t H, int32_t W, int32_t ci
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = launch_pack(static_cast<const __nv_bfloat16*>(wgt), cout, 9, cin, NT, cout / NT, wpk, s);
-    if (e == cudaSuccess) e = launch_tc(0, g, m, m, wpk, bias, co, reinterpret_cast<int*>(status), s);
+    if (e == cudaSuccess) e = launch_tc(g, m, m, wpk, bias, co, reinterpret_cast<int*>(status), s);
     if (e == cudaSuccess) {
         k_from_chunked<<<sms * 8, 256, 0, s>>>(co, H, W, cout, static_cast<__nv_bfloat16*>(out));
         e = cudaGetLastError();
