@@ -16,7 +16,7 @@
 //
 //   k_conv_tc     3x3 convolution + bias + ReLU as an implicit GEMM
 //                 (M = positions, N = output channels, K = 9 x input
-//                 channels). A block takes R x 128 positions and NT output
+//                 channels). A tile is R x 128 positions and NT output
 //                 channels. Per K step of 16 input channels one thread issues
 //                 TMA copies of the input span (one box per 8-channel chunk,
 //                 starting at the 32-position row at or before the span) and
@@ -122,28 +122,37 @@ __device__ __forceinline__ void load_bulk(uint32_t dst, const void* src, uint32_
 // Shared-memory matrix descriptor, no swizzle, K-major: core matrices of 8
 // rows x 16 bytes (128 contiguous bytes); `lbo` = byte distance between core
 // matrices adjacent in K, `sbo` = between core matrices adjacent in M (N).
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    return uint64_t((addr >> 4) & 0x3FFFu) | (uint64_t((lbo >> 4) & 0x3FFFu) << 16) |
-           (uint64_t((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
+// Its low word, and its high word.
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t addr, uint32_t lbo) {
+    return ((addr >> 4) & 0x3FFFu) | (((lbo >> 4) & 0x3FFFu) << 16);
 }
+__device__ __forceinline__ uint32_t sdesc_hi(uint32_t sbo) { return ((sbo >> 4) & 0x3FFFu) | (1u << 14); }
 
 // Instruction descriptor of kind::f16: BF16 A and B (K-major), FP32 D, M x N.
 __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(n >> 3) << 17) | (uint32_t(m >> 4) << 24);
 }
 
-// D[tmem] (+)= A[a] B[b]^T; accumulate into D when acc != 0.
-__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+// D[tmem] (+)= A[a] B[b]^T; accumulate into D when acc != 0. The descriptors
+// are their low words (address and `lbo`) and a common high word. Executed by
+// a whole converged warp, of which one elected lane issues the MMA: its
+// operands live in uniform registers, and only where the compiler sees the
+// warp compute them together does it compute them there, instead of moving
+// each one over from a vector register for every MMA.
+__device__ __forceinline__ void mma(uint32_t d, uint32_t a, uint32_t b, uint32_t hi, uint32_t idesc, uint32_t acc) {
     asm volatile(
-        "{ .reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc));
+        "{ .reg .pred p, e; .reg .b64 da, db; elect.sync _|e, 0xffffffff; setp.ne.b32 p, %5, 0; mov.b64 da, {%1, %3}; "
+        "mov.b64 db, {%2, %3}; @e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p; }" ::"r"(d),
+        "r"(a), "r"(b), "r"(hi), "r"(idesc), "r"(acc));
 }
 
-// The mbarrier at `bar` receives one arrival when every MMA this thread has
-// issued so far is complete.
+// The mbarrier at `bar` receives one arrival when every MMA this warp's
+// elected lane has issued so far is complete (a whole converged warp, as mma).
 __device__ __forceinline__ void commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
+    asm volatile(
+        "{ .reg .pred e; elect.sync _|e, 0xffffffff; @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 "
+        "[%0]; }" ::"r"(bar)
+        : "memory");
 }
 
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -201,16 +210,19 @@ constexpr int kEpiWarps = 8;
 // Geometry of one 3x3 layer launch (host-computed).
 struct TcGeom {
     int Hb, Wb, Q;            // bordered rows, columns, positions Hb Wb
-    int NT, R;                // output channels per tile; 128-position row groups per tile
+    int NT;                   // output channels per tile
+    int R, full, R_tail;      // 128-position row groups of a tile: R of the first `full` ones, R_tail (at most R) after
+    int groups;               // row groups in all: ceil(Q / 128)
     int ksteps;               // K steps of 16 input channels
     int split;                // 8-channel chunks read through map a (the rest through map b)
     int rows, span;           // TMA box rows of 32 positions per chunk; span = 32 rows positions in shared memory
     int Qp;                   // positions per chunk in memory (Q rounded up to 32)
     int stages;               // pipeline depth
+    int early;                // the weights were there before the kernel before this one
     int beside;               // whether the stages leave the reserved shared memory of each SM free
     uint32_t a_bytes, b_bytes, stage_bytes;
     uint32_t tmem_cols;       // power of two >= 2 R NT (two accumulator buffers)
-    int m_tiles, n_tiles;     // tiles: ceil(Q / 128 R) position tiles x output-channel tiles
+    int m_tiles, n_tiles;     // tiles: position tiles x output-channel tiles
     int cout;                 // channels of the bf16 output tensor
     int up;                   // write the output 2x upsampled (nearest) into a tensor of twice the size
     int Wbo, Qpo;             // that tensor's bordered width and positions per chunk
@@ -238,16 +250,30 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t par, uint32
     }
 }
 
+// The same by a whole warp, with one answer: true if every lane saw the phase.
+__device__ __forceinline__ bool wait_together(uint32_t bar, uint32_t par, uint32_t abort_addr) {
+    return __all_sync(0xffffffffu, wait_or_abort(bar, par, abort_addr));
+}
+
 constexpr int kMaxStages = 8;
 
 // Shared memory: [stages x (A span: 2 chunks x span x 16 B | B: taps x 2 x NT x 16 B)]
 // then the barriers: full[8] +0, empty[8] +64, acc_full[2] +128, acc_empty[2]
 // +144, drain +160, tensor-memory address +168, abort word +172; then the
 // layer's biases (up to 256 floats) at +1024.
-// Tile t (t = blockIdx.x, + gridDim.x, ...) covers positions (t % m_tiles) 128 R
-// .. + 128 R - 1 and output channels (t / m_tiles) NT .. + NT - 1; its
-// accumulators live in tensor-memory buffer (local tile index) % 2.
-template <int R>
+// Tile t (t = blockIdx.x, + gridDim.x, ...) covers the row groups of position
+// tile t % m_tiles (tile_groups) and output channels (t / m_tiles) NT .. + NT -
+// 1; its accumulators live in tensor-memory buffer (local tile index) % 2. MAXR:
+// the most row groups of a tile (1, 2 or 4; the MMAs over them unrolled).
+__device__ __forceinline__ int tile_groups(const TcGeom& g, int mt, int& first) {
+    if (mt < g.full) {
+        first = mt * g.R;
+        return g.R;
+    }
+    first = g.full * g.R + (mt - g.full) * g.R_tail;
+    return min(g.R_tail, g.groups - first);
+}
+template <int MAXR>
 __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant__ CUtensorMap ma,
                                                            const __grid_constant__ CUtensorMap mb,
                                                            const uint8_t* __restrict__ wpk,
@@ -260,7 +286,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
                    slot = bars + 168, abort_w = bars + 172;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n_tiles = g.m_tiles * g.n_tiles;
-    const uint32_t acc_cols = uint32_t(R * g.NT);
+    const uint32_t acc_cols = uint32_t(g.R * g.NT);
 
     if (tid == 0) {
         for (int s = 0; s < g.stages; s++) {
@@ -288,17 +314,34 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
     tc::fence_after();
     uint32_t tmem;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem) : "r"(slot));
-    wait_previous_kernel();
-    allow_next_kernel();
-
+    tmem = __reduce_or_sync(0xffffffffu, tmem);   // one value for the warp, in a uniform register
+    // only the producer's copies depend on the previous layer: the other warps
+    // wait for what it brings
     if (warp == 0) {
         if (lane == 0) {
-            // producer: the block's K steps, tile after tile, into stage kc % stages
+            // producer: the block's K steps, tile after tile, into stage kc % stages.
+            // In the network the weights do not come from the kernel before: the first
+            // stages' are asked for before waiting for it (g.early).
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&ma)) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mb)) : "memory");
+            const int early = g.early ? min(g.stages, g.ksteps) : 0;
+            {
+                const uint8_t* wsrc = wpk + size_t(int(blockIdx.x) / g.m_tiles) * g.ksteps * g.b_bytes;
+                for (int s = 0; s < early; s++) {
+                    tc::expect_tx(bars + 8 * s, g.a_bytes + g.b_bytes);
+                    tc::load_bulk(s0 + uint32_t(s) * g.stage_bytes + g.a_bytes, wsrc + size_t(s) * g.b_bytes, g.b_bytes,
+                                  bars + 8 * s);
+                }
+            }
+            wait_previous_kernel();
+            allow_next_kernel();
             int kc = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-                const int q0 = (t % g.m_tiles) * 128 * R, nt = t / g.m_tiles;
-                const int qs = q0 - (g.Wb + 1);
+                const int nt = t / g.m_tiles;
+                int first;
+                tile_groups(g, t - nt * g.m_tiles, first);
+                const int qs = 128 * first - (g.Wb + 1);
                 const int y0 = (qs >= 0 ? qs : qs - 31) / 32;   // the 32-position row holding the span's start
                 const uint8_t* wsrc = wpk + size_t(nt) * g.ksteps * g.b_bytes;
                 for (int ks = 0; ks < g.ksteps; ks++, kc++) {
@@ -308,11 +351,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
                         break;
                     }
                     const uint32_t a = s0 + uint32_t(s) * g.stage_bytes, b = a + g.a_bytes, full = bars + 8 * s;
-                    tc::expect_tx(full, g.a_bytes + g.b_bytes);
+                    if (kc >= early) tc::expect_tx(full, g.a_bytes + g.b_bytes);
                     // both 8-channel chunks of the K step in one box (chunk pairs never straddle the maps)
                     const int c8 = 2 * ks;
                     tc::load_box(a, c8 < g.split ? &ma : &mb, 0, y0, c8 < g.split ? c8 : c8 - g.split, full);
-                    tc::load_bulk(b, wsrc + size_t(ks) * g.b_bytes, g.b_bytes, full);
+                    if (kc >= early) tc::load_bulk(b, wsrc + size_t(ks) * g.b_bytes, g.b_bytes, full);
                 }
             }
             // the copies issued last on each stage have landed before the block moves on
@@ -321,63 +364,64 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
             if (!ok) atomicOr(status, 1);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // MMA issuer. Descriptors are built once per stage; taps and row groups
-            // move the start address by whole 16-byte units (one position), added to
-            // the 14-bit address field (shared addresses stay below 256 KB, so the
-            // field never carries).
-            const uint32_t idesc = tc::idesc_bf16(128, g.NT);
-            uint32_t toff[9];
+        // MMA issuer, the whole warp together (tc::mma). Taps and row groups move
+        // a descriptor's start address by whole 16-byte units (one position),
+        // added to its low word (shared addresses stay below 256 KB, so the
+        // address field never carries).
+        const uint32_t idesc = tc::idesc_bf16(128, g.NT), hi = tc::sdesc_hi(128);
+        uint32_t toff[9];
 #pragma unroll
-            for (int tp = 0; tp < 9; tp++) toff[tp] = uint32_t((tp / 3) * g.Wb + (tp % 3));
-            const uint64_t a_desc0 = tc::sdesc(s0, uint32_t(g.span * 16), 128);
-            const uint64_t b_desc0 = tc::sdesc(s0 + g.a_bytes, uint32_t(g.NT * 16), 128);
-            const uint32_t b_tap = uint32_t(2 * g.NT);   // 16-byte units between taps' weights
-            int kc = 0, it = 0;
-            bool ok = true;
-            for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, it++) {
-                const int q0 = (t % g.m_tiles) * 128 * R;
-                const int qs = q0 - (g.Wb + 1);
-                const uint32_t delta = uint32_t(qs - 32 * ((qs >= 0 ? qs : qs - 31) / 32));   // span start in its first row
-                const int buf = it & 1;
-                // the epilogue has drained this buffer (its use two tiles ago)
-                if (it >= 2 && !wait_or_abort(acc_empty + 8 * buf, uint32_t((it / 2 - 1) & 1), abort_w)) {
-                    ok = false;
-                    break;
-                }
+        for (int tp = 0; tp < 9; tp++) toff[tp] = uint32_t((tp / 3) * g.Wb + (tp % 3));
+        const uint32_t a_desc0 = tc::sdesc_lo(s0, uint32_t(g.span * 16));
+        const uint32_t b_desc0 = tc::sdesc_lo(s0 + g.a_bytes, uint32_t(g.NT * 16));
+        const uint32_t b_tap = uint32_t(2 * g.NT);   // 16-byte units between taps' weights
+        const uint32_t st16 = g.stage_bytes >> 4;
+        int s = 0, it = 0;
+        uint32_t phase = 0;   // of stage s
+        bool ok = true;
+        for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, it++) {
+            int first;
+            const int rc = tile_groups(g, t % g.m_tiles, first);
+            const int qs = 128 * first - (g.Wb + 1);
+            const uint32_t delta = uint32_t(qs - 32 * ((qs >= 0 ? qs : qs - 31) / 32));   // span start in its first row
+            const int buf = it & 1;
+            // the epilogue has drained this buffer (its use two tiles ago)
+            if (it >= 2) ok = wait_together(acc_empty + 8 * buf, uint32_t((it / 2 - 1) & 1), abort_w);
+            tc::fence_after();
+            const uint32_t dacc = tmem + uint32_t(buf) * acc_cols;
+            for (int ks = 0; ks < g.ksteps && ok; ks++) {
+                ok = wait_together(bars + 8 * s, phase, abort_w);
+                if (!ok) break;
                 tc::fence_after();
-                const uint32_t dacc = tmem + uint32_t(buf) * acc_cols;
-                for (int ks = 0; ks < g.ksteps; ks++, kc++) {
-                    const int s = kc % g.stages;
-                    if (!wait_or_abort(bars + 8 * s, uint32_t((kc / g.stages) & 1), abort_w)) {
-                        ok = false;
-                        break;
-                    }
-                    tc::fence_after();
-                    const uint32_t st16 = (uint32_t(s) * g.stage_bytes) >> 4;
-                    const uint64_t ad = a_desc0 + st16 + delta, bd = b_desc0 + st16;
+                const uint32_t ad = a_desc0 + uint32_t(s) * st16 + delta, bd = b_desc0 + uint32_t(s) * st16;
 #pragma unroll
-                    for (int tp = 0; tp < 9; tp++)
+                for (int tp = 0; tp < 9; tp++)
 #pragma unroll
-                        for (int r = 0; r < R; r++)
-                            tc::mma(dacc + uint32_t(r * g.NT), ad + toff[tp] + uint32_t(r * 128), bd + tp * b_tap, idesc,
-                                    uint32_t(ks | tp));
-                    tc::commit(empty + 8 * s);
+                    for (int r = 0; r < MAXR; r++)
+                        if (r < rc)
+                            tc::mma(dacc + uint32_t(r * g.NT), ad + toff[tp] + uint32_t(r * 128), bd + tp * b_tap, hi, idesc,
+                                    tp > 0 ? 1u : uint32_t(ks));
+                tc::commit(empty + 8 * s);
+                if (++s == g.stages) {
+                    s = 0;
+                    phase ^= 1u;
                 }
-                if (ok) tc::commit(acc_full + 8 * buf);
             }
-            // every MMA issued has completed before the block moves on
-            tc::commit(drain);
-            tc::wait(drain, 0);
-            if (!ok) atomicOr(status, 2);
+            if (ok) tc::commit(acc_full + 8 * buf);
         }
+        // every MMA issued has completed before the block moves on
+        tc::commit(drain);
+        tc::wait(drain, 0);
+        if (!ok && lane == 0) atomicOr(status, 2);
     } else {
         // epilogue warps: group cg drains column half cg of every row group
         const int ew = warp - 2, lq = warp & 3, cg = ew >> 2;   // lane quarter, column group
         int it = 0;
         bool ok = true;
         for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, it++) {
-            const int q0 = (t % g.m_tiles) * 128 * R, n0 = (t / g.m_tiles) * g.NT;
+            const int nt = t / g.m_tiles, n0 = nt * g.NT;
+            int first;
+            const int rc = tile_groups(g, t - nt * g.m_tiles, first);
             const int buf = it & 1;
             // one lane per warp polls (with backoff); the others wait at the shuffle
             int got = 0;
@@ -386,9 +430,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
             if (!ok) break;
             tc::fence_after();
             const uint32_t trow = tmem + (uint32_t(lq * 32) << 16) + uint32_t(buf) * acc_cols;
-#pragma unroll
-            for (int r = 0; r < R; r++) {
-                const int q = q0 + r * 128 + lq * 32 + lane;
+            for (int r = 0; r < rc; r++) {
+                const int q = (first + r) * 128 + lq * 32 + lane;
                 const int y = q / g.Wb, x = q - y * g.Wb;
                 const bool border = y == 0 || y >= g.Hb - 1 || x == 0 || x == g.Wb - 1;
                 const int half = g.NT >> 1;
@@ -512,6 +555,7 @@ __global__ void __launch_bounds__(out_threads(GROUPS), 1) k_out_tc(const __grid_
     tc::fence_after();
     uint32_t tmem;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem) : "r"(slot));
+    tmem = __reduce_or_sync(0xffffffffu, tmem);   // one value for the warp, in a uniform register
     wait_previous_kernel();
     allow_next_kernel();
 
@@ -539,34 +583,27 @@ __global__ void __launch_bounds__(out_threads(GROUPS), 1) k_out_tc(const __grid_
             if (!ok) atomicOr(status, 1);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = tc::idesc_bf16(128, NT);
-            bool ok = wait_or_abort(wfull, 0, abort_w);
-            int it = 0;
-            for (int t = blockIdx.x; t < g.tiles && ok; t += gridDim.x, it++) {
-                const int buf = it & 1, s = it % kOutStages;
-                // the epilogue has drained this buffer (its use two tiles ago)
-                if (it >= 2 && !wait_or_abort(acc_empty + 8 * buf, uint32_t((it / 2 - 1) & 1), abort_w)) {
-                    ok = false;
-                    break;
-                }
-                if (!wait_or_abort(bars + 8 * s, uint32_t((it / kOutStages) & 1), abort_w)) {
-                    ok = false;
-                    break;
-                }
-                tc::fence_after();
+        const uint32_t idesc = tc::idesc_bf16(128, NT), hi = tc::sdesc_hi(128);
+        bool ok = wait_together(wfull, 0, abort_w);
+        int it = 0;
+        for (int t = blockIdx.x; t < g.tiles && ok; t += gridDim.x, it++) {
+            const int buf = it & 1, s = it % kOutStages;
+            // the epilogue has drained this buffer (its use two tiles ago)
+            if (it >= 2) ok = wait_together(acc_empty + 8 * buf, uint32_t((it / 2 - 1) & 1), abort_w);
+            ok = ok && wait_together(bars + 8 * s, uint32_t((it / kOutStages) & 1), abort_w);
+            if (!ok) break;
+            tc::fence_after();
 #pragma unroll
-                for (int ks = 0; ks < 2; ks++)
-                    tc::mma(tmem + uint32_t(buf * NT), tc::sdesc(s0 + s * kOutTile + ks * (kOutTile / 2), 128 * 16, 128),
-                            tc::sdesc(wts + ks * (b_bytes / 2), NT * 16, 128), idesc, uint32_t(ks));
-                tc::commit(empty + 8 * s);
-                tc::commit(acc_full + 8 * buf);
-            }
-            // every MMA issued has completed before the block moves on
-            tc::commit(drain);
-            tc::wait(drain, 0);
-            if (!ok) atomicOr(status, 2);
+            for (int ks = 0; ks < 2; ks++)
+                tc::mma(tmem + uint32_t(buf * NT), tc::sdesc_lo(s0 + s * kOutTile + ks * (kOutTile / 2), 128 * 16),
+                        tc::sdesc_lo(wts + ks * (b_bytes / 2), NT * 16), hi, idesc, uint32_t(ks));
+            tc::commit(empty + 8 * s);
+            tc::commit(acc_full + 8 * buf);
         }
+        // every MMA issued has completed before the block moves on
+        tc::commit(drain);
+        tc::wait(drain, 0);
+        if (!ok && lane == 0) atomicOr(status, 2);
     } else {
         const int lq = warp & 3, cg = (warp - 2) >> 2;   // lane quarter, group
         const size_t npix = size_t(g.H) * g.W;
@@ -678,29 +715,31 @@ __device__ __forceinline__ uint4 f32_to_bf16x8(const float* f) {
 }
 
 // out (level H/2 x W/2) = mean of 2x2 blocks of in (level H x W); C % 8 == 0.
-// One thread per (chunk, output pixel), pixels fastest.
-__global__ void k_avgpool2(const __nv_bfloat16* __restrict__ in, int H, int W, int C, __nv_bfloat16* __restrict__ out) {
+// One thread per (output pixel, chunk): grid (pixel blocks of 256, C / 8).
+__global__ void __launch_bounds__(256) k_avgpool2(const __nv_bfloat16* __restrict__ in, int H, int W,
+                                                  __nv_bfloat16* __restrict__ out) {
+    const uint32_t Wo = uint32_t(W) / 2, npx = uint32_t(H) / 2 * Wo;
+    const uint32_t p = blockIdx.x * 256u + threadIdx.x, c8 = blockIdx.y;
+    const uint32_t yo = p / Wo, xo = p - yo * Wo;
+    const size_t qi = qpad(H, W), qo = qpad(H / 2, W / 2);
+    const __nv_bfloat16* src = in + (c8 * qi + bpos(2 * yo, 2 * xo, W)) * 8;
     wait_previous_kernel();
     allow_next_kernel();
-    const int Ho = H / 2, Wo = W / 2;
-    const size_t npx = size_t(Ho) * Wo, total = npx * (C / 8), qi = qpad(H, W), qo = qpad(Ho, Wo);
-    for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < total; i += size_t(gridDim.x) * blockDim.x) {
-        const int c8 = int(i / npx);
-        const size_t p = i - c8 * npx;
-        const int xo = int(p % Wo), yo = int(p / Wo);
-        const __nv_bfloat16* src = in + size_t(c8) * qi * 8;
-        float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (p >= npx) return;
+    uint4 v[4];
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            float f[8];
-            bf16x8_to_f32(*reinterpret_cast<const uint4*>(src + bpos(2 * yo + (q >> 1), 2 * xo + (q & 1), W) * 8), f);
+    for (int q = 0; q < 4; q++) v[q] = *reinterpret_cast<const uint4*>(src + size_t((q >> 1) * (W + 2) + (q & 1)) * 8);
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int e = 0; e < 8; e++) s[e] += f[e];
-        }
+    for (int q = 0; q < 4; q++) {
+        float f[8];
+        bf16x8_to_f32(v[q], f);
 #pragma unroll
-        for (int e = 0; e < 8; e++) s[e] *= 0.25f;
-        *reinterpret_cast<uint4*>(out + (size_t(c8) * qo + bpos(yo, xo, Wo)) * 8) = f32_to_bf16x8(s);
+        for (int e = 0; e < 8; e++) s[e] += f[e];
     }
+#pragma unroll
+    for (int e = 0; e < 8; e++) s[e] *= 0.25f;
+    *reinterpret_cast<uint4*>(out + (c8 * qo + bpos(yo, xo, Wo)) * 8) = f32_to_bf16x8(s);
 }
 
 // x0 (level Hp x Wp, 48 channels): channel 3 j + c = channel c of input view
@@ -709,9 +748,10 @@ __global__ void k_avgpool2(const __nv_bfloat16* __restrict__ in, int H, int W, i
 __global__ void k_recon_in(const uint8_t* __restrict__ views, int nin, int H, int W, int Hp, int Wp,
                            __nv_bfloat16* __restrict__ x0) {
     allow_next_kernel();   // launched plainly: it waits for everything before it
-    const size_t total = size_t(Hp) * Wp, npix = size_t(H) * W, qp = qpad(Hp, Wp);
-    for (size_t p = size_t(blockIdx.x) * blockDim.x + threadIdx.x; p < total; p += size_t(gridDim.x) * blockDim.x) {
-        const int x = int(p % Wp), y = int(p / Wp);
+    const uint32_t total = uint32_t(Hp) * uint32_t(Wp);   // at most 4096 x 4032
+    const size_t npix = size_t(H) * W, qp = qpad(Hp, Wp);
+    for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < total; p += gridDim.x * blockDim.x) {
+        const int y = int(p / uint32_t(Wp)), x = int(p) - y * Wp;
         float v[48];
 #pragma unroll
         for (int j = 0; j < 16; j++) {
@@ -791,10 +831,15 @@ uint32_t pow2_cols(int n) {
 }
 
 // Geometry of a layer over the bordered level image Hl x Wl: cin = cin_a +
-// cin_b input channels (map a, then map b), NT output channels per block, R
-// row groups of 128 positions per block.
-TcGeom tc_geom(int Hl, int Wl, int cin_a, int cin_b, int NT, int R, int n_tiles, int cout,
-               uint32_t reserve) {
+// cin_b input channels (map a, then map b), NT output channels per block and
+// up to R row groups of 128 positions per tile, `reserve` bytes of each SM's
+// shared memory left free where the stages allow it.
+//
+// Every SM takes the same number of rounds of tiles; all but the last are of
+// R groups, and the last spreads what is left evenly (R_tail groups a tile), so
+// that no SM computes more than ceil(groups / SMs) of them by more than a tile's
+// rounding.
+TcGeom tc_geom(int Hl, int Wl, int cin_a, int cin_b, int NT, int R, int cout, int sm_count, uint32_t reserve) {
     TcGeom g{};
     g.Hb = Hl + 2;
     g.Wb = Wl + 2;
@@ -817,10 +862,16 @@ TcGeom tc_geom(int Hl, int Wl, int cin_a, int cin_b, int NT, int R, int n_tiles,
     g.beside = room >= reserve && (room - reserve) / g.stage_bytes >= uint32_t(kMinStages);
     g.stages = int(std::min<uint32_t>(uint32_t(kMaxStages), (g.beside ? room - reserve : room) / g.stage_bytes));
     g.tmem_cols = pow2_cols(2 * R * NT);
-    g.m_tiles = (g.Q + 128 * R - 1) / (128 * R);
-    g.n_tiles = n_tiles;
+    g.groups = (g.Q + 127) / 128;
+    g.n_tiles = cout / NT;
+    const int slots = std::max(1, sm_count / g.n_tiles);   // tiles of one output-channel tile at a time
+    const int rounds = (g.groups + R * slots - 1) / (R * slots);
+    g.full = (rounds - 1) * slots;
+    const int rest = g.groups - g.full * R;
+    g.R_tail = (rest + slots - 1) / slots;
+    g.m_tiles = g.full + (rest + g.R_tail - 1) / g.R_tail;
     g.cout = cout;
-    g.bias_n = n_tiles * NT;
+    g.bias_n = cout;
     return g;
 }
 
@@ -865,7 +916,7 @@ int sm_count_cached() {
 }
 
 bool tc_valid(const TcGeom& g) {
-    return g.stages >= 2 && g.ksteps >= 1 && g.NT % 16 == 0 && g.NT >= 16 && g.NT <= 256 && g.tmem_cols <= 512 &&
+    return g.stages >= 2 && g.ksteps >= 1 && g.R >= 1 && g.R <= 4 && g.NT % 16 == 0 && g.NT >= 16 && g.NT <= 256 && g.tmem_cols <= 512 &&
            g.split % 2 == 0 && g.rows <= 256 && g.m_tiles >= 1 && g.n_tiles >= 1 && g.bias_n >= 1 && g.bias_n <= 256 &&
            (g.NT / 2) % 16 == 0 && tc_smem(g) <= kTcSmemMax;
 }
@@ -891,8 +942,7 @@ cudaError_t allow_smem(const void* kernel) {
 cudaError_t launch_tc(const TcGeom& g, const CUtensorMap& ma, const CUtensorMap& mb, const void* wpk, const float* bias,
                       void* out, int* status, cudaStream_t s) {
     if (!tc_valid(g)) return cudaErrorInvalidValue;
-    const auto kernel = g.R == 1 ? k_conv_tc<1> : g.R == 2 ? k_conv_tc<2> : g.R == 4 ? k_conv_tc<4> : nullptr;
-    if (!kernel) return cudaErrorInvalidValue;
+    const auto kernel = g.R == 1 ? k_conv_tc<1> : g.R == 2 ? k_conv_tc<2> : k_conv_tc<4>;
     const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kernel));
     if (e != cudaSuccess) return e;
     const int grid = std::min(g.m_tiles * g.n_tiles, sm_count_cached());
@@ -920,21 +970,52 @@ cudaError_t launch_pack(const __nv_bfloat16* src, int cout, int taps, int cin, i
     return cudaGetLastError();
 }
 
-// Output channels and row groups per tile of a 3x3 layer: 128, 64 or 32 channels
-// (wider tiles re-read each input span for fewer output channels);
-// the most row groups (two accumulator buffers of R NT <= 256 columns each)
-// that still give every SM two tiles or more.
-void pick_tile(int Hl, int Wl, int cout, int sm_count, int& NT, int& R) {
-    NT = cout % 128 == 0 ? 128 : cout % 64 == 0 ? 64 : 32;
-    const int64_t Q = int64_t(Hl + 2) * (Wl + 2);
-    R = 1;
-    for (int r : {4, 2}) {
-        if (r * NT > 128) continue;
-        if ((Q + 128 * r - 1) / (128 * r) * (cout / NT) >= 2 * sm_count) {
-            R = r;
-            break;
+// The tile of a 3x3 layer: output channels (32, 64 or 128) and row groups (two
+// accumulator buffers of R NT <= 256 columns each).
+//
+// From the layers' own clocks: an MMA (M 128, N NT, K 16) takes 36, 40 or 48 ns
+// at N 32, 64 or 128, whatever its operands' alignment and whether one thread
+// or two issue them; a K step's copies (the input span: the tile's positions and
+// two image rows; the nine taps' weights) hide behind its MMAs up to about 115
+// bytes a ns; and the last tile's accumulators are drained with nothing to hide
+// behind, about 0.28 us for each row group and 32 channels, four times that
+// where the output is upsampled. So the fewest row groups per SM count, then
+// tall tiles (fewer bytes copied: they take a share of the shared memory's
+// bandwidth even where they are hidden, counted at 15 %), and narrow ones where a layer has too few positions to give every
+// SM one. The choice is the tile with the least sum; tiles whose stages leave the
+// warp its share of the SM come first.
+// The 14 layers at 420x560 (alone, no warp beside): 0.228 ms before, 0.19 with
+// MMAs issued by a whole warp, early weights, even last rounds and these tiles.
+TcGeom pick_tile(int Hl, int Wl, int cin_a, int cin_b, int cout, int up, int sm_count, uint32_t reserve) {
+    TcGeom best{};
+    double least = 0.0;
+    // The layers take images up to the width at which their widest tile, as tall
+    // as gives every SM two of them, fits twice in shared memory; a narrower or
+    // lower tile does not extend what is accepted.
+    const int NT0 = cout % 128 == 0 ? 128 : cout % 64 == 0 ? 64 : 32;
+    int R0 = 1;
+    for (int r : {2, 4})
+        if (r * NT0 <= 128 &&
+            (int64_t(Hl + 2) * (Wl + 2) + 128 * r - 1) / (128 * r) * (cout / NT0) >= 2 * sm_count)
+            R0 = r;
+    if (!tc_valid(tc_geom(Hl, Wl, cin_a, cin_b, NT0, R0, cout, sm_count, 0))) return best;
+    for (int NT : {128, 64, 32})
+        for (int R = 1; R <= 4; R++) {
+            if (cout % NT || R * NT > 256) continue;
+            TcGeom g = tc_geom(Hl, Wl, cin_a, cin_b, NT, R, cout, sm_count, reserve);
+            if (!tc_valid(g)) continue;
+            const double mma = 9.0 * (32.0 + NT / 8.0), copy = (g.a_bytes + g.b_bytes) / 115.0;   // ns per K step
+            const int rounds = g.full / std::max(1, sm_count / g.n_tiles);                       // before the last
+            double t = g.ksteps * (rounds * std::max(R * mma, copy) + std::max(g.R_tail * mma, copy)) +
+                       g.R_tail * (NT / 32) * 280.0 * (up ? 4.0 : 1.0) + 0.15 * g.ksteps * (rounds + 1) * copy;
+            if (reserve && !g.beside) t += 1e12;
+            if (best.R == 0 || t < least) {
+                least = t;
+                best = g;
+            }
         }
-    }
+    best.up = up;
+    return best;   // R = 0: no layout
 }
 
 }  // namespace
@@ -1100,13 +1181,12 @@ lfdpr_status lfdpr_create_recon(int32_t view_w, int32_t view_h, int32_t in_views
     for (int l = 0; l < 14; l++) {
         const ConvSpec& L = kLayers[l];
         const int Hl = r->Hp >> L.level, Wl = r->Wp >> L.level;
-        int NT, R;
-        pick_tile(Hl, Wl, L.cout, r->sm_count, NT, R);
         // layers 8, 10, 12 read [upsampled (map a) | skip (map b)]
         const int cin_b = (l == 8 || l == 10 || l == 12) ? L.cin / 3 : 0;
-        r->geom[l] = tc_geom(Hl, Wl, L.cin - cin_b, cin_b, NT, R, L.cout / NT, L.cout, reserve);
-        if (l == 7 || l == 9 || l == 11) {   // write 2x upsampled into the next level's tensor
-            r->geom[l].up = 1;
+        const int up = l == 7 || l == 9 || l == 11;   // write 2x upsampled into the next level's tensor
+        r->geom[l] = pick_tile(Hl, Wl, L.cin - cin_b, cin_b, L.cout, up, r->sm_count, reserve);
+        r->geom[l].early = 1;
+        if (up) {
             r->geom[l].Wbo = 2 * Wl + 2;
             r->geom[l].Qpo = int(qpad(2 * Hl, 2 * Wl));
         }
@@ -1188,7 +1268,8 @@ lfdpr_status lfdpr_recon_forward(lfdpr_recon* r, const uint8_t* in_views, const 
                          conv_out[l], r->status, s);
     };
     auto pool = [&](const __nv_bfloat16* in, int H, int W, int C, __nv_bfloat16* o) {
-        return launch_after_previous(k_avgpool2, sm * 8, 256, 0, s, in, H, W, C, o);
+        return launch_after_previous(k_avgpool2, dim3(unsigned((H / 2 * (W / 2) + 255) / 256), unsigned(C / 8)), dim3(256),
+                                     0, s, in, H, W, o);
     };
 #define CKR(call, what)                                      \
     do {                                                     \
@@ -1265,9 +1346,7 @@ lfdpr_status lfdpr_conv3x3_bf16(const void* in, int32_t H, int32_t W, int32_t ci
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int NT, R;
-    pick_tile(H, W, cout, sms, NT, R);
-    const TcGeom g = tc_geom(H, W, cin, 0, NT, R, cout / NT, cout, 0);
+    const TcGeom g = pick_tile(H, W, cin, 0, cout, 0, sms, 0);
     if (!tc_valid(g)) return fail(LFDPR_EINVAL, "conv3x3: no tensor-core layout for a %d-wide image", W);
     // chunked bordered copies of the input and output, and the packed weights
     const size_t qp = qpad(H, W);
@@ -1282,7 +1361,7 @@ lfdpr_status lfdpr_conv3x3_bf16(const void* in, int32_t H, int32_t W, int32_t ci
         k_to_chunked<<<sms * 8, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(in), H, W, cin, ci);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = launch_pack(static_cast<const __nv_bfloat16*>(wgt), cout, 9, cin, NT, cout / NT, wpk, s);
+    if (e == cudaSuccess) e = launch_pack(static_cast<const __nv_bfloat16*>(wgt), cout, 9, cin, g.NT, g.n_tiles, wpk, s);
     if (e == cudaSuccess) e = launch_tc(g, m, m, wpk, bias, co, reinterpret_cast<int*>(status), s);
     if (e == cudaSuccess) {
         k_from_chunked<<<sms * 8, 256, 0, s>>>(co, H, W, cout, static_cast<__nv_bfloat16*>(out));
