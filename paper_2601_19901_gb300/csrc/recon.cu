@@ -921,8 +921,10 @@ bool tc_valid(const TcGeom& g) {
            (g.NT / 2) % 16 == 0 && tc_smem(g) <= kTcSmemMax;
 }
 
-// The largest dynamic shared memory for a kernel of this file, asked for once
-// per kernel and device.
+// The largest dynamic shared memory for a kernel of this file, and the SM's
+// whole shared memory as its split from L1: asked for once per kernel and
+// device. With a split sized for the layer's own block, the warp's blocks do
+// not fit beside it, though the shared memory is there.
 cudaError_t allow_smem(const void* kernel) {
     static std::mutex mu;
     static std::set<std::pair<const void*, int>> done;
@@ -931,7 +933,9 @@ cudaError_t allow_smem(const void* kernel) {
     if (d != cudaSuccess) return d;
     std::lock_guard<std::mutex> lock(mu);
     if (done.count({kernel, dev})) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTcSmemMax));
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTcSmemMax));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess) done.insert({kernel, dev});
     return e;
 }

@@ -103,10 +103,10 @@ int warp_threads(int W) {
 // 12 views of 420x560 to 48, alone, a block per pair: 0.117 -> 0.107 ms (117 M
 // -> 82 M warp instructions). Beside the layers the blocks last, two per SM on
 // shared memory that the layers leave free, the next pair's rows asked of L1:
-// the forward pass takes 0.420 -> 0.407 ms there, where the layers themselves
-// use the shared memory's bandwidth, and 0.224 -> 0.204 at 333x251, where they
-// wait for launches and copies. The minimum as two 32-bit ones in two sweeps
-// took 0.128 alone, and blocks of twice the threads 0.121.
+// the forward pass takes 0.283 ms there, 0.242 without the warp (0.353 while
+// the SMs' split between L1 and shared memory kept the two apart), and 0.156 ms
+// against 0.149 at 333x251. The minimum as two 32-bit ones in two sweeps took
+// 0.128 alone, and blocks of twice the threads 0.121.
 __global__ void __launch_bounds__(kWarpThreads) k_warp_views(WarpArgs a) {
     extern __shared__ __align__(16) uint8_t s_raw[];
     const int W = a.W, V = views_per_pass(W), WS = row_stride(W);
@@ -281,8 +281,12 @@ cudaError_t launch_warp_views(const uint8_t* views, const uint64_t* keys, const 
     if (nin < 2 || nout < 1 || W < 1 || H < 1 || W > kMaxWarpWidth || H > 65535 || nout > kMaxRenderViews || !(ipw > 0.0f))
         return cudaErrorInvalidValue;
     const size_t smem = warp_smem(nin, nout, W);
+    // the split from L1 that the network's layers have, so that it runs beside them
+    cudaError_t e = cudaFuncSetAttribute(k_warp_views, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                         cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
     if (smem > 48u * 1024u) {
-        const cudaError_t e = cudaFuncSetAttribute(k_warp_views, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        e = cudaFuncSetAttribute(k_warp_views, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         if (e != cudaSuccess) return e;
     }
     WarpArgs a{views, keys, in_eyes, out_eyes, nin, nout, W, H, ipw, out};
