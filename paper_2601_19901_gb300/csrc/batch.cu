@@ -27,7 +27,7 @@ struct lfdpr_batch {
     float* d_models = nullptr;       // [n][12] model rows read by k_setup
     float* h_models = nullptr;       // pinned staging of the same
     cudaEvent_t staged = nullptr;    // the last copy out of h_models has run
-    SplatScene* d_scenes = nullptr;  // [n] for the batched splat
+    BatchScenes scenes{};            // [n] for the batched splat
     cudaStream_t cap = nullptr;      // the stream the graph is captured on
     std::vector<cudaStream_t> br;    // branch streams
     std::vector<cudaEvent_t> ev;     // fork, fork2, joins
@@ -89,7 +89,6 @@ void free_batch(lfdpr_batch* b) {
     if (b->staged) cudaEventDestroy(b->staged);
     dev_free(b->d_models);
     host_free(b->h_models);
-    dev_free(b->d_scenes);
     delete b;
 }
 
@@ -113,7 +112,7 @@ lfdpr_status record_batch(lfdpr_batch* b) {
         CK(cudaEventRecord(b->ev[2 + j], b->br[j]), "batch: join");
         CK(cudaStreamWaitEvent(s, b->ev[2 + j], 0), "batch: join wait");
     }
-    CK(launch_splat_batch(b->d_scenes, b->n, b->cfg.splat_slots, b->cfg.splat_blocks_per_sm, b->sm_count, s),
+    CK(launch_splat_batch(b->scenes, b->n, b->cfg.splat_slots, b->cfg.splat_blocks_per_sm, b->sm_count, s),
        "launch k_splat_batch");
     CK(cudaEventRecord(fork2, s), "batch: fork");
     for (int j = 0; j < K; j++) CK(cudaStreamWaitEvent(b->br[j], fork2, 0), "batch: branch wait");
@@ -206,20 +205,18 @@ lfdpr_status lfdpr_create_batch(lfdpr_display* const* displays, lfdpr_mesh* cons
     b->cfg.branches = std::min(4, n);
     b->cfg.splat_blocks_per_sm = 16;
     b->cfg.splat_slots = fewest_slots(max_views);
-    std::vector<SplatScene> sc(n);
     for (int i = 0; i < n; i++) {
-        sc[i].dc = displays[i]->dc;
-        sc[i].ex = displays[i]->d_ex;
-        sc[i].ctr = displays[i]->ctr;
-        sc[i].work = displays[i]->work;
-        sc[i].rec = meshes[i]->rec;
-        sc[i].keys = displays[i]->keys;
+        SplatScene& sc = b->scenes.s[i];
+        sc.dc = displays[i]->dc;
+        sc.ex = displays[i]->d_ex;
+        sc.ctr = displays[i]->ctr;
+        sc.work = displays[i]->work;
+        sc.rec = meshes[i]->rec;
+        sc.keys = displays[i]->keys;
     }
     cudaError_t e;
     if ((e = dev_malloc(&b->d_models, sizeof(float) * 12 * n)) != cudaSuccess ||
         (e = host_malloc(&b->h_models, sizeof(float) * 12 * n)) != cudaSuccess ||
-        (e = dev_malloc(&b->d_scenes, sizeof(SplatScene) * n)) != cudaSuccess ||
-        (e = cudaMemcpy(b->d_scenes, sc.data(), sizeof(SplatScene) * n, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&b->staged, cudaEventDisableTiming)) != cudaSuccess ||
         (e = [&] {
             b->tev.assign(n + 1, nullptr);

@@ -373,9 +373,14 @@ struct SplatScene {
 };
 constexpr int kMaxBatchScenes = 64;
 constexpr int kMaxBatchViews = 4096;   // rendered views summed over a batch
+// A batch's scenes as one kernel parameter.
+struct BatchScenes {
+    SplatScene s[kMaxBatchScenes];
+};
+static_assert(sizeof(BatchScenes) < 32000, "kernel parameter limit");
 // Splat every scene of a batch in one persistent launch: grid_per_sm blocks
 // per SM, slots view slots per lane (1, 2, 3, 4, 6 or 8).
-cudaError_t launch_splat_batch(const SplatScene* scenes, int n_scenes, int slots, int grid_per_sm, int sm_count,
+cudaError_t launch_splat_batch(const BatchScenes& scenes, int n_scenes, int slots, int grid_per_sm, int sm_count,
                                cudaStream_t s);
 cudaError_t launch_resolve(const FrameArgs& a, cudaStream_t s);
 // pos [nr] (views on the display-view axis) and samples [n_samples][3] are

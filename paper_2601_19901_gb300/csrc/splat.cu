@@ -97,33 +97,33 @@ __device__ __forceinline__ uint32_t div_floor(uint32_t r, uint32_t n) {
     return r / n;
 }
 
-// Units of 2P points per warp: pairs per unit for S view slots per lane.
-template <int S>
-struct UnitPairs {
-    static constexpr int P = S <= 3 ? 2 : 1;
-};
+// Units of 2P points per warp: pairs per unit for S view slots per lane. Four
+// points share the unit's scan and fill its passes better than two: 96 views
+// (S = 6) 0.557 -> 0.471 ms. With S = 8 their segments would leave an SM three
+// blocks.
+__host__ __device__ constexpr int unit_pairs(int S) { return S <= 6 ? 2 : 1; }
 
 // Per-warp shared memory of the pooled splat: the unit's non-empty (point,
 // view) segments in candidate order (first candidate number,
 // x0 | n_columns << 14, view | point << 16, eye x) and its points' test
 // constants: (P0.x, -P0.y, D - P0.z, point id), (u-hat, work meta word),
 // (v-hat, u_min), (n-hat, v_min), the 2-D vertices, the cell's u and v bounds.
-template <int S>
+template <int S, int P>
 struct SplatWarpSmem {
-    static constexpr int P = UnitPairs<S>::P, kSegs = 32 * S * P;
+    static constexpr int kSegs = 32 * S * P;
     uint4 seg[kSegs];
     float4 pt[2 * P][6];
 };
 
 // Where the splat's units come from: one scene (its constants in the kernel's
-// parameters), or every scene of a batch (constants in shared memory; the
-// units of all scenes form one index range, scene by scene).
+// parameters), or every scene of a batch (an array of them there; the units of
+// all scenes form one index range, scene by scene).
 struct OneScene {
     static constexpr bool kMany = false;
     const FrameArgs& a;
     uint32_t n;       // work points
     uint32_t ex_s;    // shared-memory address of the eye positions
-    __device__ __forceinline__ int scene(uint32_t) const { return 0; }
+    __device__ __forceinline__ int scene(uint32_t, int) const { return 0; }
     __device__ __forceinline__ uint32_t first_unit(int) const { return 0u; }
     __device__ __forceinline__ const DispConst& dc(int) const { return a.dc; }
     __device__ __forceinline__ float eye(int, int v) const { return eye_x(ex_s, v); }
@@ -141,39 +141,35 @@ struct OneScene {
 
 struct ManyScenes {
     static constexpr bool kMany = true;
-    const SplatScene* scenes;
-    int n_scenes;
-    const DispConst* s_dc;
+    const BatchScenes& b;
     const uint32_t* s_unit0;   // first unit of each scene, then the total
     const uint32_t* s_n;       // work points of each scene
-    // the scene holding unit g: the last with s_unit0 <= g
-    __device__ __forceinline__ int scene(uint32_t g) const {
-        int lo = 0, hi = n_scenes - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (s_unit0[mid] <= g) lo = mid;
-            else hi = mid - 1;
-        }
-        return lo;
+    // the scene holding unit g, from that of the warp's unit before (units only
+    // go up): the last with s_unit0 <= g. One value for the warp, in a uniform
+    // register, so that the scene's constants are read from the kernel's
+    // parameters as those of a single scene are.
+    __device__ __forceinline__ int scene(uint32_t g, int from) const {
+        while (s_unit0[from + 1] <= g) from++;
+        return int(__reduce_max_sync(0xffffffffu, uint32_t(from)));
     }
     __device__ __forceinline__ uint32_t first_unit(int q) const { return s_unit0[q]; }
-    __device__ __forceinline__ const DispConst& dc(int q) const { return s_dc[q]; }
-    __device__ __forceinline__ float eye(int q, int v) const { return __ldg(scenes[q].ex + v); }
+    __device__ __forceinline__ const DispConst& dc(int q) const { return b.s[q].dc; }
+    __device__ __forceinline__ float eye(int q, int v) const { return __ldg(b.s[q].ex + v); }
     __device__ __forceinline__ uint32_t points(int q) const { return s_n[q]; }
-    __device__ __forceinline__ const WorkRec* work(int q) const { return scenes[q].work; }
-    __device__ __forceinline__ const TriRec* rec(int q) const { return scenes[q].rec; }
+    __device__ __forceinline__ const WorkRec* work(int q) const { return b.s[q].work; }
+    __device__ __forceinline__ const TriRec* rec(int q) const { return b.s[q].rec; }
     __device__ __forceinline__ unsigned long long* keys(int q) const {
-        return reinterpret_cast<unsigned long long*>(scenes[q].keys);
+        return reinterpret_cast<unsigned long long*>(b.s[q].keys);
     }
-    __device__ __forceinline__ Counters* ctr(int q) const { return scenes[q].ctr; }
+    __device__ __forceinline__ Counters* ctr(int q) const { return b.s[q].ctr; }
     __device__ __forceinline__ uint32_t lane_limit() const { return kSplatLaneLimit; }
     __device__ __forceinline__ int view_lo(int) const { return 0; }
-    __device__ __forceinline__ int view_hi(int q) const { return s_dc[q].nr; }
+    __device__ __forceinline__ int view_hi(int q) const { return b.s[q].dc.nr; }
 };
 
 // Candidate rr of segment e: its pixel, the test, and the depth-test atomic.
-template <int S>
-__device__ __forceinline__ void test_candidate(const DispConst& c, const SplatWarpSmem<S>& sm, const uint4& e,
+template <int S, int P>
+__device__ __forceinline__ void test_candidate(const DispConst& c, const SplatWarpSmem<S, P>& sm, const uint4& e,
                                                uint32_t rr, unsigned long long* keys, uint32_t npix,
                                                uint32_t& writes) {
     const float4* d = sm.pt[e.z >> 16];
@@ -203,8 +199,9 @@ __device__ __forceinline__ void test_candidate(const DispConst& c, const SplatWa
 // The splat proper: warps stride through units 0 .. total-1 of `src` (a
 // unit never spans two scenes).
 template <int S, class Src>
-__device__ __forceinline__ void splat_units(const Src& src, uint32_t total_units, SplatWarpSmem<S>& sm) {
-    constexpr int P = UnitPairs<S>::P;
+__device__ __forceinline__ void splat_units(const Src& src, uint32_t total_units,
+                                            SplatWarpSmem<S, unit_pairs(S)>& sm) {
+    constexpr int P = unit_pairs(S);
     const int lane = threadIdx.x & 31, sub = lane & 15, half = lane >> 4;
     const uint32_t lanes_below = (1u << lane) - 1u;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -213,7 +210,7 @@ __device__ __forceinline__ void splat_units(const Src& src, uint32_t total_units
     int cur = 0;
 
     for (uint32_t g = warp; g < total_units; g += n_warps) {
-        const int sc = src.scene(g);
+        const int sc = src.scene(g, cur);
         if constexpr (Src::kMany) {
             if (sc != cur) {
                 add_writes(src.ctr(cur), writes);
@@ -331,7 +328,7 @@ __device__ __forceinline__ void splat_units(const Src& src, uint32_t total_units
                     const uint4 e = sm.seg[s];
                     const uint32_t ny = (__float_as_uint(sm.pt[e.z >> 16][1].w) >> 14) & 0x7fffu;
                     const uint32_t m = (e.y >> 14) * ny;
-                    for (uint32_t rr = 0; rr < m; rr++) test_candidate<S>(c, sm, e, rr, keys, npix, writes);
+                    for (uint32_t rr = 0; rr < m; rr++) test_candidate<S, P>(c, sm, e, rr, keys, npix, writes);
                 }
                 continue;
             }
@@ -346,7 +343,7 @@ __device__ __forceinline__ void splat_units(const Src& src, uint32_t total_units
                 const uint32_t q = pass + uint32_t(lane);
                 if (q < total) {
                     const uint4 e = sm.seg[own];
-                    test_candidate<S>(c, sm, e, q - e.x, keys, npix, writes);
+                    test_candidate<S, P>(c, sm, e, q - e.x, keys, npix, writes);
                 }
             }
         }
@@ -356,8 +353,13 @@ __device__ __forceinline__ void splat_units(const Src& src, uint32_t total_units
 
 template <int S>
 __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
+    // With more than three slots the resolve is let in only when this block is
+    // done: its blocks waiting on the SMs cost a splat with 40 KB or more of shared
+    // memory a block a sixth of its time (96 views: 0.47 -> 0.56 ms). With fewer they
+    // cost nothing, and a small frame is 3 us shorter for them.
+    constexpr bool kLate = S > 3;
     wait_previous_kernel();
-    allow_next_kernel();
+    if constexpr (!kLate) allow_next_kernel();
     extern __shared__ __align__(16) uint8_t s_dyn[];
     __shared__ float s_ex[kMaxRenderViews];
     for (int v = threadIdx.x; v < a.dc.nr; v += blockDim.x) s_ex[v] = a.ex[v];
@@ -365,24 +367,28 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     if (a.ctr->overflow) return;
     const uint32_t n = a.ctr->n_work;
     const OneScene src{a, n, uint32_t(__cvta_generic_to_shared(s_ex))};
-    constexpr uint32_t unit = 2u * UnitPairs<S>::P;
-    splat_units<S>(src, (n + unit - 1u) / unit, reinterpret_cast<SplatWarpSmem<S>*>(s_dyn)[threadIdx.x >> 5]);
+    constexpr int P = unit_pairs(S);
+    constexpr uint32_t unit = 2u * P;
+    splat_units<S>(src, (n + unit - 1u) / unit, reinterpret_cast<SplatWarpSmem<S, P>*>(s_dyn)[threadIdx.x >> 5]);
+    if constexpr (kLate) allow_next_kernel();
 }
 
 // Every scene of a batch in one persistent launch: warps stride through the
-// units of all scenes, so scenes of uneven size share the machine. Each block
-// keeps every scene's display constants in shared memory.
+// units of all scenes, so scenes of uneven size share the machine. The scenes'
+// constants are kernel parameters read through a warp-uniform scene number: as
+// operands, not as shared-memory loads and registers of their own. 12 scenes of
+// 5,000 to 200,000 triangles, whole batch 4.10 -> 3.53 ms with them there and
+// four points a unit; asking L1 for the next unit's triangles as one scene does
+// costs more registers than the constants leave (3.68).
 template <int S>
-__global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat_batch(const SplatScene* __restrict__ scenes,
-                                                                     int n_scenes) {
+__global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat_batch(const __grid_constant__ BatchScenes b, int n_scenes) {
     extern __shared__ __align__(16) uint8_t s_dyn[];
-    __shared__ DispConst s_dc[kMaxBatchScenes];
     __shared__ uint32_t s_unit0[kMaxBatchScenes + 1];   // first unit of each scene
     __shared__ uint32_t s_n[kMaxBatchScenes];           // work points (0 after an overflow)
-    constexpr uint32_t unit = 2u * UnitPairs<S>::P;
+    constexpr int P = unit_pairs(S);
+    constexpr uint32_t unit = 2u * P;
     for (int q = threadIdx.x; q < n_scenes; q += blockDim.x) {
-        s_dc[q] = scenes[q].dc;
-        const Counters* ct = scenes[q].ctr;
+        const Counters* ct = b.s[q].ctr;
         s_n[q] = ct->overflow ? 0u : ct->n_work;
     }
     __syncthreads();
@@ -395,8 +401,8 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat_batch(const Splat
         s_unit0[n_scenes] = u;
     }
     __syncthreads();
-    const ManyScenes src{scenes, n_scenes, s_dc, s_unit0, s_n};
-    splat_units<S>(src, s_unit0[n_scenes], reinterpret_cast<SplatWarpSmem<S>*>(s_dyn)[threadIdx.x >> 5]);
+    const ManyScenes src{b, s_unit0, s_n};
+    splat_units<S>(src, s_unit0[n_scenes], reinterpret_cast<SplatWarpSmem<S, P>*>(s_dyn)[threadIdx.x >> 5]);
 }
 
 // Eq. 8's interpolation weight for one view pixel whose depth test kept the
@@ -600,7 +606,7 @@ __global__ void __launch_bounds__(256) k_resolve_pbr(FrameArgs a) {
 // with 8 view slots, which opts in once).
 template <int S>
 cudaError_t splat_one(const FrameArgs& a, int grid, cudaStream_t s) {
-    const size_t bytes = kSplatWarps * sizeof(SplatWarpSmem<S>);
+    const size_t bytes = kSplatWarps * sizeof(SplatWarpSmem<S, unit_pairs(S)>);
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_splat<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
     if (attr != cudaSuccess) return attr;
@@ -608,8 +614,8 @@ cudaError_t splat_one(const FrameArgs& a, int grid, cudaStream_t s) {
 }
 
 template <int S>
-cudaError_t splat_batch(const SplatScene* scenes, int n_scenes, int grid, cudaStream_t s) {
-    const size_t bytes = kSplatWarps * sizeof(SplatWarpSmem<S>);
+cudaError_t splat_batch(const BatchScenes& scenes, int n_scenes, int grid, cudaStream_t s) {
+    const size_t bytes = kSplatWarps * sizeof(SplatWarpSmem<S, unit_pairs(S)>);
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_splat_batch<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
     if (attr != cudaSuccess) return attr;
@@ -634,7 +640,7 @@ cudaError_t launch_splat(const FrameArgs& a, cudaStream_t s) {
     return splat_one<8>(a, grid, s);
 }
 
-cudaError_t launch_splat_batch(const SplatScene* scenes, int n_scenes, int slots, int grid_per_sm, int sm_count,
+cudaError_t launch_splat_batch(const BatchScenes& scenes, int n_scenes, int slots, int grid_per_sm, int sm_count,
                                cudaStream_t s) {
     if (n_scenes < 1 || n_scenes > kMaxBatchScenes || grid_per_sm < 1) return cudaErrorInvalidValue;
     const int grid = sm_count * grid_per_sm;
