@@ -305,8 +305,10 @@ lfdpr_status lfdpr_set_splat_lane_limit(lfdpr_display *disp, uint32_t limit);
  * band. With band = b > 0 and fewer than the rendered views, each frame
  * clears, splats and resolves views [0, b), then [b, 2b), ..., so that a
  * band's key buffers (8 B per pixel) can stay resident in L2 while they are
- * hit, when all the views' keys would not fit; results are identical. 0 (the
- * default) treats all views as one band. Errors: EINVAL (null display,
+ * hit, when all the views' keys would not fit; results are identical. With
+ * band >= the rendered views they form one band. 0 (the default) leaves the
+ * choice to the library: one band, or equal bands of at most 64 views where
+ * more than 64 views' keys exceed 350 MB. Errors: EINVAL (null display,
  * band < 0).
  */
 lfdpr_status lfdpr_set_view_band(lfdpr_display *disp, int32_t band);
