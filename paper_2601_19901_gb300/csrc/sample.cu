@@ -9,9 +9,9 @@
 //            total point count, overflow flag.
 //   k_emit   one thread per triangle: warp-shuffle block scan of the counts
 //            plus the block offset gives each triangle's first point id; the
-//            column summary (or, for a wider triangle, the column walk again)
-//            writes (triangle, cell) for each of its points (a warp per
-//            triangle of more than kEmitBig points).
+//            column summary writes (triangle, cell) for each of its points; a
+//            block's triangles of more columns or many points are emitted by
+//            the block together.
 //   k_fetch  one thread per point: texture coordinate of the cell centre and
 //            two trilinear fetches at LOD_min and LOD_max (Eq. 6-7); then the
 //            point's splat record (its cell projected into the views) and, if
@@ -122,16 +122,18 @@ struct ColumnWalk {
             }
         }
     }
-    __device__ __forceinline__ ColumnWalk(const float U_[3], const float V_[3], float su_, float sv_, float umax_)
+    // A walk from column `from` on.
+    __device__ __forceinline__ ColumnWalk(const float U_[3], const float V_[3], float su_, float sv_, float umax_,
+                                          int from = 0)
         : su(su_), sv(sv_), umax(umax_) {
 #pragma unroll
         for (int k = 0; k < 3; k++) {
             U[k] = U_[k];
             V[k] = V_[k];
         }
-        crossings(float(0) * su, lo_b, hi_b);
+        crossings(fminf(float(from) * su, umax), lo_b, hi_b);
     }
-    // column i: call for i = 0, 1, 2, ... in turn
+    // column i: call for i = from, from + 1, ... in turn
     __device__ __forceinline__ int rows(int i, int* j0, int* j1) {
         const float a = float(i) * su;
         const float b = fminf(float(i + 1) * su, umax);
@@ -512,101 +514,193 @@ __global__ void __launch_bounds__(1024) k_scan(FrameArgs a) {
     }
 }
 
-// The n points of triangle t from point id p on, in (column, row) order: a
-// single thread (lanes = 1) or a warp's lanes side by side in each column.
-__device__ __forceinline__ void emit_points(const FrameArgs& a, uint32_t t, uint32_t p, uint32_t n, int lane,
-                                            int lanes) {
-    if (a.colsum) {
-        // the columns k_setup found, without walking them again; the words
-        // past the last column are not written, and are not read: the
-        // columns before them hold all n points
-        const uint4 cs = a.colsum[t];
-        if (cs.x != kColSumWalk) {
-            const uint32_t w[4] = {cs.x, cs.y, cs.z, cs.w};
-            const uint32_t end = p + n;
+// The part of a triangle's record that its column walk needs.
+struct TriWalk {
+    float U[3], V[3];
+    float su, sv, umax;
+    __device__ explicit TriWalk(const TriRec* rp) {
+        TriRec r;
+        r.q[0].w = rp->q[0].w;
+        r.q[1].w = rp->q[1].w;
+        r.q[2].w = rp->q[2].w;
+        r.q[3].w = rp->q[3].w;
+        r.q[4] = rp->q[4];
+        shifted_uv(r, U, V);
+        su = r.q[0].w;
+        sv = r.q[1].w;
+        umax = rp->q[5].w;
+    }
+    __device__ int columns() const { return int(ceilf(__fdiv_rn(umax, su))); }
+    __device__ ColumnWalk from(int i) const { return ColumnWalk(U, V, su, sv, umax, i); }
+};
+
+// Inclusive scan of v over the block (kSetupThreads threads); s_warp: one value
+// a warp, free again after the next barrier. The block's total is s_warp's last.
+template <typename T>
+__device__ __forceinline__ T block_scan(T v, T* s_warp) {
+    constexpr int kWarps = kSetupThreads / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const T n = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += n;
+    }
+    if (lane == 31) s_warp[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        T w = lane < kWarps ? s_warp[lane] : T(0);
+#pragma unroll
+        for (int o = 1; o < kWarps; o <<= 1) {
+            const T n = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += n;
+        }
+        if (lane < kWarps) s_warp[lane] = w;
+    }
+    __syncthreads();
+    return warp > 0 ? v + s_warp[warp - 1] : v;
+}
+
+// The last of the block's kSetupThreads ascending numbers that is at most k
+// (the first is 0).
+__device__ __forceinline__ int last_at_most(const uint32_t* s_num, uint32_t k) {
+    int own = 0;
+#pragma unroll
+    for (int o = kSetupThreads / 2; o > 0; o >>= 1)
+        if (s_num[own + o] <= k) own += o;
+    return own;
+}
+
+// Block-level exclusive scan of the counts, plus the block's offset: each
+// triangle's first point id. Then emit its points in (column, row) order.
+//
+// A triangle of up to own_max points is emitted by its thread, from the columns
+// that k_setup kept or, of more than four columns, by walking them. The others
+// are the block's together: their columns are numbered in one sequence, of which
+// a thread takes one column at a time (its first row and row count from the
+// summary, or from the two borders), and the points of 256 columns in another,
+// of which a thread takes every 256th, finding its column by a search; so a
+// block's time follows its points, however they are spread over triangles and
+// columns, and its stores are contiguous.
+//
+// Meshes whose 256-triangle blocks do not fill the SMs spread each over `split`
+// blocks (each scans all 256 counts and emits its share of the triangles).
+// Bound by the dependent chain of a block's largest triangle while one thread or
+// one warp emits it; shared out, by the searches and stores of its points.
+// Measured on twelve meshes of 61 k to 1.2 M points (24 to 96 views): 608 us
+// before in sum (a thread a triangle, a lane a column above 128 points), 293 us
+// now; 5.4 M points on 10 k triangles 221 -> 40 us; a mesh of 871 k triangles of
+// a few points each 31 us both. With own_max 64 for unsplit and 48 for split
+// blocks instead of 128 and 24: 376 us.
+__global__ void __launch_bounds__(kSetupThreads) k_emit(FrameArgs a, uint32_t split, uint32_t own_max) {
+    wait_previous_kernel();
+    allow_next_kernel();
+    __shared__ uint32_t s_sum[kSetupThreads / 32];
+    __shared__ unsigned long long s_sum2[kSetupThreads / 32];
+    __shared__ uint32_t s_col0[kSetupThreads];    // first shared column of each triangle
+    __shared__ uint32_t s_skip[kSetupThreads];    // first point id less the shared points before it
+    __shared__ uint32_t s_num[kSetupThreads], s_id[kSetupThreads], s_tri[kSetupThreads], s_cell[kSetupThreads];
+    const uint32_t blk = blockIdx.x / split, part = blockIdx.x - blk * split, width = kSetupThreads / split;
+    const uint32_t t = blk * kSetupThreads + threadIdx.x;
+    const uint32_t cnt = t < a.n_tris ? a.counts[t] : 0u;
+    const uint32_t first = block_scan(cnt, s_sum) - cnt + a.block_sums[blk];
+    const bool mine = t < a.n_tris && threadIdx.x / width == part;
+    if (mine) a.offsets[t] = first;
+    if (a.ctr->overflow != 0u) return;
+    uint4 cs = make_uint4(kColSumWalk, 0u, 0u, 0u);
+    const bool live = mine && cnt > 0u;
+    if (live && a.colsum) cs = a.colsum[t];
+    const bool walk = cs.x == kColSumWalk, together = live && cnt > own_max;
+    const uint32_t w[4] = {cs.x, cs.y, cs.z, cs.w};
+    if (live && !together) {
+        uint32_t p = first;
+        auto emit_column = [&](int i, uint32_t j0, uint32_t rows) {
+            for (uint32_t r = 0; r < rows; r++) {
+                const uint32_t q = p + r;
+                if (LFDPR_IN_BOUNDS(q, a.max_points, 4))
+                    *reinterpret_cast<uint2*>(a.points + q) = make_uint2(t, uint32_t(i) | ((j0 + r) << 16));
+            }
+            p += rows;
+        };
+        if (walk) {
+            TriWalk tri(a.rec + t);
+            ColumnWalk column = tri.from(0);
+            const int cols = tri.columns();
+            for (int i = 0; i < cols; i++) {
+                int j0, j1;
+                const int rows = column.rows(i, &j0, &j1);
+                emit_column(i, uint32_t(j0), uint32_t(rows));
+            }
+        } else {
+            // the columns k_setup found; the words past the last column are not
+            // written, and are not read: the columns before them hold all the points
+            const uint32_t end = first + cnt;
 #pragma unroll
             for (int i = 0; i < 4; i++) {
                 if (p == end) break;
-                const uint32_t j0 = w[i] & 0xffffu, rows = w[i] >> 16;
-                for (uint32_t r = uint32_t(lane); r < rows; r += uint32_t(lanes)) {
-                    const uint32_t q = p + r;
-                    if (LFDPR_IN_BOUNDS(q, a.max_points, 4))
-                        *reinterpret_cast<uint2*>(a.points + q) = make_uint2(t, uint32_t(i) | ((j0 + r) << 16));
-                }
-                p += rows;
+                emit_column(i, w[i] & 0xffffu, w[i] >> 16);
             }
-            return;
         }
     }
-    const TriRec* rp = a.rec + t;
-    TriRec r;
-    r.q[0] = rp->q[0]; r.q[1] = rp->q[1]; r.q[2] = rp->q[2]; r.q[3] = rp->q[3];
-    r.q[4] = rp->q[4]; r.q[5] = rp->q[5];
-    float U[3], V[3];
-    shifted_uv(r, U, V);
-    const float su = r.q[0].w, sv = r.q[1].w, umax = r.q[5].w;
-    const int cols = int(ceilf(__fdiv_rn(umax, su)));
-    ColumnWalk walk(U, V, su, sv, umax);
-    for (int i = 0; i < cols; i++) {
-        int j0, j1;
-        walk.rows(i, &j0, &j1);
-        for (int j = j0 + lane; j < j1; j += lanes) {
-            const uint32_t q = p + uint32_t(j - j0);
-            if (LFDPR_IN_BOUNDS(q, a.max_points, 4))
-                *reinterpret_cast<uint2*>(a.points + q) = make_uint2(t, uint32_t(i) | (uint32_t(j) << 16));
-        }
-        p += uint32_t(j1 - j0);
-    }
-}
+    if (!__syncthreads_or(together)) return;
 
-// Block-level exclusive scan of the counts (warp shuffles), plus the block's
-// offset: each triangle's first point id. Then emit its points in (column,
-// row) order; the block's triangles of more than kEmitBig points are listed
-// in shared memory and emitted afterwards by the block's warps, a warp each,
-// so that one thread does not walk tens of thousands of points.
-__global__ void __launch_bounds__(kSetupThreads) k_emit(FrameArgs a) {
-    wait_previous_kernel();
-    allow_next_kernel();
-    __shared__ uint32_t s_warp[kSetupThreads / 32];
-    __shared__ uint32_t s_big[kSetupThreads], s_first[kSetupThreads];
-    __shared__ uint32_t s_nbig;
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t cnt = t < a.n_tris ? a.counts[t] : 0u;
-    uint32_t inc = cnt;
+    uint32_t cols = 0u;
+    if (together) {
+        if (walk) {
+            cols = uint32_t(TriWalk(a.rec + t).columns());
+        } else {
+            uint32_t n = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t n = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += n;
-    }
-    if (lane == 31) s_warp[warp] = inc;
-    if (threadIdx.x == 0) s_nbig = 0u;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t w = lane < kSetupThreads / 32 ? s_warp[lane] : 0u;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t n = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += n;
-        }
-        if (lane < kSetupThreads / 32) s_warp[lane] = w;
-    }
-    __syncthreads();
-    const bool overflow = a.ctr->overflow != 0u;
-    if (t < a.n_tris) {
-        const uint32_t first = a.block_sums[blockIdx.x] + (warp > 0 ? s_warp[warp - 1] : 0u) + inc - cnt;
-        a.offsets[t] = first;
-        if (cnt > kEmitBig && !overflow) {
-            const uint32_t b = atomicAdd(&s_nbig, 1u);
-            s_big[b] = t;
-            s_first[b] = first;
-        } else if (cnt > 0 && !overflow) {
-            emit_points(a, t, first, cnt, 0, 1);
+            for (int i = 0; i < 4; i++)
+                if (n != cnt) {
+                    n += w[i] >> 16;
+                    cols++;
+                }
         }
     }
+    // shared columns (high word) and points (low word) before each triangle's
+    const unsigned long long own = ((unsigned long long)cols << 32) | (together ? cnt : 0u);
+    const unsigned long long before = block_scan(own, s_sum2) - own;
+    s_col0[threadIdx.x] = uint32_t(before >> 32);
+    s_skip[threadIdx.x] = first - uint32_t(before);
+    const uint32_t n_cols = uint32_t(s_sum2[kSetupThreads / 32 - 1] >> 32);
     __syncthreads();
-    for (uint32_t b = uint32_t(warp); b < s_nbig; b += kSetupThreads / 32)
-        emit_points(a, s_big[b], s_first[b], a.counts[s_big[b]], lane, 32);
+    uint32_t done = 0;   // shared points of the columns before
+    for (uint32_t c0 = 0; c0 < n_cols; c0 += kSetupThreads) {
+        const uint32_t c = c0 + threadIdx.x;
+        uint32_t rows = 0, tri = 0, cell = 0;
+        if (c < n_cols) {
+            const uint32_t k = uint32_t(last_at_most(s_col0, c));
+            const int i = int(c - s_col0[k]);
+            tri = blk * kSetupThreads + k;
+            int j0, j1;
+            uint32_t word = kColSumWalk;
+            if (a.colsum) word = reinterpret_cast<const uint32_t*>(a.colsum + tri)[0];
+            if (word == kColSumWalk) {
+                ColumnWalk column = TriWalk(a.rec + tri).from(i);
+                rows = uint32_t(column.rows(i, &j0, &j1));
+            } else {
+                if (i > 0) word = reinterpret_cast<const uint32_t*>(a.colsum + tri)[i];
+                j0 = int(word & 0xffffu);
+                rows = word >> 16;
+            }
+            cell = uint32_t(i) | (uint32_t(j0) << 16);
+            s_id[threadIdx.x] = s_skip[k];
+        }
+        const uint32_t num = block_scan(rows, s_sum) - rows, total = s_sum[kSetupThreads / 32 - 1];
+        s_num[threadIdx.x] = num;
+        if (c < n_cols) s_id[threadIdx.x] += done + num;   // the column's first point id
+        s_tri[threadIdx.x] = tri;
+        s_cell[threadIdx.x] = cell;
+        __syncthreads();
+        for (uint32_t k = threadIdx.x; k < total; k += kSetupThreads) {
+            const int o = last_at_most(s_num, k);
+            const uint32_t r = k - s_num[o], q = s_id[o] + r;
+            if (LFDPR_IN_BOUNDS(q, a.max_points, 4))
+                *reinterpret_cast<uint2*>(a.points + q) = make_uint2(s_tri[o], s_cell[o] + (r << 16));
+        }
+        done += total;
+        __syncthreads();
+    }
 }
 
 // One mip level's bilinear sample at texture coordinates (fs, ft) in [0, 1):
@@ -1183,7 +1277,11 @@ cudaError_t launch_scan(const FrameArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_emit(const FrameArgs& a, cudaStream_t s) {
-    return launch_after_previous(k_emit, dim3(a.n_blocks), dim3(kSetupThreads), 0, s, a);
+    // the largest split (a power of two up to 8) that leaves an SM at most two blocks
+    uint32_t split = 1;
+    while (split < 8u && 2u * split * a.n_blocks <= 2u * uint32_t(a.sm_count)) split *= 2u;
+    return launch_after_previous(k_emit, dim3(a.n_blocks * split), dim3(kSetupThreads), 0, s, a, split,
+                                 split == 1u ? kEmitOwn : kEmitOwnFew);
 }
 
 cudaError_t launch_fetch_mat(const FrameArgs& a, cudaStream_t s) {
