@@ -112,6 +112,51 @@ struct ResolveRec {
     uint4 b;      // vpuv_max bits, tv_min RGBA8, tv_max RGBA8, roughness/metallic bytes (materials)
 };
 
+// Shading data of a point of a mesh of materials, made by the fetch so that the
+// resolve's pixels (two or more to a point) gather one sector instead of the normal-map
+// values, the triangle's id and, through it, five parts of its record: the unit
+// normal N, the unit tangent, the normal map's tv_min (its alpha byte replaced:
+// 1 where the bitangent is -(N x tangent)) and tv_max.
+struct MatRec {
+    float4 a;     // N, tangent x
+    uint4 b;      // tangent y and z bits, normal tv_min RGB | bitangent sign << 24, normal tv_max
+};
+
+// The 32 bytes at p (32-byte aligned, not written by the running kernel).
+__device__ __forceinline__ void load32(const void* p, float4& a, uint4& b) {
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+        : "l"(p));
+}
+__device__ __forceinline__ void load32(const void* p, float4& a, float4& b) {
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "l"(p));
+}
+__device__ __forceinline__ void store32(void* p, const float4& a, const uint4& b) {
+    asm volatile("st.global.v8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
+                 :: "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w), "l"(p)
+                 : "memory");
+}
+__device__ __forceinline__ void store32(void* p, const float4& a, const float4& b) {
+    asm volatile("st.global.v8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
+                 :: "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w), "l"(p)
+                 : "memory");
+}
+
+__device__ __forceinline__ float3 f3(float x, float y, float z) { return make_float3(x, y, z); }
+__device__ __forceinline__ float dot(const float3& a, const float3& b) {
+    return fmaf(a.x, b.x, fmaf(a.y, b.y, a.z * b.z));
+}
+// The shading runs in binary32 against a double-precision oracle with a
+// tolerance of one level of 255, so it uses the hardware's approximate
+// reciprocal square root and division (relative errors near 1e-7).
+__device__ __forceinline__ float3 normalized(const float3& v) {
+    const float l2 = dot(v, v);
+    const float r = l2 > 0.0f ? rsqrtf(l2) : 0.0f;
+    return l2 > 0.0f ? f3(v.x * r, v.y * r, v.z * r) : v;
+}
+
 // Physically based shading of a mesh of materials: one directional light
 // (unit direction toward the light, radiance) and an ambient term.
 struct Shading {
@@ -305,6 +350,7 @@ struct FrameArgs {
     uint32_t* near;                  // [max_points] points whose cell or triangle reaches within near_z of the eyes' plane
     ResolveRec* rrec;                // [max_points] per-point resolve data
     uint2* rmat;                     // [max_points] normal-map tv_min, tv_max (meshes of materials)
+    MatRec* mrec;                    // [max_points] shading data (meshes of materials)
     uint64_t* keys;
     uint8_t* views;
     Counters* ctr;

@@ -31,6 +31,7 @@ struct lfdpr_display {
     uint32_t* near = nullptr;     // points whose cell or triangle reaches within near_z of the eyes' plane
     lfdpr::ResolveRec* rrec = nullptr;
     uint2* rmat = nullptr;        // normal-map tv_min / tv_max per point (allocated with the first mesh of materials)
+    lfdpr::MatRec* mrec = nullptr; // shading data per point (allocated with it)
     uint64_t* keys = nullptr;
     uint8_t* views = nullptr;
     uint8_t* panel = nullptr;      // device scratch for host-memory panels

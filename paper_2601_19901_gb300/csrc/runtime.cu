@@ -134,6 +134,7 @@ FrameArgs frame_args(const lfdpr_display* disp, const lfdpr_mesh* mesh) {
     a.near = disp->near;
     a.rrec = disp->rrec;
     a.rmat = disp->rmat;
+    a.mrec = disp->mrec;
     a.keys = disp->keys;
     a.views = disp->views;
     a.ctr = disp->ctr;
@@ -245,6 +246,7 @@ void free_display(lfdpr_display* d) {
     dev_free(d->near);
     dev_free(d->rrec);
     dev_free(d->rmat);
+    dev_free(d->mrec);
     dev_free(d->keys);
     dev_free(d->views);
     dev_free(d->panel);
@@ -734,6 +736,10 @@ lfdpr_status lfdpr_upload_mesh_materials(lfdpr_display* disp, const float* xyz, 
     if (!disp->rmat) {
         const cudaError_t e = dev_malloc(&disp->rmat, sizeof(uint2) * (uint64_t)disp->max_points);
         if (e != cudaSuccess) return cuda_fail(e, "upload_mesh_materials: normal-map buffer");
+    }
+    if (!disp->mrec) {
+        const cudaError_t e = dev_malloc(&disp->mrec, sizeof(MatRec) * (uint64_t)disp->max_points);
+        if (e != cudaSuccess) return cuda_fail(e, "upload_mesh_materials: shading buffer");
     }
     lfdpr_mesh* m = nullptr;
     // the material ids are checked against n_mat like texture ids

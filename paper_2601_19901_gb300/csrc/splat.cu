@@ -434,7 +434,8 @@ __device__ __forceinline__ uint32_t resolve_pixel(float Ex, const float4& ra, co
 
 // kResolvePix view pixels per thread, 256 apart (grid: pixel blocks x
 // views): every key is loaded, then every winner's record, so each thread
-// keeps that many dependent gathers in flight.
+// keeps that many dependent gathers in flight. A record is one 32-byte load
+// (48 views of 420x560: 45 us; as two of 16 bytes 47).
 constexpr int kResolvePix = 2;
 __global__ void __launch_bounds__(256) k_resolve(FrameArgs a) {
     wait_previous_kernel();
@@ -456,9 +457,7 @@ __global__ void __launch_bounds__(256) k_resolve(FrameArgs a) {
     for (int k = 0; k < kResolvePix; k++) {
         if (key[k] != ~0ull && !LFDPR_IN_BOUNDS(uint32_t(key[k]), a.max_points, 12)) key[k] = ~0ull;
         if (key[k] != ~0ull) {
-            const ResolveRec* rp = a.rrec + uint32_t(key[k]);
-            ra[k] = __ldg(&rp->a);
-            rb[k] = __ldg(&rp->b);
+            load32(a.rrec + uint32_t(key[k]), ra[k], rb[k]);
         }
     }
     const float Ex = __ldg(a.ex + v);
@@ -473,19 +472,6 @@ __global__ void __launch_bounds__(256) k_resolve(FrameArgs a) {
 // ---------------------------------------------------------------------------
 // Physically based resolve of a mesh of materials
 // ---------------------------------------------------------------------------
-
-__device__ __forceinline__ float3 f3(float x, float y, float z) { return make_float3(x, y, z); }
-__device__ __forceinline__ float dot(const float3& a, const float3& b) {
-    return fmaf(a.x, b.x, fmaf(a.y, b.y, a.z * b.z));
-}
-// The shading runs in binary32 against a double-precision oracle with a
-// tolerance of one level of 255, so it uses the hardware's approximate
-// reciprocal square root and division (relative errors near 1e-7).
-__device__ __forceinline__ float3 normalized(const float3& v) {
-    const float l2 = dot(v, v);
-    const float r = l2 > 0.0f ? rsqrtf(l2) : 0.0f;
-    return l2 > 0.0f ? f3(v.x * r, v.y * r, v.z * r) : v;
-}
 
 // Outgoing linear RGB of one surface sample (unit n, v, l): metallic-roughness
 // microfacet BRDF, GGX distribution D = a^2 / (pi ((n.h)^2 (a^2 - 1) + 1)^2),
@@ -524,11 +510,12 @@ __device__ __forceinline__ float3 pbr_shade(const float3& albedo, float rough, f
 // interpolated by Eq. 9 (unrounded); the surface point where the pixel
 // centre's ray meets the triangle (the key's t: P = E + t (F - E)); the
 // shading normal = the normal map's (2 c / 255 - 1) vector in the triangle's
-// frame (tangent and bitangent = world directions of increasing s and t, from
-// the inverse of the record's texture map over u-hat, v-hat; tangent made
-// orthogonal to N, bitangent = N x T signed by the t direction), flipped when
+// frame (of k_fetch_mat, with the normal map's values in the point's record), flipped when
 // the triangle faces away from the eye; RGB = pbr_shade clamped, times 255,
-// rounded half to even, alpha 255.
+// rounded half to even, alpha 255. Bound by its gathers (a warp's 32 points are
+// 32 places): two sectors a pixel, each by one 32-byte load. 48 views of 420x560:
+// 158 us with the frame formed from the triangle's record by every pixel (nine
+// loads in six sectors), 107 now, for 10 us more in k_fetch_mat.
 __global__ void __launch_bounds__(256) k_resolve_pbr(FrameArgs a) {
     wait_previous_kernel();
     allow_next_kernel();
@@ -545,10 +532,11 @@ __global__ void __launch_bounds__(256) k_resolve_pbr(FrameArgs a) {
         const uint32_t p = uint32_t(key);
         const float t = __uint_as_float(uint32_t(key >> 32));
         const float Ex = __ldg(a.ex + v);
-        const ResolveRec* rp = a.rrec + p;
-        const float4 ra = __ldg(&rp->a);
-        const uint4 rb = __ldg(&rp->b);
-        const uint2 nm = __ldg(a.rmat + p);
+        float4 ra, ma;
+        uint4 rb, mb;
+        load32(a.rrec + p, ra, rb);
+        load32(a.mrec + p, ma, mb);
+        const uint2 nm = make_uint2(mb.z, mb.w);
         const float w = eq8_weight(Ex, ra, rb);
         auto lerp8 = [w](uint32_t lo, uint32_t hi, int ch) {
             const float a0 = float((lo >> (8 * ch)) & 255u), b0 = float((hi >> (8 * ch)) & 255u);
@@ -567,27 +555,10 @@ __global__ void __launch_bounds__(256) k_resolve_pbr(FrameArgs a) {
         const float Fx = fmaf(float(x) + 0.5f, c.pw, c.x0), Fy = fmaf(float(y) + 0.5f, -c.ph, c.y0);
         const float3 P = f3(fmaf(t, Fx - Ex, Ex), t * Fy, fmaf(-t, c.D, c.D));
         const float3 V = normalized(f3(Ex - P.x, -P.y, c.D - P.z));
-        // the triangle's shading frame
-        const TriRec* r = a.rec + __ldg(&a.points[p].x);
-        const float4 q1 = __ldg(&r->q[1]), q2 = __ldg(&r->q[2]), q3 = __ldg(&r->q[3]);
-        const float4 q6 = __ldg(&r->q[6]), q7 = __ldg(&r->q[7]);
-        const float3 N = f3(q3.x, q3.y, q3.z);
-        const float gsu = q6.y, gsv = q6.z, gtu = q7.x, gtv = q7.y;
-        const float det = fmaf(gsu, gtv, -(gsv * gtu));
-        float dus = 1.0f, dvs = 0.0f, dut = 0.0f, dvt = 1.0f;
-        if (det != 0.0f) {
-            const float id = 1.0f / det;
-            dus = gtv * id;
-            dvs = -gtu * id;
-            dut = -gsv * id;
-            dvt = gsu * id;
-        }
-        const float3 ts = f3(fmaf(q1.x, dus, q2.x * dvs), fmaf(q1.y, dus, q2.y * dvs), fmaf(q1.z, dus, q2.z * dvs));
-        const float3 tt = f3(fmaf(q1.x, dut, q2.x * dvt), fmaf(q1.y, dut, q2.y * dvt), fmaf(q1.z, dut, q2.z * dvt));
-        const float dn = dot(ts, N);
-        const float3 Tg = normalized(f3(fmaf(-N.x, dn, ts.x), fmaf(-N.y, dn, ts.y), fmaf(-N.z, dn, ts.z)));
+        // the shading frame: N, the tangent and their cross product by its sign
+        const float3 N = f3(ma.x, ma.y, ma.z), Tg = f3(ma.w, __uint_as_float(mb.x), __uint_as_float(mb.y));
         float3 Bt = f3(fmaf(N.y, Tg.z, -(N.z * Tg.y)), fmaf(N.z, Tg.x, -(N.x * Tg.z)), fmaf(N.x, Tg.y, -(N.y * Tg.x)));
-        if (dot(Bt, tt) < 0.0f) Bt = f3(-Bt.x, -Bt.y, -Bt.z);
+        if (mb.z >> 24) Bt = f3(-Bt.x, -Bt.y, -Bt.z);
         float3 n = f3(fmaf(nt.x, Tg.x, fmaf(nt.y, Bt.x, nt.z * N.x)), fmaf(nt.x, Tg.y, fmaf(nt.y, Bt.y, nt.z * N.y)),
                       fmaf(nt.x, Tg.z, fmaf(nt.y, Bt.z, nt.z * N.z)));
         if (dot(n, n) == 0.0f) n = N;
