@@ -55,20 +55,37 @@ __device__ __forceinline__ bool seen_by(const DispConst& c, float e, const float
     return !(out_l || out_r);
 }
 
-// The eye whose x is nearest `target` (eyes ascending in x): binary search
-// for the first eye at or beyond it, then the nearer of it and the one
-// before (the earlier on a tie). Only a starting guess for the searches
-// below: culling and the closest / farthest eye do not depend on it.
-__device__ __forceinline__ int nearest_eye(const float* __restrict__ ex, int nr, float target) {
-    int lo = 0, hi = nr;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (ex[mid] < target) lo = mid + 1;
-        else hi = mid;
+// A view whose eye x is near `target` (eyes ascending in x): the nearest one of
+// evenly spaced eyes. Only a starting guess for the searches below: culling and
+// the closest / farthest eye do not depend on it. (A NaN, of a zero span or of
+// the target, gives view 0.) A binary search for it, twice a triangle, was a
+// chain of twelve shared-memory loads: 101 -> 97 us of set-up on 10^6 triangles.
+__device__ __forceinline__ int near_eye(const float* __restrict__ ex, int nr, float target) {
+    const float x0 = ex[0], last = float(nr - 1);
+    const float i = __fdividef((target - x0) * last, ex[nr - 1] - x0);
+    return int(fminf(fmaxf(i, 0.0f), last) + 0.5f);
+}
+
+// Whether the triangle is surely outside the left plane of every view, or the
+// right one of every view. A vertex's signed distances l and r of seen_by are
+// linear in the eye's x and computed to within 6 u m (u = 2^-24, m the sum of
+// their terms' magnitudes, at its largest over the eyes): below -2^-20 m at both
+// end eyes, they are negative at every eye between, as computed. A culled
+// triangle mostly ends here instead of asking every view in turn (10^6
+// triangles, 7 % culled: set-up 97 -> 87 us with 48 views, 109 -> 88 with 96).
+__device__ __forceinline__ bool outside_all(const DispConst& c, float e0, float e1, const float P[3][3]) {
+    const float E = fmaxf(fabsf(e0), fabsf(e1));
+    bool out_l = true, out_r = true;
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const float dep = c.D - P[k][2];
+        const float m = 0x1p-20f * fmaf(fabsf(P[k][0]) + E, c.D, (c.fw2 + E) * fabsf(dep));
+        const float l0 = fmaf(P[k][0] - e0, c.D, (c.fw2 + e0) * dep), l1 = fmaf(P[k][0] - e1, c.D, (c.fw2 + e1) * dep);
+        const float r0 = fmaf(e0 - P[k][0], c.D, (c.fw2 - e0) * dep), r1 = fmaf(e1 - P[k][0], c.D, (c.fw2 - e1) * dep);
+        out_l &= fmaxf(l0, l1) < -m;
+        out_r &= fmaxf(r0, r1) < -m;
     }
-    if (lo == 0) return 0;
-    if (lo == nr) return nr - 1;
-    return fabsf(ex[lo] - target) < fabsf(ex[lo - 1] - target) ? lo : lo - 1;
+    return out_l || out_r;
 }
 
 __device__ bool culled(const DispConst& c, const float* __restrict__ ex, const float P[3][3]) {
@@ -90,8 +107,9 @@ __device__ bool culled(const DispConst& c, const float* __restrict__ ex, const f
     const float cx = (P[0][0] + P[1][0] + P[2][0]) * (1.0f / 3.0f);
     const float cz = (P[0][2] + P[1][2] + P[2][2]) * (1.0f / 3.0f);
     const float target = fabsf(cz) > 1e-6f ? __fdividef(cx * c.D, cz) : 0.0f;
-    const int vb = nearest_eye(ex, c.nr, target);
+    const int vb = near_eye(ex, c.nr, target);
     if (seen_by(c, ex[vb], P)) return false;
+    if (outside_all(c, ex[0], ex[c.nr - 1], P)) return true;
     for (int v = 0; v < c.nr; v++)
         if (seen_by(c, ex[v], P)) return false;
     return true;
@@ -281,7 +299,7 @@ __device__ SetupOut setup_triangle(const FrameArgs& a, const float* ex, uint32_t
     const float S = fmaxf(fabsf(x_first - P[0][0]), fabsf(x_last - P[0][0])) * 1.0001f + fabsf(qy) + fabsf(qz);
     const float SL = S + ((fabsf(a1) + fabsf(b1)) + (fabsf(a2) + fabsf(b2)));
     const float E2 = 0x1p-17f * (SL * SL);   // 2E
-    const int g = nearest_eye(ex, nr, (P[0][0] + P[1][0] + P[2][0]) * (1.0f / 3.0f));
+    const int g = near_eye(ex, nr, (P[0][0] + P[1][0] + P[2][0]) * (1.0f / 3.0f));
     const float fg = exact_d2(g);
     float d2min = fg, d2max = fg;
     int hi = g, lo = g;
