@@ -27,10 +27,9 @@ struct lfdpr_batch {
     float* d_models = nullptr;       // [n][12] model rows read by k_setup
     float* h_models = nullptr;       // pinned staging of the same
     cudaEvent_t staged = nullptr;    // the last copy out of h_models has run
-    BatchScenes scenes{};            // [n] for the batched splat
     cudaStream_t cap = nullptr;      // the stream the graph is captured on
     std::vector<cudaStream_t> br;    // branch streams
-    std::vector<cudaEvent_t> ev;     // fork, fork2, joins
+    std::vector<cudaEvent_t> ev;     // fork, joins
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     bool stale = true;               // capture again before the next replay
@@ -96,7 +95,7 @@ void free_batch(lfdpr_batch* b) {
 lfdpr_status record_batch(lfdpr_batch* b) {
     const int K = b->cfg.branches;
     cudaStream_t s = b->cap;
-    cudaEvent_t fork = b->ev[0], fork2 = b->ev[1];
+    cudaEvent_t fork = b->ev[0];   // then the branches' joins
     // timing events as event-record nodes of the graph (a plain record during
     // capture would only join streams)
     CK(cudaEventRecordWithFlags(b->tev[0], s, cudaEventRecordExternal), "batch: start event");
@@ -107,17 +106,7 @@ lfdpr_status record_batch(lfdpr_batch* b) {
         a.model_dev = b->d_models + 12 * i;
         const lfdpr_status st = record_frame_front(b->disp[i], b->mesh[i], a, b->br[i % K], false);
         if (st != LFDPR_OK) return st;
-    }
-    for (int j = 0; j < K; j++) {
-        CK(cudaEventRecord(b->ev[2 + j], b->br[j]), "batch: join");
-        CK(cudaStreamWaitEvent(s, b->ev[2 + j], 0), "batch: join wait");
-    }
-    CK(launch_splat_batch(b->scenes, b->n, b->cfg.splat_slots, b->cfg.splat_blocks_per_sm, b->sm_count, s),
-       "launch k_splat_batch");
-    CK(cudaEventRecord(fork2, s), "batch: fork");
-    for (int j = 0; j < K; j++) CK(cudaStreamWaitEvent(b->br[j], fork2, 0), "batch: branch wait");
-    for (int i = 0; i < b->n; i++) {
-        const FrameArgs a = frame_args(b->disp[i], b->mesh[i]);
+        CK(launch_splat(a, b->br[i % K], b->cfg.splat_blocks_per_sm, b->cfg.splat_slots), "launch k_splat");
         CK(launch_resolve(a, b->br[i % K]), "launch k_resolve");
         lfdpr_display* d = b->disp[i];
         if ((d->desc.recon == 2 || d->desc.recon == 3) && d->n_samples == 0)
@@ -127,8 +116,8 @@ lfdpr_status record_batch(lfdpr_batch* b) {
         CK(cudaEventRecordWithFlags(b->tev[1 + i], b->br[i % K], cudaEventRecordExternal), "batch: scene event");
     }
     for (int j = 0; j < K; j++) {
-        CK(cudaEventRecord(b->ev[2 + K + j], b->br[j]), "batch: join");
-        CK(cudaStreamWaitEvent(s, b->ev[2 + K + j], 0), "batch: join wait");
+        CK(cudaEventRecord(b->ev[1 + j], b->br[j]), "batch: join");
+        CK(cudaStreamWaitEvent(s, b->ev[1 + j], 0), "batch: join wait");
     }
     return LFDPR_OK;
 }
@@ -139,7 +128,7 @@ lfdpr_status capture(lfdpr_batch* b) {
     if ((int)b->br.size() != K) {
         drop_branches(b);
         b->br.resize(K, nullptr);
-        b->ev.resize(2 + 2 * K, nullptr);
+        b->ev.resize(1 + K, nullptr);
         for (auto& s : b->br) CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking), "batch: stream");
         for (auto& e : b->ev) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "batch: event");
     }
@@ -205,15 +194,6 @@ lfdpr_status lfdpr_create_batch(lfdpr_display* const* displays, lfdpr_mesh* cons
     b->cfg.branches = std::min(4, n);
     b->cfg.splat_blocks_per_sm = 16;
     b->cfg.splat_slots = fewest_slots(max_views);
-    for (int i = 0; i < n; i++) {
-        SplatScene& sc = b->scenes.s[i];
-        sc.dc = displays[i]->dc;
-        sc.ex = displays[i]->d_ex;
-        sc.ctr = displays[i]->ctr;
-        sc.work = displays[i]->work;
-        sc.rec = meshes[i]->rec;
-        sc.keys = displays[i]->keys;
-    }
     cudaError_t e;
     if ((e = dev_malloc(&b->d_models, sizeof(float) * 12 * n)) != cudaSuccess ||
         (e = host_malloc(&b->h_models, sizeof(float) * 12 * n)) != cudaSuccess ||
@@ -283,10 +263,9 @@ lfdpr_status lfdpr_render_batch(lfdpr_batch* b, const float* models, void* strea
     for (int i = 0; i < b->n; i++) {
         b->disp[i]->ev_frame = b->disp[i]->ev_interleave = false;
         // set-up, scan, emission, fetch, near-limit records (and the
-        // materials' fetch), resolve, (view mips,) interleave
-        b->disp[i]->launches += (b->mesh[i]->n_tris ? (b->mesh[i]->mat_tex ? 8 : 7) : 2) + (b->disp[i]->ss_level > 0);
+        // materials' fetch), splat, resolve, (view mips,) interleave
+        b->disp[i]->launches += (b->mesh[i]->n_tris ? (b->mesh[i]->mat_tex ? 9 : 8) : 3) + (b->disp[i]->ss_level > 0);
     }
-    b->disp[0]->launches += 1;
     return LFDPR_OK;
 }
 

@@ -406,29 +406,10 @@ cudaError_t launch_emit(const FrameArgs& a, cudaStream_t s);
 cudaError_t launch_fetch(const FrameArgs& a, cudaStream_t s);
 cudaError_t launch_fetch_mat(const FrameArgs& a, cudaStream_t s);   // meshes of materials, after launch_fetch
 cudaError_t launch_near_work(const FrameArgs& a, cudaStream_t s);   // after launch_fetch
-cudaError_t launch_splat(const FrameArgs& a, cudaStream_t s);
-
-// One scene of a batched splat: its display constants and the buffers the
-// splat reads and writes.
-struct SplatScene {
-    DispConst dc;
-    const float* ex;
-    Counters* ctr;
-    const WorkRec* work;
-    const TriRec* rec;
-    uint64_t* keys;
-};
+// blocks_per_sm blocks per SM, at most max_slots views per lane (1, 2, 3, 4, 6 or 8).
+cudaError_t launch_splat(const FrameArgs& a, cudaStream_t s, int blocks_per_sm = 16, int max_slots = 8);
 constexpr int kMaxBatchScenes = 64;
 constexpr int kMaxBatchViews = 4096;   // rendered views summed over a batch
-// A batch's scenes as one kernel parameter.
-struct BatchScenes {
-    SplatScene s[kMaxBatchScenes];
-};
-static_assert(sizeof(BatchScenes) < 32000, "kernel parameter limit");
-// Splat every scene of a batch in one persistent launch: grid_per_sm blocks
-// per SM, slots view slots per lane (1, 2, 3, 4, 6 or 8).
-cudaError_t launch_splat_batch(const BatchScenes& scenes, int n_scenes, int slots, int grid_per_sm, int sm_count,
-                               cudaStream_t s);
 cudaError_t launch_resolve(const FrameArgs& a, cudaStream_t s);
 // pos [nr] (views on the display-view axis) and samples [n_samples][3] are
 // read only for Gaussian reconstruction (recon 2, 3).

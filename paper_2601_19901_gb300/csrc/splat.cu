@@ -97,11 +97,18 @@ __device__ __forceinline__ uint32_t div_floor(uint32_t r, uint32_t n) {
     return r / n;
 }
 
-// Units of 2P points per warp: pairs per unit for S view slots per lane. Four
-// points share the unit's scan and fill its passes better than two: 96 views
-// (S = 6) 0.557 -> 0.471 ms. With S = 8 their segments would leave an SM three
-// blocks.
-__host__ __device__ constexpr int unit_pairs(int S) { return S <= 6 ? 2 : 1; }
+// Units of 2P points per warp: pairs per unit for S view slots per lane. More
+// points share the unit's scan and fill its passes better; more segments take
+// more shared memory and registers, and a small mesh has fewer units to spread.
+// Splat of 10^6 triangles (200 instances), P = 1 for S = 6, else 2, against
+// these: 8 views (S = 1) 172 -> 131 us, 24 (S = 2) 220 -> 190, 48 (S = 3)
+// 292 -> 283, 96 (S = 6) 557 -> 471. P = 5 for S = 1 gave 124 but a frame of
+// 2,048 triangles 1 us more; P = 5 for S = 2 223; P = 4 for S = 3 286; P = 3 for
+// S = 4 350 against 353 but slower small frames. With S = 8 two pairs would
+// leave an SM three blocks.
+__host__ __device__ constexpr int unit_pairs(int S) {
+    return S <= 2 ? 4 : S == 3 ? 3 : S <= 6 ? 2 : 1;
+}
 
 // Per-warp shared memory of the pooled splat: the unit's non-empty (point,
 // view) segments in candidate order (first candidate number,
@@ -113,58 +120,6 @@ struct SplatWarpSmem {
     static constexpr int kSegs = 32 * S * P;
     uint4 seg[kSegs];
     float4 pt[2 * P][6];
-};
-
-// Where the splat's units come from: one scene (its constants in the kernel's
-// parameters), or every scene of a batch (an array of them there; the units of
-// all scenes form one index range, scene by scene).
-struct OneScene {
-    static constexpr bool kMany = false;
-    const FrameArgs& a;
-    uint32_t n;       // work points
-    uint32_t ex_s;    // shared-memory address of the eye positions
-    __device__ __forceinline__ int scene(uint32_t, int) const { return 0; }
-    __device__ __forceinline__ uint32_t first_unit(int) const { return 0u; }
-    __device__ __forceinline__ const DispConst& dc(int) const { return a.dc; }
-    __device__ __forceinline__ float eye(int, int v) const { return eye_x(ex_s, v); }
-    __device__ __forceinline__ uint32_t points(int) const { return n; }
-    __device__ __forceinline__ const WorkRec* work(int) const { return a.work; }
-    __device__ __forceinline__ const TriRec* rec(int) const { return a.rec; }
-    __device__ __forceinline__ unsigned long long* keys(int) const {
-        return reinterpret_cast<unsigned long long*>(a.keys);
-    }
-    __device__ __forceinline__ Counters* ctr(int) const { return a.ctr; }
-    __device__ __forceinline__ uint32_t lane_limit() const { return a.splat_lane_limit; }
-    __device__ __forceinline__ int view_lo(int) const { return a.view_lo; }
-    __device__ __forceinline__ int view_hi(int) const { return a.view_hi; }
-};
-
-struct ManyScenes {
-    static constexpr bool kMany = true;
-    const BatchScenes& b;
-    const uint32_t* s_unit0;   // first unit of each scene, then the total
-    const uint32_t* s_n;       // work points of each scene
-    // the scene holding unit g, from that of the warp's unit before (units only
-    // go up): the last with s_unit0 <= g. One value for the warp, in a uniform
-    // register, so that the scene's constants are read from the kernel's
-    // parameters as those of a single scene are.
-    __device__ __forceinline__ int scene(uint32_t g, int from) const {
-        while (s_unit0[from + 1] <= g) from++;
-        return int(__reduce_max_sync(0xffffffffu, uint32_t(from)));
-    }
-    __device__ __forceinline__ uint32_t first_unit(int q) const { return s_unit0[q]; }
-    __device__ __forceinline__ const DispConst& dc(int q) const { return b.s[q].dc; }
-    __device__ __forceinline__ float eye(int q, int v) const { return __ldg(b.s[q].ex + v); }
-    __device__ __forceinline__ uint32_t points(int q) const { return s_n[q]; }
-    __device__ __forceinline__ const WorkRec* work(int q) const { return b.s[q].work; }
-    __device__ __forceinline__ const TriRec* rec(int q) const { return b.s[q].rec; }
-    __device__ __forceinline__ unsigned long long* keys(int q) const {
-        return reinterpret_cast<unsigned long long*>(b.s[q].keys);
-    }
-    __device__ __forceinline__ Counters* ctr(int q) const { return b.s[q].ctr; }
-    __device__ __forceinline__ uint32_t lane_limit() const { return kSplatLaneLimit; }
-    __device__ __forceinline__ int view_lo(int) const { return 0; }
-    __device__ __forceinline__ int view_hi(int q) const { return b.s[q].dc.nr; }
 };
 
 // Candidate rr of segment e: its pixel, the test, and the depth-test atomic.
@@ -196,59 +151,52 @@ __device__ __forceinline__ void test_candidate(const DispConst& c, const SplatWa
     writes++;
 }
 
-// The splat proper: warps stride through units 0 .. total-1 of `src` (a
-// unit never spans two scenes).
-template <int S, class Src>
-__device__ __forceinline__ void splat_units(const Src& src, uint32_t total_units,
+// The splat proper: warps stride through the units of the work list's n points.
+// ex_s: shared-memory address of the eye positions.
+template <int S>
+__device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint32_t ex_s,
                                             SplatWarpSmem<S, unit_pairs(S)>& sm) {
     constexpr int P = unit_pairs(S);
     const int lane = threadIdx.x & 31, sub = lane & 15, half = lane >> 4;
     const uint32_t lanes_below = (1u << lane) - 1u;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t n_warps = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t total_units = (n + 2u * P - 1u) / (2u * P);
+    const DispConst& c = a.dc;
+    const WorkRec* work = a.work;
+    unsigned long long* keys = reinterpret_cast<unsigned long long*>(a.keys);
+    const uint32_t npix = uint32_t(c.W) * uint32_t(c.H);
+    const int vlo = a.view_lo, vhi = a.view_hi;
     uint32_t writes = 0;
-    int cur = 0;
 
     for (uint32_t g = warp; g < total_units; g += n_warps) {
-        const int sc = src.scene(g, cur);
-        if constexpr (Src::kMany) {
-            if (sc != cur) {
-                add_writes(src.ctr(cur), writes);
-                writes = 0;
-                cur = sc;
-            }
-        }
-        const DispConst& c = src.dc(sc);
-        const uint32_t n = src.points(sc);
-        const WorkRec* work = src.work(sc);
-        unsigned long long* keys = src.keys(sc);
-        const uint32_t npix = uint32_t(c.W) * uint32_t(c.H);
-        const uint32_t k0 = 2u * P * (g - src.first_unit(sc));   // the unit's first work point
+        const uint32_t k0 = 2u * P * g;   // the unit's first work point
         {
             const uint32_t kn = k0 + 2u * P * n_warps + uint32_t(lane);   // the next unit's records
             if (lane < 2 * P && kn < n) prefetch_l2(work + kn);
         }
-        // the next unit's triangles (of one scene): read their ids now (the
+        // the next unit's triangles: read their ids now (the
         // work records were asked for a unit ago), ask L1 for their records'
         // 128-byte lines once this unit's candidates are formed, so that the
         // next unit's staging finds them there
         uint32_t next_tri = 0xffffffffu;
-        if constexpr (!Src::kMany) {
+        {
             const uint32_t kn = k0 + 2u * P * n_warps + uint32_t(lane);
             if (lane < 2 * P && kn < n) next_tri = __ldg(&work[kn].meta.z);
         }
-        const int vlo = src.view_lo(sc), vhi = src.view_hi(sc);
         for (int g0 = vlo; g0 < vhi; g0 += 16 * S) {
             __syncwarp();   // the previous passes are done with sm
             if (g0 == vlo) {
-                // the unit's test constants, one float4 a lane: lane 6 q + f
-                // stages float4 f of point k0 + q (a point past the end takes
+                // the unit's test constants, one float4 a lane and turn: number
+                // 6 q + f is float4 f of point k0 + q (a point past the end takes
                 // the unit's first record; it has no rows)
-                const int q = lane / 6, f = lane - 6 * q;
-                if (q < 2 * P) {
+#pragma unroll
+                for (int z = 0; z < 12 * P; z += 32) {
+                    const int q = (lane + z) / 6, f = lane + z - 6 * q;
+                    if (q >= 2 * P) break;
                     const uint32_t k = k0 + uint32_t(q);
                     const uint4 meta = __ldg(&work[k < n ? k : k0].meta);
-                    const TriRec* r = src.rec(sc) + meta.z;
+                    const TriRec* r = a.rec + meta.z;
                     float4 v = __ldg(&r->q[f < 5 ? f : 0]);
                     if (f == 0) {
                         v.y = 0.0f - v.y;
@@ -280,7 +228,7 @@ __device__ __forceinline__ void splat_units(const Src& src, uint32_t total_units
 #pragma unroll
                 for (int sl = 0; sl < S; sl++) {
                     const int v = g0 + 16 * sl + sub;
-                    if (p == 0) ex[sl] = src.eye(sc, v < vhi ? v : vlo);
+                    if (p == 0) ex[sl] = eye_x(ex_s, v < vhi ? v : vlo);
                     const float Ex = ex[sl];
                     const float lo = fmaxf(fmaf(l0.y, Ex, l0.x), fmaf(l1.y, Ex, l1.x));
                     const float hi = fminf(fmaf(l0.w, Ex, l0.z), fmaf(l1.w, Ex, l1.z));
@@ -295,7 +243,7 @@ __device__ __forceinline__ void splat_units(const Src& src, uint32_t total_units
             }
             // a segment holds at most 2^26 candidates (one view), so lanes
             // below the limit (at most 2^24) keep the unit's numbering below 2^32
-            const bool big = __any_sync(0xffffffffu, cnt >= src.lane_limit());
+            const bool big = __any_sync(0xffffffffu, cnt >= a.splat_lane_limit);
             // the unit's candidates and segments numbered in (lane, pair, slot)
             // order: one scan of both counts, the candidates in the high word
             // (wrapping as 32-bit sums would, only when the unit is walked)
@@ -320,7 +268,7 @@ __device__ __forceinline__ void splat_units(const Src& src, uint32_t total_units
                     rank += ok ? 1u : 0u;
                     first += (pk[p][sl] >> 14) * ny[p];
                 }
-            if (next_tri != 0xffffffffu && g0 == vlo) prefetch_l1(src.rec(sc) + next_tri);
+            if (next_tri != 0xffffffffu && g0 == vlo) prefetch_l1(a.rec + next_tri);
             __syncwarp();
             if (big) {
                 // huge cells: each lane walks whole segments
@@ -348,16 +296,16 @@ __device__ __forceinline__ void splat_units(const Src& src, uint32_t total_units
             }
         }
     }
-    add_writes(src.ctr(cur), writes);
+    add_writes(a.ctr, writes);
 }
 
 template <int S>
 __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
-    // With more than three slots the resolve is let in only when this block is
+    // With more than two slots the resolve is let in only when this block is
     // done: its blocks waiting on the SMs cost a splat with 40 KB or more of shared
     // memory a block a sixth of its time (96 views: 0.47 -> 0.56 ms). With fewer they
     // cost nothing, and a small frame is 3 us shorter for them.
-    constexpr bool kLate = S > 3;
+    constexpr bool kLate = S > 2;
     wait_previous_kernel();
     if constexpr (!kLate) allow_next_kernel();
     extern __shared__ __align__(16) uint8_t s_dyn[];
@@ -366,43 +314,9 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     __syncthreads();
     if (a.ctr->overflow) return;
     const uint32_t n = a.ctr->n_work;
-    const OneScene src{a, n, uint32_t(__cvta_generic_to_shared(s_ex))};
-    constexpr int P = unit_pairs(S);
-    constexpr uint32_t unit = 2u * P;
-    splat_units<S>(src, (n + unit - 1u) / unit, reinterpret_cast<SplatWarpSmem<S, P>*>(s_dyn)[threadIdx.x >> 5]);
+    splat_units<S>(a, n, uint32_t(__cvta_generic_to_shared(s_ex)),
+                   reinterpret_cast<SplatWarpSmem<S, unit_pairs(S)>*>(s_dyn)[threadIdx.x >> 5]);
     if constexpr (kLate) allow_next_kernel();
-}
-
-// Every scene of a batch in one persistent launch: warps stride through the
-// units of all scenes, so scenes of uneven size share the machine. The scenes'
-// constants are kernel parameters read through a warp-uniform scene number: as
-// operands, not as shared-memory loads and registers of their own. 12 scenes of
-// 5,000 to 200,000 triangles, whole batch 4.10 -> 3.53 ms with them there and
-// four points a unit; asking L1 for the next unit's triangles as one scene does
-// costs more registers than the constants leave (3.68).
-template <int S>
-__global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat_batch(const __grid_constant__ BatchScenes b, int n_scenes) {
-    extern __shared__ __align__(16) uint8_t s_dyn[];
-    __shared__ uint32_t s_unit0[kMaxBatchScenes + 1];   // first unit of each scene
-    __shared__ uint32_t s_n[kMaxBatchScenes];           // work points (0 after an overflow)
-    constexpr int P = unit_pairs(S);
-    constexpr uint32_t unit = 2u * P;
-    for (int q = threadIdx.x; q < n_scenes; q += blockDim.x) {
-        const Counters* ct = b.s[q].ctr;
-        s_n[q] = ct->overflow ? 0u : ct->n_work;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t u = 0;
-        for (int q = 0; q < n_scenes; q++) {
-            s_unit0[q] = u;
-            u += (s_n[q] + unit - 1u) / unit;
-        }
-        s_unit0[n_scenes] = u;
-    }
-    __syncthreads();
-    const ManyScenes src{b, s_unit0, s_n};
-    splat_units<S>(src, s_unit0[n_scenes], reinterpret_cast<SplatWarpSmem<S, P>*>(s_dyn)[threadIdx.x >> 5]);
 }
 
 // Eq. 8's interpolation weight for one view pixel whose depth test kept the
@@ -572,9 +486,7 @@ __global__ void __launch_bounds__(256) k_resolve_pbr(FrameArgs a) {
     reinterpret_cast<uint32_t*>(a.views)[o] = out;
 }
 
-// Launch with the per-warp pooling buffers as dynamic shared memory (above
-// 48 KB per block together with the static arrays only for the batched splat
-// with 8 view slots, which opts in once).
+// Launch with the per-warp pooling buffers as dynamic shared memory.
 template <int S>
 cudaError_t splat_one(const FrameArgs& a, int grid, cudaStream_t s) {
     const size_t bytes = kSplatWarps * sizeof(SplatWarpSmem<S, unit_pairs(S)>);
@@ -584,46 +496,22 @@ cudaError_t splat_one(const FrameArgs& a, int grid, cudaStream_t s) {
     return launch_after_previous(k_splat<S>, dim3(grid), dim3(kSplatWarps * 32), bytes, s, a);
 }
 
-template <int S>
-cudaError_t splat_batch(const BatchScenes& scenes, int n_scenes, int grid, cudaStream_t s) {
-    const size_t bytes = kSplatWarps * sizeof(SplatWarpSmem<S, unit_pairs(S)>);
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_splat_batch<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
-    if (attr != cudaSuccess) return attr;
-    k_splat_batch<S><<<grid, kSplatWarps * 32, bytes, s>>>(scenes, n_scenes);
-    return cudaGetLastError();
-}
-
 }  // namespace
 
 LFDPR_CHECK_READER(checks_splat)
 
-cudaError_t launch_splat(const FrameArgs& a, cudaStream_t s) {
+cudaError_t launch_splat(const FrameArgs& a, cudaStream_t s, int blocks_per_sm, int max_slots) {
     // the fewest view slots per lane that hold every view of the range
-    // [view_lo, view_hi) in one group (more than 128 views take several
-    // groups of 128)
-    const int nr = a.view_hi - a.view_lo, grid = a.sm_count * 16;
-    if (nr <= 16) return splat_one<1>(a, grid, s);
-    if (nr <= 32) return splat_one<2>(a, grid, s);
-    if (nr <= 48) return splat_one<3>(a, grid, s);
-    if (nr <= 64) return splat_one<4>(a, grid, s);
-    if (nr <= 96) return splat_one<6>(a, grid, s);
+    // [view_lo, view_hi) in one group (more than 16 max_slots views take
+    // several groups)
+    const int nr = a.view_hi - a.view_lo, grid = a.sm_count * blocks_per_sm;
+    const int slots = min((nr + 15) / 16, max_slots);
+    if (slots <= 1) return splat_one<1>(a, grid, s);
+    if (slots <= 2) return splat_one<2>(a, grid, s);
+    if (slots <= 3) return splat_one<3>(a, grid, s);
+    if (slots <= 4) return splat_one<4>(a, grid, s);
+    if (slots <= 6) return splat_one<6>(a, grid, s);
     return splat_one<8>(a, grid, s);
-}
-
-cudaError_t launch_splat_batch(const BatchScenes& scenes, int n_scenes, int slots, int grid_per_sm, int sm_count,
-                               cudaStream_t s) {
-    if (n_scenes < 1 || n_scenes > kMaxBatchScenes || grid_per_sm < 1) return cudaErrorInvalidValue;
-    const int grid = sm_count * grid_per_sm;
-    switch (slots) {
-        case 1: return splat_batch<1>(scenes, n_scenes, grid, s);
-        case 2: return splat_batch<2>(scenes, n_scenes, grid, s);
-        case 3: return splat_batch<3>(scenes, n_scenes, grid, s);
-        case 4: return splat_batch<4>(scenes, n_scenes, grid, s);
-        case 6: return splat_batch<6>(scenes, n_scenes, grid, s);
-        case 8: return splat_batch<8>(scenes, n_scenes, grid, s);
-        default: return cudaErrorInvalidValue;
-    }
 }
 
 cudaError_t launch_resolve(const FrameArgs& a, cudaStream_t s) {
