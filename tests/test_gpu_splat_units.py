@@ -1,0 +1,37 @@
+"""The splat's units and blocks: view counts at the edges of every number of view
+slots a lane, work lists from a few points to beyond a wave of blocks (where the
+splat takes more blocks); sampling equals the oracle's and so do the views looked
+at."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2601_19901_gb300 import lfdpr, scenes as S
+from parity import check_sampling, check_views, gpu_frame
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2601_19901_gb300 import build
+    build.build()
+    lfdpr.lib()
+
+
+# views, horizontal sampling bias (lower: more points)
+@pytest.mark.parametrize("views,bias", [(1, 2.0), (16, 2.0), (17, 2.0), (32, 4.0), (33, 2.0), (48, 4.0), (49, 2.0),
+                                        (64, 4.0), (65, 4.0), (96, 2.0), (97, 4.0), (128, 4.0), (16, 0.05),
+                                        (33, 0.08), (96, 0.1)])
+def test_views_equal_the_oracles(views, bias):
+    d = replace(S.display_tiny(), n_views=views, view_w=96, view_h=96, bias_h=bias, bias_v=min(bias, 1.0))
+    sc, m = S.scene_tiny(), S.model_matrix(4)
+    looked_at = sorted({0, views // 2, views - 1})
+    o = O.render(d, sc, m, views=looked_at, panel=False)
+    g = gpu_frame(d, sc, m, max_points=len(o.points) + 1, panel=False)
+    check_sampling(g, o)
+    check_views(g, o, views=looked_at)
