@@ -262,9 +262,10 @@ lfdpr_status lfdpr_render_batch(lfdpr_batch* b, const float* models, void* strea
     b->replayed = true;
     for (int i = 0; i < b->n; i++) {
         b->disp[i]->ev_frame = b->disp[i]->ev_interleave = false;
-        // set-up, scan, emission, fetch, near-limit records (and the
+        // set-up, (scan,) emission, fetch, near-limit records (and the
         // materials' fetch), splat, resolve, (view mips,) interleave
-        b->disp[i]->launches += (b->mesh[i]->n_tris ? (b->mesh[i]->mat_tex ? 9 : 8) : 3) + (b->disp[i]->ss_level > 0);
+        b->disp[i]->launches += (b->mesh[i]->n_tris ? (b->mesh[i]->mat_tex ? 8 : 7) : 3) +
+                                (b->mesh[i]->n_blocks > kEmitScans) + (b->disp[i]->ss_level > 0);
     }
     return LFDPR_OK;
 }

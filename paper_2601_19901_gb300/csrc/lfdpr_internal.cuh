@@ -15,8 +15,11 @@ constexpr int kMaxRenderViews = 512;
 constexpr int kMaxCell = 65535;          // lattice indices are stored as u16
 constexpr int kMaxLevels = 16;           // mip levels of a texture (16384 = 2^14 texels a side)
 constexpr int kSetupThreads = 256;       // triangles per set-up / emit block
+// Blocks of triangles up to which k_emit's blocks sum the blocks before them
+// themselves instead of k_scan for all (the reads grow with the square: at 3,900
+// blocks the two take the same 40 us).
+constexpr uint32_t kEmitScans = 2048;
 constexpr uint32_t kEmitOwn = 128;       // points up to which a triangle is emitted by its own thread
-constexpr uint32_t kEmitOwnFew = 24;     // the same for meshes of few triangles
 constexpr float kBoxPad = 1.0f / 256.0f; // margin (pixels) of candidate pixel ranges against rounding
                                          // (projection error is about 1e-4 pixel)
 
@@ -341,7 +344,8 @@ struct FrameArgs {
     uint32_t* counts;
     uint32_t* offsets;
     uint4* colsum;                   // [n_tris] column summaries (k_setup -> k_emit); null: k_emit walks
-    uint32_t* block_sums;            // [n_blocks]
+    uint32_t* block_sums;            // [n_blocks] points of each block of triangles, then the points before it
+    uint32_t* block_live;            // [n_blocks] its live triangles, and those of too many cells << 16
     uint32_t n_blocks;
     uint4* points;
     uint32_t max_points;

@@ -29,7 +29,7 @@ constexpr uint32_t kNoAllocBlocks = (kNoAllocMaxTris + kSetupThreads - 1) / kSet
 struct NoAllocScratch {
     TriRec rec[kNoAllocMaxTris];
     uint32_t offsets[kNoAllocMaxTris];
-    uint32_t block_sums[kNoAllocBlocks];
+    uint32_t block_sums[kNoAllocBlocks], block_live[kNoAllocBlocks];
     Counters ctr;
     float ex[kMaxRenderViews];
     TexDesc tex[kNoAllocMaxTex];
@@ -191,6 +191,7 @@ extern "C" lfdpr_status lfdpr_sample_points_noalloc(
     a.counts = counts;
     a.offsets = scr->offsets;
     a.block_sums = scr->block_sums;
+    a.block_live = scr->block_live;
     a.n_blocks = (n_tris + kSetupThreads - 1) / kSetupThreads;
     a.points = reinterpret_cast<uint4*>(points);
     a.max_points = max_points;

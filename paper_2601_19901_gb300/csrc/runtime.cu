@@ -126,6 +126,7 @@ FrameArgs frame_args(const lfdpr_display* disp, const lfdpr_mesh* mesh) {
     a.offsets = mesh->offsets;
     a.colsum = mesh->colsum;
     a.block_sums = mesh->block_sums;
+    a.block_live = mesh->block_sums + mesh->n_blocks;
     a.n_blocks = mesh->n_blocks;
     a.points = disp->points;
     a.max_points = disp->max_points;
@@ -160,7 +161,8 @@ lfdpr_status record_frame_front(lfdpr_display* disp, lfdpr_mesh* mesh, const Fra
         cudaError_t e_ = (call);                             \
         if (e_ != cudaSuccess) return cuda_fail(e_, what);   \
     } while (0)
-    CKF(cudaMemsetAsync(disp->ctr, 0, sizeof(Counters), s), "reset counters");
+    // the point generation writes the counters whole; an empty mesh has none
+    if (!mesh->n_tris) CKF(cudaMemsetAsync(disp->ctr, 0, sizeof(Counters), s), "reset counters");
     mk(0);
     if (mesh->n_tris) {
         CKF(launch_setup(a, s), "launch k_setup");
@@ -171,7 +173,7 @@ lfdpr_status record_frame_front(lfdpr_display* disp, lfdpr_mesh* mesh, const Fra
         mk(3);
         CKF(launch_fetch(a, s), "launch k_fetch");
         CKF(launch_near_work(a, s), "launch k_near_work");
-        disp->launches += 5;
+        disp->launches += a.n_blocks > kEmitScans ? 5 : 4;
         if (a.mat_tex) {
             CKF(launch_fetch_mat(a, s), "launch k_fetch_mat");
             disp->launches += 1;
@@ -399,7 +401,7 @@ lfdpr_status upload_geometry(lfdpr_display* disp, const float* xyz, const float*
         (e = dev_malloc(&m->tproj, sizeof(TriProj) * nt)) != cudaSuccess ||
         (e = dev_malloc(&m->counts, 4u * nt)) != cudaSuccess || (e = dev_malloc(&m->offsets, 4u * nt)) != cudaSuccess ||
         (e = dev_malloc(&m->colsum, sizeof(uint4) * nt)) != cudaSuccess ||
-        (e = dev_malloc(&m->block_sums, 4u * (m->n_blocks ? m->n_blocks : 1))) != cudaSuccess) {
+        (e = dev_malloc(&m->block_sums, 8u * (uint64_t)(m->n_blocks ? m->n_blocks : 1))) != cudaSuccess) {
         free_mesh(m);
         return cuda_fail(e, "upload_mesh: allocation");
     }

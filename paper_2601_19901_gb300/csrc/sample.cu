@@ -5,8 +5,8 @@
 //            eye, Eq. 1-3 texture limit, Eq. 4-7 mip set-up, point count by the
 //            lattice column walk (each column's first row and row count kept
 //            for k_emit when there are at most four); block sums for the scan.
-//   k_scan   one block: exclusive scan of the block sums -> block offsets,
-//            total point count, overflow flag.
+//   k_scan   (meshes of many blocks) one block: exclusive scan of the block
+//            sums -> block offsets, the frame's counters.
 //   k_emit   one thread per triangle: warp-shuffle block scan of the counts
 //            plus the block offset gives each triangle's first point id; the
 //            column summary writes (triangle, cell) for each of its points; a
@@ -18,8 +18,9 @@
 //            some view can hold a candidate pixel of it, its place in the
 //            splat's work list; the pass ends with the frame's key reset.
 //
-// Every kernel after k_setup is launched as a programmatic dependent of the
-// one before it and waits for it at its top (wait_previous_kernel).
+// Every kernel is launched as a programmatic dependent of the one before it on
+// the stream (of k_setup, the frame before's last) and waits for it at its top
+// (wait_previous_kernel).
 //   k_near_work  one thread per point whose cell or triangle reaches within
 //            near_z of the eyes' plane: the splat record of its cell and
 //            triangle clipped to that limit.
@@ -478,31 +479,51 @@ __global__ void __launch_bounds__(kSetupThreads, 4) k_setup(FrameArgs a) {
         for (int k = 0; k < 8; k += 2) store32(&dst->q[k], r.q[k], r.q[k + 1]);
         if (o.live && a.tproj) a.tproj[t] = tp;
         count = o.count;
-        live = o.live ? 1u : 0u;
+        live = (o.live ? 1u : 0u) | (o.cell_overflow ? 1u << 16 : 0u);
         a.counts[t] = count;
-        if (o.cell_overflow) atomicExch(&a.ctr->cell_overflow, 1u);
     }
     const uint32_t bs = block_sum(count, s_cnt);
     const uint32_t bl = block_sum(live, s_live);
     if (threadIdx.x == 0) {
         a.block_sums[blockIdx.x] = bs;
-        if (bl) atomicAdd(&a.ctr->n_live, bl);
+        a.block_live[blockIdx.x] = bl;
     }
+}
+
+// The frame's counters, from the whole mesh's totals; those that later kernels
+// add to start at zero.
+__device__ __forceinline__ void write_counters(const FrameArgs& a, unsigned long long points, uint32_t live,
+                                               bool cell_overflow) {
+    Counters c{};
+    c.n_points = uint32_t(points > 0xffffffffull ? 0xffffffffull : points);
+    c.overflow = points > (unsigned long long)a.max_points ? 1u : 0u;
+    c.cell_overflow = cell_overflow ? 1u : 0u;
+    c.n_live = live;
+    *a.ctr = c;
 }
 
 // Exclusive scan of the per-block point counts in one block of 1024 threads:
 // each thread sums a contiguous run of ceil(n / 1024) block sums, the block
 // scans those 1024 sums, and each thread writes its run's prefixes; the
-// total decides overflow. Prefixes saturate at 2^32 - 1.
+// total decides overflow. Prefixes saturate at 2^32 - 1. (Of smaller meshes
+// k_emit's blocks do the same for themselves: see launch_scan.)
 __global__ void __launch_bounds__(1024) k_scan(FrameArgs a) {
     wait_previous_kernel();
     allow_next_kernel();
     __shared__ unsigned long long s_warp[32];
+    __shared__ uint32_t s_live, s_cell;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t n = a.n_blocks, per = (n + 1023u) / 1024u;
     const uint32_t lo = min(n, threadIdx.x * per), hi = min(n, lo + per);
+    if (threadIdx.x == 0) s_live = s_cell = 0u;
     unsigned long long run = 0ull;
-    for (uint32_t k = lo; k < hi; k++) run += a.block_sums[k];
+    uint32_t live = 0u, cell = 0u;
+    for (uint32_t k = lo; k < hi; k++) {
+        run += a.block_sums[k];
+        const uint32_t l = a.block_live[k];
+        live += l & 0xffffu;
+        cell |= l >> 16;
+    }
     unsigned long long inc = run;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -511,6 +532,12 @@ __global__ void __launch_bounds__(1024) k_scan(FrameArgs a) {
     }
     if (lane == 31) s_warp[warp] = inc;
     __syncthreads();
+    live = __reduce_add_sync(0xffffffffu, live);
+    cell = __reduce_or_sync(0xffffffffu, cell);
+    if (lane == 0) {
+        atomicAdd(&s_live, live);
+        atomicOr(&s_cell, cell);
+    }
     if (warp == 0) {
         unsigned long long w = s_warp[lane];
 #pragma unroll
@@ -527,11 +554,7 @@ __global__ void __launch_bounds__(1024) k_scan(FrameArgs a) {
         a.block_sums[k] = uint32_t(excl > 0xffffffffull ? 0xffffffffull : excl);
         excl += v;
     }
-    if (threadIdx.x == 1023) {
-        const unsigned long long total = s_warp[31];
-        a.ctr->n_points = uint32_t(total > 0xffffffffull ? 0xffffffffull : total);
-        a.ctr->overflow = total > (unsigned long long)a.max_points ? 1u : 0u;
-    }
+    if (threadIdx.x == 1023) write_counters(a, s_warp[31], s_live, s_cell != 0u);
 }
 
 // The part of a triangle's record that its column walk needs.
@@ -593,7 +616,7 @@ __device__ __forceinline__ int last_at_most(const uint32_t* s_num, uint32_t k) {
 // Block-level exclusive scan of the counts, plus the block's offset: each
 // triangle's first point id. Then emit its points in (column, row) order.
 //
-// A triangle of up to own_max points is emitted by its thread, from the columns
+// A triangle of up to kEmitOwn points is emitted by its thread, from the columns
 // that k_setup kept or, of more than four columns, by walking them. The others
 // are the block's together: their columns are numbered in one sequence, of which
 // a thread takes one column at a time (its first row and row count from the
@@ -607,11 +630,17 @@ __device__ __forceinline__ int last_at_most(const uint32_t* s_num, uint32_t k) {
 // Bound by the dependent chain of a block's largest triangle while one thread or
 // one warp emits it; shared out, by the searches and stores of its points.
 // Measured on twelve meshes of 61 k to 1.2 M points (24 to 96 views): 608 us
-// before in sum (a thread a triangle, a lane a column above 128 points), 293 us
-// now; 5.4 M points on 10 k triangles 221 -> 40 us; a mesh of 871 k triangles of
-// a few points each 31 us both. With own_max 64 for unsplit and 48 for split
-// blocks instead of 128 and 24: 376 us.
-__global__ void __launch_bounds__(kSetupThreads) k_emit(FrameArgs a, uint32_t split, uint32_t own_max) {
+// before in sum (a thread a triangle, a lane a column above 128 points), 310 us
+// now; 5.4 M points on 10 k triangles 221 -> 47 us; a mesh of 871 k triangles of
+// a few points each 31 us both. With kEmitOwn 64 for meshes of many blocks 2 %
+// more; with 24 for those of few 299 us, but points alone of 32,400 triangles at
+// eight poses 332 us instead of 318.
+//
+// kScanned: block_sums are k_scan's prefixes. Else each block sums the blocks
+// before it, and block 0 writes the frame's counters. (Two kernels: the walk of
+// one that chooses as it runs has fewer registers, 45 -> 56 us at one pose.)
+template <bool kScanned>
+__global__ void __launch_bounds__(kSetupThreads) k_emit(FrameArgs a, uint32_t split) {
     wait_previous_kernel();
     allow_next_kernel();
     __shared__ uint32_t s_sum[kSetupThreads / 32];
@@ -628,12 +657,56 @@ __global__ void __launch_bounds__(kSetupThreads) k_emit(FrameArgs a, uint32_t sp
     const bool mine = t < a.n_tris && threadIdx.x / width == part;
     uint4 cs = make_uint4(kColSumWalk, 0u, 0u, 0u);
     if (mine && a.colsum) cs = __ldcg(a.colsum + t);
-    const uint32_t before = a.block_sums[blk], overflow = a.ctr->overflow;
-    const uint32_t first = block_scan(cnt, s_sum) - cnt + before;
+    uint32_t first;
+    bool overflow;
+    if constexpr (kScanned) {
+        const uint32_t before = a.block_sums[blk];
+        overflow = a.ctr->overflow != 0u;
+        first = block_scan(cnt, s_sum) - cnt + before;
+    } else {
+        // the points of the blocks before this one, and of all
+        unsigned long long before = 0ull, all = 0ull;
+        for (uint32_t k = threadIdx.x; k < a.n_blocks; k += kSetupThreads) {
+            const uint32_t v = a.block_sums[k];
+            all += v;
+            before += k < blk ? v : 0u;
+        }
+        __shared__ unsigned long long s_all[2][kSetupThreads / 32];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            before += __shfl_xor_sync(0xffffffffu, before, o);
+            all += __shfl_xor_sync(0xffffffffu, all, o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            s_all[0][threadIdx.x >> 5] = before;
+            s_all[1][threadIdx.x >> 5] = all;
+        }
+        first = block_scan(cnt, s_sum) - cnt;   // (its barriers are those of s_all too)
+        before = all = 0ull;
+#pragma unroll
+        for (int w = 0; w < kSetupThreads / 32; w++) {
+            before += s_all[0][w];
+            all += s_all[1][w];
+        }
+        first += uint32_t(before > 0xffffffffull ? 0xffffffffull : before);
+        overflow = all > (unsigned long long)a.max_points;
+        if (blockIdx.x == 0) {
+            uint32_t live = 0u, cell = 0u;
+            for (uint32_t k = threadIdx.x; k < a.n_blocks; k += kSetupThreads) {
+                const uint32_t l = a.block_live[k];
+                live += l & 0xffffu;
+                cell |= l >> 16;
+            }
+            __shared__ uint32_t s_live[kSetupThreads / 32];
+            live = block_sum(live, s_live);
+            const bool any = __syncthreads_or(cell != 0u);
+            if (threadIdx.x == 0) write_counters(a, all, live, any);
+        }
+    }
     if (mine) a.offsets[t] = first;
-    if (overflow != 0u) return;
+    if (overflow) return;
     const bool live = mine && cnt > 0u;
-    const bool walk = cs.x == kColSumWalk, together = live && cnt > own_max;
+    const bool walk = cs.x == kColSumWalk, together = live && cnt > kEmitOwn;
     const uint32_t w[4] = {cs.x, cs.y, cs.z, cs.w};
     if (live && !together) {
         uint32_t p = first;
@@ -1320,11 +1393,13 @@ __global__ void __launch_bounds__(256) k_fetch_mat(FrameArgs a) {
 LFDPR_CHECK_READER(checks_sample)
 
 cudaError_t launch_setup(const FrameArgs& a, cudaStream_t s) {
-    k_setup<<<a.n_blocks, kSetupThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_after_previous(k_setup, dim3(a.n_blocks), dim3(kSetupThreads), 0, s, a);
 }
 
+// One launch and its wait less: a frame of 2,048 triangles 38.4 -> 33.7 us, with
+// the counters' memset and k_setup's plain launch gone too.
 cudaError_t launch_scan(const FrameArgs& a, cudaStream_t s) {
+    if (a.n_blocks <= kEmitScans) return cudaSuccess;
     return launch_after_previous(k_scan, dim3(1), dim3(1024), 0, s, a);
 }
 
@@ -1332,8 +1407,7 @@ cudaError_t launch_emit(const FrameArgs& a, cudaStream_t s) {
     // the largest split (a power of two up to 8) that leaves an SM at most two blocks
     uint32_t split = 1;
     while (split < 8u && 2u * split * a.n_blocks <= 2u * uint32_t(a.sm_count)) split *= 2u;
-    return launch_after_previous(k_emit, dim3(a.n_blocks * split), dim3(kSetupThreads), 0, s, a, split,
-                                 split == 1u ? kEmitOwn : kEmitOwnFew);
+    return launch_after_previous(a.n_blocks > kEmitScans ? k_emit<true> : k_emit<false>, dim3(a.n_blocks * split), dim3(kSetupThreads), 0, s, a, split);
 }
 
 cudaError_t launch_fetch_mat(const FrameArgs& a, cudaStream_t s) {

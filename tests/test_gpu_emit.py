@@ -83,3 +83,38 @@ def test_the_allocation_free_point_set_is_the_oracles(n, bias, largest):
     assert np.array_equal(counts.cpu().numpy().view(np.uint32), want_counts)
     got = pts.cpu().numpy().view(np.uint32)
     assert np.array_equal(got[:total, :2], want[:, :2]) and not got[total:].any()
+
+
+# blocks of triangles where a block's sums over the blocks before it end (2,048), and one past
+@pytest.mark.parametrize("blocks,over", [(2048, 0), (2048, 1), (1, 0), (5, 7)])
+@pytest.mark.parametrize("short", [0, 1])
+def test_counters_and_offsets_of_whole_meshes(blocks, over, short):
+    import torch
+    n = 256 * blocks + over
+    d = replace(S.display_tiny(), bias_h=4.0, bias_v=4.0)
+    rng = np.random.default_rng(n)
+    tris = rng.uniform(-0.9, 0.9, (n, 1, 3)) + 0.02 * rng.uniform(-1, 1, (n, 3, 3))
+    tris[rng.random(n) < 0.1] += 40.0                 # some out of sight
+    sc = S.Scene(xyz=tris.reshape(-1, 3).astype(np.float32), uv=rng.uniform(0, 1, (3 * n, 2)).astype(np.float32),
+                 idx=np.arange(3 * n, dtype=np.uint32).reshape(n, 3), tri_tex=np.zeros(n, np.uint32),
+                 textures=[S.value_noise_texture(64, 64, 7)])
+    m = np.eye(4, dtype=np.float32)
+    _, tri, want = O.setup(d, sc, m)
+    total, live = int(want.sum()), int((tri[:, O.F["live"]] == 1).sum())
+    offsets = np.concatenate([[0], np.cumsum(want.astype(np.int64))[:-1]])
+    assert 0 < live < n or n < 300
+    s = torch.cuda.current_stream()
+    with lfdpr.Renderer(d, sc, total - short) as R:
+        for _ in range(2):                            # the second frame finds the first one's counters
+            R.render(m, s)
+            if short:
+                with pytest.raises(lfdpr.LfdprError, match="needed %d points" % total):
+                    R.stats(s)
+            else:
+                st = R.stats(s)
+                assert (st.n_points, st.n_live_tris, st.overflow, st.cell_overflow) == (total, live, 0, 0)
+            b = R.buffers()
+            assert np.array_equal(lfdpr.device_to_numpy(b.offsets, (n,), np.uint32), offsets)
+            if not short:
+                got = lfdpr.device_to_numpy(b.points, (total, 4), np.uint32)
+                assert np.array_equal(got[:, :2], O.emit(tri, want)[:, :2])
