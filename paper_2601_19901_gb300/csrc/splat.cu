@@ -108,14 +108,14 @@ __device__ __forceinline__ uint32_t div_floor(uint32_t r, uint32_t n) {
 // Units of 2P points per warp: pairs per unit for S view slots per lane. More
 // points share the unit's scan and fill its passes better; more segments take
 // more shared memory and registers, and a small mesh has fewer units to spread.
-// Splat of 10^6 triangles (200 instances), P = 1 for S = 6, else 2, against
-// these: 8 views (S = 1) 172 -> 131 us, 24 (S = 2) 220 -> 190, 48 (S = 3)
-// 292 -> 283, 96 (S = 6) 557 -> 471. P = 5 for S = 1 gave 124 but a frame of
-// 2,048 triangles 1 us more; P = 5 for S = 2 223; P = 4 for S = 3 286; P = 3 for
-// S = 4 350 against 353 but slower small frames. With S = 8 two pairs would
+// Splat of 10^6 triangles (200 instances), P = 1 for S = 6 and 8, else 2, against
+// these: 8 views (S = 1) 172 -> 104 us, 24 (S = 2) 220 -> 180, 48 (S = 3)
+// 292 -> 265, 96 (S = 6) 557 -> 462. P = 4 for S = 1 gave 121 (and a frame of
+// 2,048 triangles 0.4 us less); P = 5 for S = 2 223; P = 4 for S = 3 286 of 283;
+// P = 3 for S = 4 350 of 353 but slower small frames. With S = 8 two pairs would
 // leave an SM three blocks.
 __host__ __device__ constexpr int unit_pairs(int S) {
-    return S <= 2 ? 4 : S == 3 ? 3 : S <= 6 ? 2 : 1;
+    return S == 1 ? 6 : S <= 2 ? 4 : S == 3 ? 3 : S <= 6 ? 2 : 1;
 }
 
 // Per-warp shared memory of the pooled splat: the unit's non-empty (point,
@@ -192,32 +192,36 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
         }
         for (int g0 = vlo; g0 < vhi; g0 += 16 * S) {
             __syncwarp();   // the previous passes are done with sm
-            if (g0 == vlo) {
+            // (formed after the candidates where the registers allow: 64 views 345 -> 337 us,
+            // 48 views 270 -> 265; with six slots it costs 3 %)
+            auto stage = [&] {
+                if (g0 != vlo) return;
                 // the unit's test constants, one float4 a lane and turn: number
-                // 6 q + f is float4 f of point k0 + q (a point past the end takes
-                // the unit's first record; it has no rows)
+                // 5 q + f is float4 f of point k0 + q (a point past the end takes
+                // the unit's first record; it has no rows), and with the cell's
+                // spacings (f = 0 and 1) go its u and its v bounds. Five numbers a
+                // point, not six, are one turn for six points: 10^6 triangles at 48
+                // views 285 -> 270 us, at 8 views 131 -> 121, at 96 467 -> 465.
 #pragma unroll
-                for (int z = 0; z < 12 * P; z += 32) {
-                    const int q = (lane + z) / 6, f = lane + z - 6 * q;
+                for (int z = 0; z < 10 * P; z += 32) {
+                    const int q = (lane + z) / 5, f = lane + z - 5 * q;
                     if (q >= 2 * P) break;
                     const uint32_t k = k0 + uint32_t(q);
                     const uint4 meta = __ldg(&work[k < n ? k : k0].meta);
-                    const TriRec* r = a.rec + meta.z;
-                    float4 v = __ldg(&r->q[f < 5 ? f : 0]);
+                    float4 v = __ldg(&a.rec[meta.z].q[f]);
+                    if (f < 2) {
+                        const uint32_t ij = f == 0 ? meta.y & 0xffffu : meta.y >> 16;
+                        reinterpret_cast<float2*>(&sm.pt[q][5])[f] = make_float2(float(int(ij)) * v.w, float(int(ij) + 1) * v.w);
+                        v.w = __uint_as_float(f == 0 ? meta.w : meta.x);
+                    }
                     if (f == 0) {
                         v.y = 0.0f - v.y;
                         v.z = c.D - v.z;
-                        v.w = __uint_as_float(meta.w);
-                    } else if (f == 1) {
-                        v.w = __uint_as_float(meta.x);
-                    } else if (f == 5) {
-                        const float sv = __ldg(&r->q[1].w);
-                        const int i = int(meta.y & 0xffffu), j = int(meta.y >> 16);
-                        v = make_float4(float(i) * v.w, float(i + 1) * v.w, float(j) * sv, float(j + 1) * sv);
                     }
                     sm.pt[q][f] = v;
                 }
-            }
+            };
+            if constexpr (S > 4) stage();
             uint32_t pk[P][S], ny[P];
             float ex[S];   // the lane's views' eyes, the same for every pair
             uint32_t cnt = 0, nz = 0;   // the lane's candidates and non-empty (point, view) segments
@@ -247,6 +251,7 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
                     nz += ok ? 1u : 0u;
                 }
             }
+            if constexpr (S <= 4) stage();
             // a segment holds at most 2^26 candidates (one view), so lanes
             // below the limit (at most 2^24) keep the unit's numbering below 2^32
             const bool big = __any_sync(0xffffffffu, cnt >= a.splat_lane_limit);
