@@ -213,12 +213,9 @@ __device__ __forceinline__ bool inside_either(float w0, float w1, float w2) {
 // log2 by the atanh series (Eq. 6-7): x = m 2^e from the bits, m folded into
 // [sqrt(1/2), sqrt(2)], ln m = 2 atanh(z) with z = (m-1)/(m+1) summed through
 // the z^9/9 term, log2 x = e + ln m / ln 2.
-__device__ __forceinline__ float log2_series(float x) {
-    if (isnan(x)) return x;
-    if (x <= 0.0f) return -INFINITY;
-    if (isinf(x)) return INFINITY;
+// log2_parts: e and ln m of a positive finite x.
+__device__ __forceinline__ float log2_parts(float x, int& e) {
     uint32_t b = __float_as_uint(x);
-    int e;
     if ((b >> 23) == 0u) {
         b = __float_as_uint(x * 16777216.0f);
         e = int(b >> 23) - 151;
@@ -233,8 +230,18 @@ __device__ __forceinline__ float log2_series(float x) {
     s = fmaf(z2, s, (float)(1.0 / 5.0));
     s = fmaf(z2, s, (float)(1.0 / 3.0));
     s = fmaf(z2, s, 1.0f);
-    const float ln_m = (2.0f * z) * s;
+    return (2.0f * z) * s;
+}
+__device__ __forceinline__ float log2_of(float ln_m, int e) {
     return fmaf(ln_m, (float)(1.0 / 0.69314718055994530942), float(e));   // / ln 2
+}
+__device__ __forceinline__ float log2_series(float x) {
+    if (isnan(x)) return x;
+    if (x <= 0.0f) return -INFINITY;
+    if (isinf(x)) return INFINITY;
+    int e;
+    const float ln_m = log2_parts(x, e);
+    return log2_of(ln_m, e);
 }
 
 __device__ __forceinline__ uint8_t round_u8(float v) {

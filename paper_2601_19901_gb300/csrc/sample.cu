@@ -839,6 +839,7 @@ __device__ __forceinline__ float bilinear_channel(const BilinearTap& b, int ch) 
 // levels' samples are shared instead of loaded and blended twice (the LOD
 // pair of a triangle mostly lies within one level). loff[l] is the byte
 // offset of level l in the pool.
+template <bool kThird = true>
 __device__ __forceinline__ void trilinear_pair(const uint8_t* __restrict__ pool, const uint64_t* __restrict__ loff,
                                                uint32_t w, uint32_t h, int L, float s, float t, float lod_a,
                                                float lod_b, uint32_t& out_a, uint32_t& out_b) {
@@ -861,7 +862,7 @@ __device__ __forceinline__ void trilinear_pair(const uint8_t* __restrict__ pool,
     BilinearTap ta, tb, te;
     bilinear_load(pool, loff, w, h, A, fs, ft, ta);
     bilinear_load(pool, loff, w, h, B, fs, ft, tb);
-    bilinear_load(pool, loff, w, h, D, fs, ft, te);
+    if (kThird || C != A) bilinear_load(pool, loff, w, h, D, fs, ft, te);
     uint32_t out[2] = {0u, 0u};
     const bool blend0 = frac[0] > 0.0f && lev[0] < L, blend1 = frac[1] > 0.0f && lev[1] < L;
 #pragma unroll
@@ -1330,6 +1331,10 @@ __global__ void __launch_bounds__(256) k_near_work(FrameArgs a) {
 // texture coordinate (as k_fetch); the normal map's two RGBA8 values go to
 // rmat, the roughness and metallic R channels to the resolve record's b.w as
 // bytes (min, max, min, max).
+// Bound by issue and the texel gathers. 2.6 M points, maps of three sizes: 146 us
+// with two logarithms a map, an unconditional third level and a 16-byte record;
+// 158 with the shading record (which takes 51 us off the resolve), 142 with the
+// logarithms' series taken once and the third level only where it is used.
 __global__ void __launch_bounds__(256) k_fetch_mat(FrameArgs a) {
     wait_previous_kernel();
     allow_next_kernel();
@@ -1347,14 +1352,21 @@ __global__ void __launch_bounds__(256) k_fetch_mat(FrameArgs a) {
         const float s = fmaf(q6.y, uc, fmaf(q6.z, vc, q6.x));
         const float t = fmaf(q7.x, uc, fmaf(q7.y, vc, q6.w));
         const uint4 mt = __ldg(a.mat_tex + __ldg(a.tri_tex + pt.x));
+        // the LODs' logarithms: a texture's sides are powers of two, at most 2^14, so
+        // that for bounds well inside the normal range (x w) h is x with a larger
+        // exponent, and the series of x serves all three
+        const bool scales = q5.y >= 0x1p-126f && q5.z <= 0x1p96f && q5.z >= 0x1p-126f && q5.y <= 0x1p96f;
+        int e_lo = 0, e_hi = 0;
+        const float ln_lo = scales ? log2_parts(q5.y, e_lo) : 0.0f, ln_hi = scales ? log2_parts(q5.z, e_hi) : 0.0f;
         uint32_t lo[3], hi[3];
 #pragma unroll
         for (int k = 0; k < 3; k++) {
             const uint32_t id = k == 0 ? mt.y : k == 1 ? mt.z : mt.w;
             const TexDesc tk = a.tex[id];
-            const float lod_lo = 0.5f * log2_series((q5.y * float(tk.w)) * float(tk.h));
-            const float lod_hi = 0.5f * log2_series((q5.z * float(tk.w)) * float(tk.h));
-            trilinear_pair(a.pool, a.lvl + (size_t)id * kMaxLevels, tk.w, tk.h, int(tk.levels) - 1, s, t, lod_lo,
+            const int sides = 62 - __clz(int(tk.w)) - __clz(int(tk.h));   // log2 w + log2 h
+            const float lod_lo = 0.5f * (scales ? log2_of(ln_lo, e_lo + sides) : log2_series((q5.y * float(tk.w)) * float(tk.h)));
+            const float lod_hi = 0.5f * (scales ? log2_of(ln_hi, e_hi + sides) : log2_series((q5.z * float(tk.w)) * float(tk.h)));
+            trilinear_pair<false>(a.pool, a.lvl + (size_t)id * kMaxLevels, tk.w, tk.h, int(tk.levels) - 1, s, t, lod_lo,
                            lod_hi, lo[k], hi[k]);
         }
         a.rmat[p] = make_uint2(lo[0], hi[0]);
