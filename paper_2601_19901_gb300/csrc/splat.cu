@@ -161,10 +161,10 @@ __device__ __forceinline__ void test_candidate(const DispConst& c, const SplatWa
 
 // The splat proper: n_warps warps stride through the units of the work list's n
 // points. ex_s: shared-memory address of the eye positions.
-template <int S>
-__device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint32_t total_units, uint32_t n_warps, uint32_t ex_s,
-                                            SplatWarpSmem<S, unit_pairs(S)>& sm) {
-    constexpr int P = unit_pairs(S);
+template <int S, int P>
+__device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint32_t unit, uint32_t total_units,
+                                            uint32_t n_warps, uint32_t ex_s, SplatWarpSmem<S, P>& sm) {
+    const uint32_t per = S <= 3 ? unit : 2u * P;   // points of a unit
     const int lane = threadIdx.x & 31, sub = lane & 15, half = lane >> 4;
     const uint32_t lanes_below = (1u << lane) - 1u;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -176,9 +176,10 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
     uint32_t writes = 0;
 
     for (uint32_t g = warp; g < total_units; g += n_warps) {
-        const uint32_t k0 = 2u * P * g;   // the unit's first work point
+        const uint32_t k0 = per * g;   // the unit's first work point, and the end of its points
+        const uint32_t k_end = S <= 3 ? min(n, k0 + per) : n;
         {
-            const uint32_t kn = k0 + 2u * P * n_warps + uint32_t(lane);   // the next unit's records
+            const uint32_t kn = k0 + per * n_warps + uint32_t(lane);   // the next unit's records
             if (lane < 2 * P && kn < n) prefetch_l2(work + kn);
         }
         // the next unit's triangles: read their ids now (the
@@ -187,7 +188,7 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
         // next unit's staging finds them there
         uint32_t next_tri = 0xffffffffu;
         {
-            const uint32_t kn = k0 + 2u * P * n_warps + uint32_t(lane);
+            const uint32_t kn = k0 + per * n_warps + uint32_t(lane);
             if (lane < 2 * P && kn < n) next_tri = __ldg(&work[kn].meta.z);
         }
         for (int g0 = vlo; g0 < vhi; g0 += 16 * S) {
@@ -207,7 +208,7 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
                     const int q = (lane + z) / 5, f = lane + z - 5 * q;
                     if (q >= 2 * P) break;
                     const uint32_t k = k0 + uint32_t(q);
-                    const uint4 meta = __ldg(&work[k < n ? k : k0].meta);
+                    const uint4 meta = __ldg(&work[k < k_end ? k : k0].meta);
                     float4 v = __ldg(&a.rec[meta.z].q[f]);
                     if (f < 2) {
                         const uint32_t ij = f == 0 ? meta.y & 0xffffu : meta.y >> 16;
@@ -229,10 +230,10 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
             for (int p = 0; p < P; p++) {
                 // a half past the end takes the unit's first record, with no rows
                 const uint32_t k = k0 + 2u * p + uint32_t(half);
-                const WorkRec* wr = work + (k < n ? k : k0);
+                const WorkRec* wr = work + (k < k_end ? k : k0);
                 const float4 l0 = __ldg(&wr->L0), l1 = __ldg(&wr->L1);
                 const uint4 meta = __ldg(&wr->meta);
-                ny[p] = k < n ? (meta.x >> 14) & 0x7fffu : 0u;
+                ny[p] = k < k_end ? (meta.x >> 14) & 0x7fffu : 0u;
                 // branch-free: every slot computes its range, an empty or
                 // absent one is masked to zero
 #pragma unroll
@@ -310,7 +311,7 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
     add_writes(a.ctr, writes);
 }
 
-template <int S>
+template <int S, int P>
 __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     // With more than two slots the resolve is let in only when this block is
     // done: its blocks waiting on the SMs cost a splat with 40 KB or more of shared
@@ -326,13 +327,20 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     // (the reductions of one value keep it in a uniform register: of the kernel's 64
     // registers one more for the warps costs 96 views 3 %)
     const uint32_t n = __reduce_max_sync(0xffffffffu, a.ctr->n_work);
-    const uint32_t units = (n + 2u * unit_pairs(S) - 1u) / (2u * unit_pairs(S)), wave = 4u * uint32_t(a.sm_count);
-    const uint32_t blocks = min(gridDim.x, wave * (1u + units / (wave * kSplatWarps * kUnitsPerWarp)));
+    const uint32_t wave = 4u * uint32_t(a.sm_count);
+    uint32_t unit = 2u * P;
+    // few points (often large cells, whose units are long): a unit for every warp
+    // (2,048 points of 18,000 pixels over 48 views: 8.2 -> 1.9 ms a frame; of small
+    // cells, 7,000 points at 8 views, 44 -> 47 us)
+    if (S <= 3 && n < 2u * wave * kSplatWarps) unit = min(unit, max(1u, n / (wave * kSplatWarps)));
+    const uint32_t units = (n + unit - 1u) / unit;
+    uint32_t blocks = gridDim.x;
+    if (P == unit_pairs(S)) blocks = min(blocks, wave * (1u + units / (wave * kSplatWarps * kUnitsPerWarp)));
     if (blockIdx.x >= blocks) return;
     __syncthreads();
-    splat_units<S>(a, n, units, __reduce_max_sync(0xffffffffu, blocks * kSplatWarps),
-                   uint32_t(__cvta_generic_to_shared(s_ex)),
-                   reinterpret_cast<SplatWarpSmem<S, unit_pairs(S)>*>(s_dyn)[threadIdx.x >> 5]);
+    splat_units<S, P>(a, n, __reduce_max_sync(0xffffffffu, unit), units, __reduce_max_sync(0xffffffffu, blocks * kSplatWarps),
+                      uint32_t(__cvta_generic_to_shared(s_ex)),
+                      reinterpret_cast<SplatWarpSmem<S, P>*>(s_dyn)[threadIdx.x >> 5]);
     if constexpr (kLate) allow_next_kernel();
 }
 
@@ -504,13 +512,23 @@ __global__ void __launch_bounds__(256) k_resolve_pbr(FrameArgs a) {
 }
 
 // Launch with the per-warp pooling buffers as dynamic shared memory.
+template <int S, int P>
+cudaError_t splat_as(const FrameArgs& a, int grid, cudaStream_t s) {
+    const size_t bytes = kSplatWarps * sizeof(SplatWarpSmem<S, P>);
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(k_splat<S, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+    if (attr != cudaSuccess) return attr;
+    return launch_after_previous(k_splat<S, P>, dim3(grid), dim3(kSplatWarps * 32), bytes, s, a);
+}
+
+// Coarse cells, of a sampling bias of eight pixels and more, fill the passes of
+// small units and make large ones uneven: two pairs (one with more slots) and every
+// block, as 48 views of 420x560 at bias 16: 50,000 points 178 -> 158 us a frame,
+// 310,000 points 369 -> 336. Up to 16 views the large units are as good.
 template <int S>
 cudaError_t splat_one(const FrameArgs& a, int grid, cudaStream_t s) {
-    const size_t bytes = kSplatWarps * sizeof(SplatWarpSmem<S, unit_pairs(S)>);
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_splat<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
-    if (attr != cudaSuccess) return attr;
-    return launch_after_previous(k_splat<S>, dim3(grid), dim3(kSplatWarps * 32), bytes, s, a);
+    if (S > 1 && a.dc.bias_h * a.dc.bias_v >= 8.0f) return splat_as<S, (S == 1 ? unit_pairs(S) : S <= 3 ? 2 : 1)>(a, grid, s);
+    return splat_as<S, unit_pairs(S)>(a, grid, s);
 }
 
 }  // namespace

@@ -35,3 +35,19 @@ def test_views_equal_the_oracles(views, bias):
     g = gpu_frame(d, sc, m, max_points=len(o.points) + 1, panel=False)
     check_sampling(g, o)
     check_views(g, o, views=looked_at)
+
+
+# views, bias, triangles: coarse cells (small units), and fewer points than warps
+@pytest.mark.parametrize("views,bias,n", [(8, 12.0, 2048), (24, 12.0, 2048), (40, 30.0, 2048), (60, 12.0, 600),
+                                          (90, 12.0, 2048), (120, 12.0, 300), (8, 2.0, 3), (40, 2.0, 50), (24, 60.0, 5)])
+def test_few_points_and_coarse_cells(views, bias, n):
+    d = replace(S.display_tiny(), n_views=views, view_w=160, view_h=160, bias_h=bias, bias_v=max(1.0, bias / 4))
+    whole = S.scene_tiny()
+    sc = replace(whole, idx=whole.idx[-n:], tri_tex=whole.tri_tex[-n:])
+    m = S.model_matrix(4)
+    looked_at = sorted({0, views // 2, views - 1})
+    o = O.render(d, sc, m, views=looked_at, panel=False)
+    g = gpu_frame(d, sc, m, max_points=len(o.points) + 1, panel=False)
+    assert len(o.points) > 0
+    check_sampling(g, o)
+    check_views(g, o, views=looked_at)
