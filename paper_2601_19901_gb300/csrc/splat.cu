@@ -15,7 +15,7 @@
 namespace lfdpr {
 namespace {
 
-// A warp takes a unit of 2P consecutive points of the work list: for each of
+// A warp takes a unit of 2P points of the work list, neighbours or spread over it: for each of
 // its P pairs, one half-warp (16 lanes) per point, each lane taking up to S
 // views of the point (views g + 16 s + lane of a group g of 16 S views, S
 // chosen so that one group holds every rendered view where it can).
@@ -58,6 +58,7 @@ constexpr int kSplatWarps = 8;
 // 5,000 triangles at 48 views 125 -> 116 us a frame, at 96 views 201 -> 182; twelve
 // scenes of a batch 2.88 -> 2.77 ms; from 300,000 triangles on the same.
 constexpr uint32_t kUnitsPerWarp = 14;
+constexpr uint32_t kSpreadUnits = 20;   // units a warp of a wave up to which they are spread over the list
 
 // The per-pixel test; every condition is evaluated (no early exits), so the
 // lanes' different candidates do not diverge.
@@ -109,11 +110,12 @@ __device__ __forceinline__ uint32_t div_floor(uint32_t r, uint32_t n) {
 // points share the unit's scan and fill its passes better; more segments take
 // more shared memory and registers, and a small mesh has fewer units to spread.
 // Splat of 10^6 triangles (200 instances), P = 1 for S = 6 and 8, else 2, against
-// these: 8 views (S = 1) 172 -> 104 us, 24 (S = 2) 220 -> 180, 48 (S = 3)
-// 292 -> 265, 96 (S = 6) 557 -> 462. P = 4 for S = 1 gave 121 (and a frame of
+// these: 8 views (S = 1) 172 -> 106 us, 24 (S = 2) 220 -> 181, 48 (S = 3)
+// 292 -> 273, 96 (S = 6) 557 -> 464. P = 4 for S = 1 gave 121 (and a frame of
 // 2,048 triangles 0.4 us less); P = 5 for S = 2 223; P = 4 for S = 3 286 of 283;
 // P = 3 for S = 4 350 of 353 but slower small frames. With S = 8 two pairs would
-// leave an SM three blocks.
+// leave an SM three blocks. (Smaller units for few points, coarse cells and small
+// meshes: see k_splat and splat_one.)
 __host__ __device__ constexpr int unit_pairs(int S) {
     return S == 1 ? 6 : S <= 2 ? 4 : S == 3 ? 3 : S <= 6 ? 2 : 1;
 }
@@ -161,10 +163,12 @@ __device__ __forceinline__ void test_candidate(const DispConst& c, const SplatWa
 
 // The splat proper: n_warps warps stride through the units of the work list's n
 // points. ex_s: shared-memory address of the eye positions.
-template <int S, int P>
-__device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint32_t unit, uint32_t total_units,
-                                            uint32_t n_warps, uint32_t ex_s, SplatWarpSmem<S, P>& sm) {
-    const uint32_t per = S <= 3 ? unit : 2u * P;   // points of a unit
+template <int S, int P, bool kSpread>
+__device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint32_t total_units, uint32_t n_warps,
+                                            uint32_t ex_s, SplatWarpSmem<S, P>& sm) {
+    // unit g: work points 2 P g + q, q < 2 P, or (spread over the list, of which it
+    // may have fewer than 2 P) g + q total_units; those below n
+    const uint32_t A = kSpread ? 1u : 2u * P, B = kSpread ? total_units : 1u;
     const int lane = threadIdx.x & 31, sub = lane & 15, half = lane >> 4;
     const uint32_t lanes_below = (1u << lane) - 1u;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -176,10 +180,9 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
     uint32_t writes = 0;
 
     for (uint32_t g = warp; g < total_units; g += n_warps) {
-        const uint32_t k0 = per * g;   // the unit's first work point, and the end of its points
-        const uint32_t k_end = S <= 3 ? min(n, k0 + per) : n;
+        const uint32_t k0 = A * g;   // the unit's first work point
         {
-            const uint32_t kn = k0 + per * n_warps + uint32_t(lane);   // the next unit's records
+            const uint32_t kn = k0 + A * n_warps + B * uint32_t(lane);   // the next unit's records
             if (lane < 2 * P && kn < n) prefetch_l2(work + kn);
         }
         // the next unit's triangles: read their ids now (the
@@ -188,7 +191,7 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
         // next unit's staging finds them there
         uint32_t next_tri = 0xffffffffu;
         {
-            const uint32_t kn = k0 + per * n_warps + uint32_t(lane);
+            const uint32_t kn = k0 + A * n_warps + B * uint32_t(lane);
             if (lane < 2 * P && kn < n) next_tri = __ldg(&work[kn].meta.z);
         }
         for (int g0 = vlo; g0 < vhi; g0 += 16 * S) {
@@ -207,8 +210,8 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
                 for (int z = 0; z < 10 * P; z += 32) {
                     const int q = (lane + z) / 5, f = lane + z - 5 * q;
                     if (q >= 2 * P) break;
-                    const uint32_t k = k0 + uint32_t(q);
-                    const uint4 meta = __ldg(&work[k < k_end ? k : k0].meta);
+                    const uint32_t k = k0 + B * uint32_t(q);
+                    const uint4 meta = __ldg(&work[k < n ? k : k0].meta);
                     float4 v = __ldg(&a.rec[meta.z].q[f]);
                     if (f < 2) {
                         const uint32_t ij = f == 0 ? meta.y & 0xffffu : meta.y >> 16;
@@ -229,11 +232,11 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
 #pragma unroll
             for (int p = 0; p < P; p++) {
                 // a half past the end takes the unit's first record, with no rows
-                const uint32_t k = k0 + 2u * p + uint32_t(half);
-                const WorkRec* wr = work + (k < k_end ? k : k0);
+                const uint32_t k = k0 + B * uint32_t(2 * p + half);
+                const WorkRec* wr = work + (k < n ? k : k0);
                 const float4 l0 = __ldg(&wr->L0), l1 = __ldg(&wr->L1);
                 const uint4 meta = __ldg(&wr->meta);
-                ny[p] = k < k_end ? (meta.x >> 14) & 0x7fffu : 0u;
+                ny[p] = k < n ? (meta.x >> 14) & 0x7fffu : 0u;
                 // branch-free: every slot computes its range, an empty or
                 // absent one is masked to zero
 #pragma unroll
@@ -334,13 +337,24 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     // cells, 7,000 points at 8 views, 44 -> 47 us)
     if (S <= 3 && n < 2u * wave * kSplatWarps) unit = min(unit, max(1u, n / (wave * kSplatWarps)));
     const uint32_t units = (n + unit - 1u) / unit;
+    // Neighbouring points are alike, and a unit of the coarse ones of a mesh is much
+    // longer than the others: of few units, each takes its points from all over the
+    // list. Of many it takes neighbours, which share triangles. (Meshes of 20,000 and
+    // 110,000 triangles with textures of 256 texels a side: at 16 views 98 -> 72 and
+    // 160 -> 144 us a frame, at 48 views 182 -> 146 and 284 -> 258; 10^6 triangles at
+    // 48 views 572 us with neighbours, 587 with points from all over.)
+    const bool spread = S <= 3 && units <= wave * kSplatWarps * kSpreadUnits;
     uint32_t blocks = gridDim.x;
     if (P == unit_pairs(S)) blocks = min(blocks, wave * (1u + units / (wave * kSplatWarps * kUnitsPerWarp)));
     if (blockIdx.x >= blocks) return;
     __syncthreads();
-    splat_units<S, P>(a, n, __reduce_max_sync(0xffffffffu, unit), units, __reduce_max_sync(0xffffffffu, blocks * kSplatWarps),
-                      uint32_t(__cvta_generic_to_shared(s_ex)),
-                      reinterpret_cast<SplatWarpSmem<S, P>*>(s_dyn)[threadIdx.x >> 5]);
+    const uint32_t n_warps = __reduce_max_sync(0xffffffffu, blocks * kSplatWarps);
+    const uint32_t ex_s = uint32_t(__cvta_generic_to_shared(s_ex));
+    SplatWarpSmem<S, P>& sm = reinterpret_cast<SplatWarpSmem<S, P>*>(s_dyn)[threadIdx.x >> 5];
+    if (S <= 3 && spread)
+        splat_units<S, P, true>(a, n, __reduce_max_sync(0xffffffffu, units), n_warps, ex_s, sm);
+    else
+        splat_units<S, P, false>(a, n, units, n_warps, ex_s, sm);
     if constexpr (kLate) allow_next_kernel();
 }
 
@@ -525,9 +539,17 @@ cudaError_t splat_as(const FrameArgs& a, int grid, cudaStream_t s) {
 // small units and make large ones uneven: two pairs (one with more slots) and every
 // block, as 48 views of 420x560 at bias 16: 50,000 points 178 -> 158 us a frame,
 // 310,000 points 369 -> 336. Up to 16 views the large units are as good.
+// With six slots so do those of meshes below 150,000 triangles, where the points
+// of a unit are too unlike for one of two pairs (82 and 96 views; 110,000 triangles,
+// textures of 256 texels 413 -> 367 and 458 -> 406 us a frame, of up to 4,096 423 ->
+// 447; from 200,000 on two pairs gain: 10^6 triangles 912 -> 836), and with four
+// below 50,000 (60 views, 20,000 triangles: 148 -> 139 and 193 -> 170).
 template <int S>
 cudaError_t splat_one(const FrameArgs& a, int grid, cudaStream_t s) {
-    if (S > 1 && a.dc.bias_h * a.dc.bias_v >= 8.0f) return splat_as<S, (S == 1 ? unit_pairs(S) : S <= 3 ? 2 : 1)>(a, grid, s);
+    constexpr int kFew = S <= 3 ? 2 : 1;
+    if (S > 1 && a.dc.bias_h * a.dc.bias_v >= 8.0f) return splat_as<S, (S == 1 ? unit_pairs(S) : kFew)>(a, grid, s);
+    if ((S == 6 && a.n_tris < 150000u) || (S == 4 && a.n_tris < 50000u))
+        return splat_as<S, (S == 4 || S == 6 ? kFew : unit_pairs(S))>(a, grid, s);
     return splat_as<S, unit_pairs(S)>(a, grid, s);
 }
 

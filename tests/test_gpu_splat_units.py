@@ -26,7 +26,7 @@ def _lib():
 # views, horizontal sampling bias (lower: more points)
 @pytest.mark.parametrize("views,bias", [(1, 2.0), (16, 2.0), (17, 2.0), (32, 4.0), (33, 2.0), (48, 4.0), (49, 2.0),
                                         (64, 4.0), (65, 4.0), (96, 2.0), (97, 4.0), (128, 4.0), (16, 0.05),
-                                        (33, 0.08), (96, 0.1)])
+                                        (33, 0.08), (96, 0.1), (8, 0.12), (24, 0.2), (48, 0.25), (60, 0.2)])
 def test_views_equal_the_oracles(views, bias):
     d = replace(S.display_tiny(), n_views=views, view_w=96, view_h=96, bias_h=bias, bias_v=min(bias, 1.0))
     sc, m = S.scene_tiny(), S.model_matrix(4)
