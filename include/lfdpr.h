@@ -76,7 +76,7 @@ typedef enum {
  * interleaving (for recon 2 and 3: the reconstruction one view away). max_points is the point-buffer
  * capacity (0 = 1 << 23); each point of capacity takes 100 B of device
  * memory (the 16-B point record, a 48-B splat work record, a 4-B near-list
- * entry and a 32-B resolve record), and 8 B more once a mesh of materials is
+ * entry and a 32-B resolve record), and 40 B more once a mesh of materials is
  * uploaded to the display.
  */
 typedef struct {
@@ -455,18 +455,17 @@ lfdpr_status lfdpr_set_shading(lfdpr_display *disp, const lfdpr_shading *shading
  * Batched frames: n (display, mesh) scenes, each with its own display (view
  * count, view size, panel), rendered and interleaved together. One call runs
  * every scene's frame, Sec. 3.1-4 as lfdpr_render_frame followed by
- * lfdpr_interleave, as one CUDA graph: per-scene set-up, scan, emission and
- * fetch on `branches` concurrent graph branches, then one persistent splat
- * launch over the point pairs of all scenes, then per-scene resolve and
- * interleave into each display's own panel buffer (lfdpr_batch_panel). The
+ * lfdpr_interleave, as one CUDA graph: the scenes' frames on `branches`
+ * concurrent graph branches (scene i on branch i mod branches), each
+ * interleaved into its display's own panel buffer (lfdpr_batch_panel). The
  * graph is captured on the first lfdpr_render_batch after creation or a
  * configuration change; later calls replay it with new model matrices. Each
  * scene's views, keys and panel are bit-identical to rendering it alone.
  */
 typedef struct {
-    int32_t branches;             /* concurrent graph branches for the per-scene stages, 1..32 */
-    int32_t splat_blocks_per_sm;  /* persistent splat grid: blocks of 256 threads per SM, 1..64 */
-    int32_t splat_slots;          /* views per lane in the splat: 1, 2, 3, 4, 6 or 8 */
+    int32_t branches;             /* concurrent graph branches, 1..32 */
+    int32_t splat_blocks_per_sm;  /* splat grid: blocks of 256 threads per SM, 1..64 */
+    int32_t splat_slots;          /* most views per lane in the splat: 1, 2, 3, 4, 6 or 8 */
 } lfdpr_batch_config;
 
 /*

@@ -1,9 +1,7 @@
 // Batched frames (lfdpr_create_batch ... lfdpr_batch_panel in include/lfdpr.h):
 // several (display, mesh) scenes of uneven size rendered and interleaved by
-// one CUDA graph. The per-scene stages up to the key clear (Sec. 3.1, 3.3) run
-// on concurrent graph branches, one persistent launch splats the point pairs
-// of every scene (Sec. 3.2), and per-scene resolve (Eq. 8-9) and interleave
-// (Sec. 4) follow on the branches. Each scene runs exactly the kernels and
+// one CUDA graph: each scene's frame, from set-up (Sec. 3.1) to interleave
+// (Sec. 4), on one of the concurrent branches. Each scene runs exactly the kernels and
 // arithmetic of lfdpr_render_frame + lfdpr_interleave, so its keys, views and
 // panel are bit-identical to rendering it alone; the model matrices come from
 // device memory so one captured graph replays every frame.
