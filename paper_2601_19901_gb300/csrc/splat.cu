@@ -525,13 +525,17 @@ __global__ void __launch_bounds__(256) k_resolve_pbr(FrameArgs a) {
     reinterpret_cast<uint32_t*>(a.views)[o] = out;
 }
 
-// Launch with the per-warp pooling buffers as dynamic shared memory.
+// Launch with the per-warp pooling buffers as dynamic shared memory. Beyond 48 KB
+// (with the kernel's eye positions) the launch needs the attribute, which holds for
+// the current device only: it is set at every such launch.
 template <int S, int P>
 cudaError_t splat_as(const FrameArgs& a, int grid, cudaStream_t s) {
-    const size_t bytes = kSplatWarps * sizeof(SplatWarpSmem<S, P>);
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_splat<S, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
-    if (attr != cudaSuccess) return attr;
+    constexpr size_t bytes = kSplatWarps * sizeof(SplatWarpSmem<S, P>);
+    if (bytes + sizeof(float) * kMaxRenderViews > 48u * 1024u) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k_splat<S, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+        if (e != cudaSuccess) return e;
+    }
     return launch_after_previous(k_splat<S, P>, dim3(grid), dim3(kSplatWarps * 32), bytes, s, a);
 }
 

@@ -1,0 +1,79 @@
+// The library's launch code (its own objects) against the stand-in runtime of
+// fake_cudart.cpp; needs no GPU. Prints the failed checks and returns their number.
+#include <cstdio>
+#include <cstring>
+
+#include "fake_cudart.h"
+#include "objects.h"
+
+namespace {
+int g_failed = 0;
+
+void check(bool ok, const char* what) {
+    if (ok) return;
+    printf("failed: %s\n", what);
+    g_failed++;
+}
+}  // namespace
+
+namespace lfdpr {
+thread_local char g_last_error[512];
+lfdpr_status fail(lfdpr_status s, const char*, ...) { return s; }
+lfdpr_status cuda_fail(cudaError_t, const char*) { return LFDPR_ECUDA; }
+}  // namespace lfdpr
+
+using namespace lfdpr;
+
+static cudaError_t splat(int views, uint32_t tris) {
+    FrameArgs a{};
+    a.n_tris = tris;
+    a.sm_count = 152;
+    a.dc.bias_h = a.dc.bias_v = 1.0f;
+    a.dc.nr = a.view_hi = views;
+    return launch_splat(a, nullptr);
+}
+
+static cudaError_t interleave(int recon, int n, int w, int panel_w) {
+    DispConst c{};
+    c.recon = recon;
+    c.n_views = n;
+    c.nr = recon == 1 ? 2 * n : n;
+    c.W = w;
+    c.H = 64;
+    c.Wp = panel_w;
+    c.Hp = 64;
+    c.inv_pitch = 0.125f;
+    return launch_interleave(c, nullptr, nullptr, nullptr, 0, nullptr, nullptr);
+}
+
+static cudaError_t warp(int w) { return launch_warp_views(nullptr, nullptr, nullptr, 2, nullptr, 4, w, 64, 1.0f, nullptr, 1, nullptr); }
+
+// every number of view slots a lane, and both unit sizes, on one device and then another
+static void devices() {
+    for (int dev = 0; dev < 2; dev++) {
+        g_device = dev;
+        for (int views : {1, 32, 48, 64, 96, 128})
+            for (uint32_t tris : {1000u, 1000000u}) {
+                char what[96];
+                snprintf(what, sizeof what, "splat of %d views, %u triangles on device %d", views, tris, dev);
+                check(splat(views, tris) == cudaSuccess, what);
+            }
+        check(interleave(0, 48, 420, 1000) == cudaSuccess && interleave(1, 48, 420, 1000) == cudaSuccess, "interleave");
+        check(warp(4032) == cudaSuccess, "warp");
+    }
+}
+
+// a call after a failed one
+static void retry() {
+    g_fail_attributes = 1;
+    splat(96, 1000000u);
+    g_fail_attributes = 0;
+    check(splat(96, 1000000u) == cudaSuccess, "splat after a failed attribute call");
+}
+
+int main(int, char** argv) {
+    if (!strcmp(argv[1], "devices")) devices();
+    if (!strcmp(argv[1], "retry")) retry();
+    check(g_launched > 0, "something was launched");
+    return g_failed;
+}
