@@ -774,7 +774,8 @@ cudaError_t launch_interleave(const DispConst& dc, const uint8_t* views, const f
     if (bytes <= smem_max / 2) {
         const auto kernel = !tent ? k_interleave_tile
                             : dc.xtalk > 0.0f ? k_interleave_tent<true> : k_interleave_tent<false>;
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+        // the most that a tile takes, not this one's: another thread's tile may need more
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max / 2);
         if (e != cudaSuccess) return e;
         return launch_after_previous(kernel, dim3((dc.Wp + cols - 1) / cols, dc.H), dim3(tent ? kTentThreads : kTileThreads),
                                      size_t(bytes), s,

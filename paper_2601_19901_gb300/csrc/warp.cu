@@ -286,7 +286,9 @@ cudaError_t launch_warp_views(const uint8_t* views, const uint64_t* keys, const 
                                          cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     if (smem > 48u * 1024u) {
-        e = cudaFuncSetAttribute(k_warp_views, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        // the most that a row takes, not this one's: another thread's views may be wider
+        e = cudaFuncSetAttribute(k_warp_views, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 int(warp_smem(kMaxRenderViews, kMaxRenderViews, kMaxWarpWidth)));
         if (e != cudaSuccess) return e;
     }
     WarpArgs a{views, keys, in_eyes, out_eyes, nin, nout, W, H, ipw, out};

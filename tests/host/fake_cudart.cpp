@@ -11,6 +11,7 @@
 
 int g_device = 0;
 int g_fail_attributes = 0;
+void (*g_meanwhile)() = nullptr;
 int g_launched = 0;
 
 namespace {
@@ -45,7 +46,13 @@ cudaError_t cudaFuncSetAttribute(const void* kernel, cudaFuncAttribute a, int v)
         g_fail_attributes--;
         return cudaErrorMemoryAllocation;
     }
-    if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) g_limit[{kernel, g_device}] = v;
+    if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) {
+        g_limit[{kernel, g_device}] = v;
+        if (void (*other)() = g_meanwhile) {
+            g_meanwhile = nullptr;
+            other();
+        }
+    }
     return cudaSuccess;
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* kernel, void**) {

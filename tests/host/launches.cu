@@ -71,9 +71,21 @@ static void retry() {
     check(splat(96, 1000000u) == cudaSuccess, "splat after a failed attribute call");
 }
 
+// two threads' displays of different sizes: the smaller one's call between the
+// larger one's attribute and its launch
+static void threads() {
+    g_meanwhile = [] { check(interleave(0, 4, 420, 2560) == cudaSuccess, "small tile"); };
+    check(interleave(0, 48, 420, 1000) == cudaSuccess, "large tile beside a small one");
+    g_meanwhile = [] { check(interleave(1, 4, 420, 2560) == cudaSuccess, "small tent tile"); };
+    check(interleave(1, 48, 420, 1000) == cudaSuccess, "large tent tile beside a small one");
+    g_meanwhile = [] { check(warp(1200) == cudaSuccess, "narrow warp"); };
+    check(warp(4000) == cudaSuccess, "wide warp beside a narrow one");
+}
+
 int main(int, char** argv) {
     if (!strcmp(argv[1], "devices")) devices();
     if (!strcmp(argv[1], "retry")) retry();
+    if (!strcmp(argv[1], "threads")) threads();
     check(g_launched > 0, "something was launched");
     return g_failed;
 }

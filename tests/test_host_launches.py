@@ -23,7 +23,7 @@ def program(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("what", ["devices", "retry"])
+@pytest.mark.parametrize("what", ["devices", "retry", "threads"])
 def test_shared_memory_is_allowed_where_a_launch_needs_it(program, what):
     r = subprocess.run([program, what], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout
