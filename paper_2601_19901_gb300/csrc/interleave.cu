@@ -634,8 +634,9 @@ int gauss_stride(const DispConst& c) {
         int last_view = -1, last_line = -1;
         for (int l = 0; l < 32; l++) {
             const double ph = double(l) * S * double(c.inv_pitch);
-            // half a view up, so that a stride of whole periods stays in one view whatever its rounding
-            const int view = int((ph - std::floor(ph)) * c.nr + 0.5) % c.nr;
+            // half a view up, so that a stride of whole periods stays in one view whatever its
+            // rounding; no number where the pitch's reciprocal overflows
+            const int view = std::isfinite(ph) ? int((ph - std::floor(ph)) * c.nr + 0.5) % c.nr : 0;
             const int line = int(double(l) * S * c.W / c.Wp) / 32;
             lines += view != last_view || line != last_line;
             last_view = view;

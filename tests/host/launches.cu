@@ -1,5 +1,6 @@
 // The library's launch code (its own objects) against the stand-in runtime of
 // fake_cudart.cpp; needs no GPU. Prints the failed checks and returns their number.
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 
@@ -46,6 +47,20 @@ static cudaError_t interleave(int recon, int n, int w, int panel_w) {
     return launch_interleave(c, nullptr, nullptr, nullptr, 0, nullptr, nullptr);
 }
 
+// a lens pitch whose reciprocal overflows: the lens phase is no number
+static void tiny_pitch() {
+    for (int recon : {2, 3}) {
+        DispConst c{};
+        c.recon = recon;
+        c.n_views = 8;
+        c.nr = recon == 2 ? 16 : 8;
+        c.W = c.H = 64;
+        c.Wp = c.Hp = 200;
+        c.inv_pitch = INFINITY;
+        check(launch_interleave(c, nullptr, nullptr, nullptr, 1, nullptr, nullptr) == cudaSuccess, "tiny pitch");
+    }
+}
+
 static cudaError_t warp(int w) { return launch_warp_views(nullptr, nullptr, nullptr, 2, nullptr, 4, w, 64, 1.0f, nullptr, 1, nullptr); }
 
 // every number of view slots a lane, and both unit sizes, on one device and then another
@@ -86,6 +101,7 @@ int main(int, char** argv) {
     if (!strcmp(argv[1], "devices")) devices();
     if (!strcmp(argv[1], "retry")) retry();
     if (!strcmp(argv[1], "threads")) threads();
+    if (!strcmp(argv[1], "tiny_pitch")) tiny_pitch();
     check(g_launched > 0, "something was launched");
     return g_failed;
 }
