@@ -267,14 +267,12 @@ __global__ void __launch_bounds__(kTentThreads, 10) k_interleave_tent(DispConst 
     const int xg = x0 + 4 * threadIdx.x;
     if (xg >= x1) return;
     const float xc4 = 0.25f * c.xtalk_c, x4 = 0.25f * c.xtalk;
-    const uint32_t pitch = 4u * uint32_t(stride), s0 = uint32_t(__cvta_generic_to_shared(s_tent));
-    const uint32_t view0 = s0 + uint32_t(N + 2) * pitch;
+    const uint32_t pitch = 4u * uint32_t(stride), view0 = uint32_t(N + 2) * pitch;
     // four times the display view in row `at` of the words (column and channel
-    // as given); view 0's are the binary32 ones
+    // as given, byte offsets); view 0's are the binary32 ones
     auto value4 = [&](uint32_t at, uint32_t col, int ch, bool first) -> float {
-        const uint32_t addr = first ? view0 + uint32_t(ch) * pitch + col : at;
-        uint32_t w;
-        asm("ld.shared.u32 %0, [%1];" : "=r"(w) : "r"(addr));
+        const uint32_t off = first ? view0 + uint32_t(ch) * pitch + col : at;
+        const uint32_t w = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(s_tent) + off);
         // 2^23 + the sum, by its bits
         const float t = __uint_as_float(((w >> (10 * ch)) & 0x3ffu) | 0x4b000000u) - 8388608.0f;
         return first ? __uint_as_float(w) : t;
@@ -290,7 +288,7 @@ __global__ void __launch_bounds__(kTentThreads, 10) k_interleave_tent(DispConst 
 #pragma unroll
             for (int ch = 0; ch < 3; ch++) {
                 const int k = view_of_subpixel(c, xg + e, y, ch);
-                const uint32_t at = s0 + col[e] + uint32_t(k) * pitch;   // view k - 1's row
+                const uint32_t at = col[e] + uint32_t(k) * pitch;   // view k - 1's row
                 float val;
                 if constexpr (XT) {
                     val = value4(at + pitch, col[e], ch, k == 0) * xc4;
@@ -432,7 +430,7 @@ constexpr float kGaussApart = 0x1p-12f;
 constexpr int kGaussSteps = 16;
 constexpr int kGaussMaxStride = 64;    // largest column stride between a warp's lanes
 
-struct GaussBin {
+struct __align__(8) GaussBin {
     float from;       // the next view's bytes start here (+inf: not in this bin)
     uint32_t off;     // byte offset of the bin's first view
 };
@@ -468,9 +466,8 @@ __device__ __forceinline__ bool gauss_bin(const float* pos, int nr, float r, int
     return step < kGaussSteps;
 }
 
-// Panel pixel (x, y) as gauss_pixel, its views found in the table at shared
-// address bins (less the bias of the bin number below): the same view bytes,
-// summed as integers (exact, as the sums of at most 32 bytes are in binary32).
+// Panel pixel (x, y) as gauss_pixel, its views found in the table (bins, in
+// shared memory): the same view bytes, summed as integers (exact, as the sums of at most 32 bytes are in binary32).
 // The bin number is floor(8 a) + 32, the low bits of one fma rounded down
 // onto 1.5 2^23. mean: 1 / ns where ns is a power of two (the product is then
 // the quotient), else 0.
@@ -478,7 +475,7 @@ constexpr float kGaussMagic = 12582912.0f;              // 1.5 2^23
 constexpr uint32_t kGaussMagicBits = 0x4b400000u;
 template <bool XT>
 __device__ __forceinline__ uint32_t gauss_pixel_table(const DispConst& c, const uint8_t* __restrict__ views,
-                                                      uint32_t bins, uint32_t view_bytes, const float4* smp, int ns,
+                                                      const GaussBin* bins, uint32_t view_bytes, const float4* smp, int ns,
                                                       float mean, int x, int y, float sxw, float syh) {
     constexpr int K = XT ? 3 : 1;
     const int W = c.W, H = c.H;
@@ -514,10 +511,9 @@ __device__ __forceinline__ uint32_t gauss_pixel_table(const DispConst& c, const 
             for (int k = 0; k < K; k++) {
                 const float a = phi[ch][k] + q.z;
                 const uint32_t n = __float_as_uint(__fmaf_rd(a, float(kGaussBins), kGaussMagic + float(kGaussBins * kGaussMargin)));
-                float from;
-                uint32_t off;
-                asm("ld.shared.v2.b32 {%0, %1}, [%2];" : "=f"(from), "=r"(off) : "r"(bins + 8u * n));
-                if (a >= from) off += view_bytes;
+                const GaussBin b = bins[n - kGaussMagicBits];
+                uint32_t off = b.off;
+                if (a >= b.from) off += view_bytes;
                 uint64_t p;   // at + off in one instruction
                 asm("mad.wide.u32 %0, %1, 1, %2;" : "=l"(p) : "r"(off), "l"(at));
                 acc[ch][k] += __ldg(reinterpret_cast<const uint8_t*>(p) + ch);
@@ -589,7 +585,6 @@ __global__ void __launch_bounds__(kGaussThreads, 4) k_interleave_gauss(DispConst
         s_bins[b] = o;
     }
     slow = __syncthreads_or(slow);
-    const uint32_t bins = uint32_t(__cvta_generic_to_shared(s_bins)) - 8u * kGaussMagicBits;
     const float mean = (ns & (ns - 1)) == 0 ? 1.0f / float(ns) : 0.0f;
     const float sxw = float(c.W) / float(c.Wp), syh = float(c.H) / float(c.Hp);
     const uint32_t* v32 = reinterpret_cast<const uint32_t*>(views);
@@ -613,7 +608,7 @@ __global__ void __launch_bounds__(kGaussThreads, 4) k_interleave_gauss(DispConst
                 exact |= !(p0 >= 0.0f && p0 <= float(c.n_views));
             }
             row[j + S * lane] = exact ? gauss_pixel(c, v32, s_pos, s_smp, ns, x, y, sxw, syh)
-                                      : gauss_pixel_table<XT>(c, views, bins, view_bytes, s_smp4, ns, mean, x, y, sxw, syh);
+                                      : gauss_pixel_table<XT>(c, views, s_bins, view_bytes, s_smp4, ns, mean, x, y, sxw, syh);
         }
         __syncthreads();   // the row is complete; the other buffer's readers are past their barrier
         uint32_t* dst = reinterpret_cast<uint32_t*>(panel) + (uint64_t)y * c.Wp + x0;

@@ -125,7 +125,8 @@ struct MatRec {
     uint4 b;      // tangent y and z bits, normal tv_min RGB | bitangent sign << 24, normal tv_max
 };
 
-// The 32 bytes at p (32-byte aligned, not written by the running kernel).
+// The 32 bytes at p (32-byte aligned, not written by the running kernel, p from a
+// value loaded after its wait_previous_kernel: the statement is ordered by p alone).
 __device__ __forceinline__ void load32(const void* p, float4& a, uint4& b) {
     asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
