@@ -11,7 +11,8 @@
 // coalesced loads, then forms every panel row that samples that view row,
 // one thread per 4 adjacent panel pixels and one 16-byte store per row.
 // k_interleave_tent stages the tent's display views instead.
-// k_interleave (the direct gather) serves displays whose tile would not fit.
+// k_interleave (the direct gather) serves displays whose tile would not fit, or
+// of whose view pixels the panel shows too few (tent_pays).
 // k_interleave_gauss is the Gaussian reconstruction of Sec. 4 (recon 2, 3):
 // per subpixel the mean of the caller's samples, each the nearest rendered
 // view to the subpixel's phase plus the sample's angular offset at the view
@@ -647,6 +648,26 @@ int gauss_stride(const DispConst& c) {
     return best;
 }
 
+// Whether the tent's tiles, of `bytes` of shared memory and `blocks` in all, are
+// faster than the direct gather. The tiles stage every rendered view's rows,
+// whatever share of them the panel shows: they pay with the panel pixels per view
+// pixel staged, and with the blocks that an SM holds to cover each other's staging
+// (128 threads each, 10 at most); less where a staged row feeds one panel row.
+// Over seventeen pairs of view and panel sizes and 1 to 256 views, tiles against
+// gather: with crosstalk (nine views a pixel to gather instead of three) 48 views
+// of 420x560 to 2560x1600 46 against 172 us, 128 123 against 179, 200 280 against
+// 186, 96 of 333x251 to 1277x719 45 against 36; without, 48 39 against 68, 96 90
+// against 73, 256 466 against 76, 48 of 640x480 to 640x480 108 against 11. At the
+// lines they are mostly within a fifth of each other. Without crosstalk a panel of
+// few tiles (100x50 to 400x2000) is left to the gather too, 12.7 against 15.8.
+bool tent_pays(const DispConst& c, int64_t bytes, int64_t blocks, int sms, int smem_sm) {
+    const double shown = double(c.Wp) * c.Hp / (double(c.nr) * c.W * std::min(c.H, c.Hp));
+    const double resident = double(std::min<int64_t>(10, smem_sm / (bytes + 1024)));
+    const bool xt = c.xtalk > 0.0f;
+    const double line = c.Hp > c.H ? (xt ? 1.25 : 7.9) : (xt ? 15.0 : 60.0);
+    return shown * resident * resident >= line && (xt || 2 * blocks >= sms);
+}
+
 }  // namespace
 
 namespace {
@@ -744,10 +765,11 @@ cudaError_t launch_view_mip(const uint8_t* views, int W, int H, int nr, int leve
 
 cudaError_t launch_interleave(const DispConst& dc, const uint8_t* views, const float* pos, const float* samples,
                               int n_samples, uint8_t* panel, cudaStream_t s) {
-    int dev = 0, sms = 0, smem_max = 0;
+    int dev = 0, sms = 0, smem_max = 0, smem_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     if (dc.recon == 2 || dc.recon == 3) {
         if (n_samples < 1 || n_samples > 32) return cudaErrorInvalidValue;
         const int S = gauss_stride(dc);
@@ -767,15 +789,15 @@ cudaError_t launch_interleave(const DispConst& dc, const uint8_t* views, const f
     const int cols = tent ? kTentCols : kTileCols;
     const int64_t seg = ((int64_t)(cols - 1) * dc.W) / dc.Wp + 2;
     const int64_t words = tent ? dc.n_views + 5 : dc.nr, bytes = words * seg * 4;
-    if (bytes <= smem_max / 2) {
+    const dim3 tiles((dc.Wp + cols - 1) / cols, dc.H);
+    if (bytes <= smem_max / 2 && (!tent || tent_pays(dc, bytes, int64_t(tiles.x) * tiles.y, sms, smem_sm))) {
         const auto kernel = !tent ? k_interleave_tile
                             : dc.xtalk > 0.0f ? k_interleave_tent<true> : k_interleave_tent<false>;
         // the most that a tile takes, not this one's: another thread's tile may need more
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max / 2);
         if (e != cudaSuccess) return e;
-        return launch_after_previous(kernel, dim3((dc.Wp + cols - 1) / cols, dc.H), dim3(tent ? kTentThreads : kTileThreads),
-                                     size_t(bytes), s,
-                                     dc, views, panel, cols, int(seg));
+        return launch_after_previous(kernel, tiles, dim3(tent ? kTentThreads : kTileThreads), size_t(bytes), s, dc, views,
+                                     panel, cols, int(seg));
     }
     return launch_after_previous(k_interleave, dim3(sms * 8), dim3(256), 0, s, dc, views, panel);
 }

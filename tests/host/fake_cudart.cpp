@@ -13,15 +13,19 @@ int g_device = 0;
 int g_fail_attributes = 0;
 void (*g_meanwhile)() = nullptr;
 int g_launched = 0;
+size_t g_last_smem = 0;
+unsigned g_last_blocks = 0;
 
 namespace {
 cudaError_t g_last = cudaSuccess;
 
 std::map<std::pair<const void*, int>, int> g_limit;   // (kernel, device) -> bytes allowed
-cudaError_t launch(const void* kernel, size_t smem) {
+cudaError_t launch(const void* kernel, dim3 grid, size_t smem) {
     const auto it = g_limit.find({kernel, g_device});
     if (smem > size_t(it == g_limit.end() ? 48 * 1024 : it->second)) return g_last = cudaErrorInvalidValue;
     g_launched++;
+    g_last_smem = smem;
+    g_last_blocks = grid.x * grid.y;
     return cudaSuccess;
 }
 
@@ -38,7 +42,10 @@ cudaError_t cudaGetLastError() {
     return e;
 }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
-    *v = a == cudaDevAttrMultiProcessorCount ? 152 : a == cudaDevAttrMaxSharedMemoryPerBlockOptin ? 227 * 1024 : 0;
+    *v = a == cudaDevAttrMultiProcessorCount                ? 152
+         : a == cudaDevAttrMaxSharedMemoryPerBlockOptin       ? 227 * 1024
+         : a == cudaDevAttrMaxSharedMemoryPerMultiprocessor ? 228 * 1024
+                                                              : 0;
     return cudaSuccess;
 }
 cudaError_t cudaFuncSetAttribute(const void* kernel, cudaFuncAttribute a, int v) {
@@ -56,14 +63,14 @@ cudaError_t cudaFuncSetAttribute(const void* kernel, cudaFuncAttribute a, int v)
     return cudaSuccess;
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* kernel, void**) {
-    return launch(kernel, c->dynamicSmemBytes);
+    return launch(kernel, c->gridDim, c->dynamicSmemBytes);
 }
 cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) {
     memcpy(k, &f, sizeof f);
     return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void**, size_t smem, cudaStream_t) {
-    return launch(reinterpret_cast<const void*>(k), smem);
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void**, size_t smem, cudaStream_t) {
+    return launch(reinterpret_cast<const void*>(k), grid, smem);
 }
 unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t smem, struct CUstream_st* s) {
     g_grid = g, g_block = b, g_smem = smem, g_stream = s;

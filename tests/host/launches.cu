@@ -34,28 +34,54 @@ static cudaError_t splat(int views, uint32_t tris) {
     return launch_splat(a, nullptr);
 }
 
-static cudaError_t interleave(int recon, int n, int w, int panel_w) {
+static DispConst display(int recon, int n, int w, int h, int panel_w, int panel_h, float xtalk) {
     DispConst c{};
     c.recon = recon;
     c.n_views = n;
-    c.nr = recon == 1 ? 2 * n : n;
+    c.nr = recon == 1 || recon == 2 ? 2 * n : n;
     c.W = w;
-    c.H = 64;
+    c.H = h;
     c.Wp = panel_w;
-    c.Hp = 64;
+    c.Hp = panel_h;
     c.inv_pitch = 0.125f;
-    return launch_interleave(c, nullptr, nullptr, nullptr, 0, nullptr, nullptr);
+    c.xtalk = xtalk;
+    return c;
+}
+
+static cudaError_t interleave(int recon, int n, int w, int panel_w) {
+    return launch_interleave(display(recon, n, w, 64, panel_w, 640, 0.15f), nullptr, nullptr, nullptr, 0, nullptr, nullptr);
+}
+
+// which form a tent interleave takes: tiles (dynamic shared memory) or the gather
+static void tent() {
+    const struct {
+        int n, w, h, pw, ph;
+        float xtalk;
+        bool tiles;
+    } cases[] = {{1, 420, 560, 2560, 1600, 0.0f, true},     {48, 420, 560, 2560, 1600, 0.0f, true},
+                 {96, 420, 560, 2560, 1600, 0.0f, false},   {256, 420, 560, 2560, 1600, 0.0f, false},
+                 {128, 420, 560, 2560, 1600, 0.15f, true},  {256, 420, 560, 2560, 1600, 0.15f, false},
+                 {24, 333, 251, 1277, 719, 0.0f, true},     {64, 333, 251, 1277, 719, 0.0f, false},
+                 {64, 333, 251, 1277, 719, 0.15f, true},    {96, 333, 251, 1277, 719, 0.15f, false},
+                 {1, 640, 480, 640, 480, 0.0f, false},      {48, 640, 480, 640, 480, 0.15f, false},
+                 {2, 1200, 300, 200, 200, 0.0f, false},     {8, 128, 128, 512, 512, 0.0f, true},
+                 {12, 840, 1120, 2560, 1600, 0.0f, true},   {64, 840, 1120, 2560, 1600, 0.15f, false},
+                 {128, 100, 50, 400, 2000, 0.0f, false},    {8, 120, 640, 2560, 300, 0.0f, true},
+                 {48, 120, 640, 2560, 300, 0.15f, true},    {48, 480, 360, 1920, 1080, 0.0f, true},    {8, 160, 120, 3840, 2160, 0.0f, true}};
+    for (const auto& k : cases) {
+        char what[96];
+        snprintf(what, sizeof what, "%d views of %dx%d to %dx%d, crosstalk %g", k.n, k.w, k.h, k.pw, k.ph, k.xtalk);
+        check(launch_interleave(display(1, k.n, k.w, k.h, k.pw, k.ph, k.xtalk), nullptr, nullptr, nullptr, 0, nullptr,
+                                nullptr) == cudaSuccess &&
+                  (g_last_smem > 0) == k.tiles,
+              what);
+    }
 }
 
 // a lens pitch whose reciprocal overflows: the lens phase is no number
 static void tiny_pitch() {
     for (int recon : {2, 3}) {
-        DispConst c{};
-        c.recon = recon;
-        c.n_views = 8;
-        c.nr = recon == 2 ? 16 : 8;
-        c.W = c.H = 64;
-        c.Wp = c.Hp = 200;
+        DispConst c = display(recon, 8, 64, 64, 200, 200, 0.0f);
         c.inv_pitch = INFINITY;
         check(launch_interleave(c, nullptr, nullptr, nullptr, 1, nullptr, nullptr) == cudaSuccess, "tiny pitch");
     }
@@ -73,7 +99,7 @@ static void devices() {
                 snprintf(what, sizeof what, "splat of %d views, %u triangles on device %d", views, tris, dev);
                 check(splat(views, tris) == cudaSuccess, what);
             }
-        check(interleave(0, 48, 420, 1000) == cudaSuccess && interleave(1, 48, 420, 1000) == cudaSuccess, "interleave");
+        check(interleave(0, 48, 420, 1000) == cudaSuccess && interleave(1, 100, 240, 1000) == cudaSuccess, "interleave");
         check(warp(4032) == cudaSuccess, "warp");
     }
 }
@@ -92,7 +118,7 @@ static void threads() {
     g_meanwhile = [] { check(interleave(0, 4, 420, 2560) == cudaSuccess, "small tile"); };
     check(interleave(0, 48, 420, 1000) == cudaSuccess, "large tile beside a small one");
     g_meanwhile = [] { check(interleave(1, 4, 420, 2560) == cudaSuccess, "small tent tile"); };
-    check(interleave(1, 48, 420, 1000) == cudaSuccess, "large tent tile beside a small one");
+    check(interleave(1, 100, 240, 1000) == cudaSuccess, "large tent tile beside a small one");
     g_meanwhile = [] { check(warp(1200) == cudaSuccess, "narrow warp"); };
     check(warp(4000) == cudaSuccess, "wide warp beside a narrow one");
 }
@@ -102,6 +128,7 @@ int main(int, char** argv) {
     if (!strcmp(argv[1], "retry")) retry();
     if (!strcmp(argv[1], "threads")) threads();
     if (!strcmp(argv[1], "tiny_pitch")) tiny_pitch();
+    if (!strcmp(argv[1], "tent")) tent();
     check(g_launched > 0, "something was launched");
     return g_failed;
 }

@@ -1,0 +1,36 @@
+"""The interleave's forms on either side of the rules that choose between them,
+byte for byte against the oracle on views of random bytes: the tent's tiles
+(panels of many rows a view row) and the gather, with and without crosstalk.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+from test_gpu_interleave import _display, _lib, _panel, _views  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+# (views, view w, h, panel w, h, pitch, slant, recon, crosstalk)
+TENT = [(48, 42, 9, 512, 33, 8.0, 0.2, 1, 0.15),          # tiles: one whole strip of panel columns
+        (48, 42, 9, 513, 34, 8.0, 0.2, 1, 0.15),          # two, uneven
+        (37, 33, 25, 1277, 131, 5.3, 1.0 / 6.0, 1, 0.2),
+        (24, 33, 80, 1277, 200, 5.3, 1.0 / 6.0, 1, 0.0),
+        (8, 16, 90, 514, 270, 8.0, -0.2, 1, 0.0),
+        (1, 40, 90, 515, 200, 2.5, 0.1, 1, 0.4),          # one view, whose neighbours are itself
+        (1, 40, 90, 515, 200, 2.5, 0.1, 1, 0.0),
+        (2, 40, 90, 515, 200, 2.5, 0.1, 1, 0.4),
+        (3, 40, 90, 515, 200, 2.5, 0.1, 1, 0.4),
+        (256, 12, 9, 260, 200, 9.0, 0.2, 1, 0.15),        # the most views
+        (100, 240, 8, 1000, 80, 8.0, 0.2, 1, 0.15),       # more than 48 KB of shared memory
+        (4, 12, 200, 1030, 100, 8.0, 0.2, 1, 0.15),       # tiles of one panel row
+        (4, 12, 200, 1030, 100, 8.0, 0.2, 1, 0.0),
+        (48, 42, 56, 512, 56, 8.0, 0.2, 1, 0.15),         # gather: a panel row per view row
+        (96, 42, 56, 512, 120, 8.0, 0.2, 1, 0.0),         # gather: many views a panel pixel
+        (200, 42, 20, 256, 60, 8.0, 0.2, 1, 0.15)]
+
+
+@pytest.mark.parametrize("case", range(len(TENT)))
+def test_tent_matches_oracle(case):
+    d = _display(*TENT[case])
+    views = _views(d, 80 + case)
+    assert np.array_equal(_panel(d, views), O.interleave(d, views))

@@ -34,6 +34,11 @@ def test_shared_memory_is_allowed_where_a_launch_needs_it(program, what):
     assert r.returncode == 0, r.stdout
 
 
+def test_the_tent_takes_tiles_where_they_are_faster(program):
+    r = subprocess.run([program, "tent"], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout
+
+
 def test_a_phase_that_is_no_number_is_not_made_an_integer(tmp_path):
     """With the host code's float to integer conversions checked."""
     flags = ["-Xptxas", "-O0", "-Xcompiler", "-fsanitize=float-cast-overflow,-fno-sanitize-recover=all"]
