@@ -20,7 +20,8 @@
 // gathers a pixel with crosstalk and eight samples. The searches go through a
 // table of thresholds in shared memory, and a warp's lanes take panel columns
 // a stride apart at which the lens phase repeats, so that they mostly gather
-// from the same view (see there).
+// from the same view (see there); k_interleave_gauss_plain serves what is too
+// little for a table.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -426,7 +427,6 @@ __device__ __forceinline__ uint32_t gauss_pixel(const DispConst& c, const uint32
 // on the same border of their intervals), or the few steps do not settle a
 // threshold, the block keeps to nearest_view for every pixel.
 constexpr int kGaussBins = 8;          // bins per display view
-constexpr int kGaussMargin = 4;        // display views covered on either side of [0, N]
 constexpr float kGaussApart = 0x1p-12f;
 constexpr int kGaussSteps = 16;
 constexpr int kGaussMaxStride = 64;    // largest column stride between a warp's lanes
@@ -552,26 +552,25 @@ __device__ __forceinline__ uint32_t gauss_pixel_table(const DispConst& c, const 
 // now, bound by issue (two thirds of the slots; 72 searches and gathers of
 // about a dozen instructions) and the L1 wavefronts of the gathers (half their
 // rate). 64 registers and four blocks per SM: five at 48 registers take 0.195.
-// table: the views' bytes fit 32-bit offsets and every sample's angular
-// offset lies within the table's margin (the launch cannot know the offsets:
-// they are checked here).
+// The views' bytes fit 32-bit offsets (gauss_table). Whether every sample's angular
+// offset lies within the table's margin is checked here: a captured launch may
+// meet other samples than it was recorded with.
 constexpr int kGaussThreads = 256;
 template <bool XT>
 __global__ void __launch_bounds__(kGaussThreads, 4) k_interleave_gauss(DispConst c, const uint8_t* __restrict__ views,
                                                                     const float* __restrict__ pos,
                                                                     const float* __restrict__ samples, int ns,
-                                                                    uint8_t* __restrict__ panel, int S, int table) {
+                                                                    uint8_t* __restrict__ panel, int S, int n_bins) {
     wait_previous_kernel();
     allow_next_kernel();
     extern __shared__ __align__(16) uint8_t s_dyn[];
     GaussBin* s_bins = reinterpret_cast<GaussBin*>(s_dyn);
-    const int n_bins = table ? gauss_bins(c.n_views) : 0;
     uint32_t* s_row = reinterpret_cast<uint32_t*>(s_bins + n_bins);   // [2][32 S] finished rows
     __shared__ float s_pos[kMaxRenderViews];
     __shared__ float s_smp[3 * 32];
     __shared__ float4 s_smp4[32];
     const uint32_t view_bytes = 4u * uint32_t(c.W) * uint32_t(c.H);
-    bool slow = !table;
+    bool slow = false;
     for (int i = threadIdx.x; i < c.nr; i += kGaussThreads) s_pos[i] = pos[i];
     for (int i = threadIdx.x; i < 3 * ns; i += kGaussThreads) s_smp[i] = samples[i];
     for (int i = threadIdx.x; i < ns; i += kGaussThreads) {
@@ -615,6 +614,42 @@ __global__ void __launch_bounds__(kGaussThreads, 4) k_interleave_gauss(DispConst
         uint32_t* dst = reinterpret_cast<uint32_t*>(panel) + (uint64_t)y * c.Wp + x0;
         for (int q = threadIdx.x; q < cols && x0 + q < c.Wp; q += kGaussThreads) dst[q] = row[q];
     }
+}
+
+// The same a thread a pixel, each search among four positions: where a table's
+// making costs more than it saves, for views beyond its 32-bit offsets and for
+// angular offsets beyond its margin (gauss_table).
+__global__ void __launch_bounds__(kGaussThreads) k_interleave_gauss_plain(DispConst c, const uint8_t* __restrict__ views,
+                                                                          const float* __restrict__ pos,
+                                                                          const float* __restrict__ samples, int ns,
+                                                                          uint8_t* __restrict__ panel) {
+    wait_previous_kernel();
+    allow_next_kernel();
+    __shared__ float s_pos[kMaxRenderViews];
+    __shared__ float s_smp[3 * 32];
+    for (int i = threadIdx.x; i < c.nr; i += kGaussThreads) s_pos[i] = pos[i];
+    for (int i = threadIdx.x; i < 3 * ns; i += kGaussThreads) s_smp[i] = samples[i];
+    __syncthreads();
+    const uint64_t total = (uint64_t)c.Wp * c.Hp;
+    const float sxw = float(c.W) / float(c.Wp), syh = float(c.H) / float(c.Hp);
+    const uint32_t* v32 = reinterpret_cast<const uint32_t*>(views);
+    for (uint64_t i = (uint64_t)blockIdx.x * kGaussThreads + threadIdx.x; i < total; i += (uint64_t)gridDim.x * kGaussThreads) {
+        const int y = int(i / c.Wp), x = int(i - (uint64_t)y * c.Wp);
+        reinterpret_cast<uint32_t*>(panel)[i] = gauss_pixel(c, v32, s_pos, s_smp, ns, x, y, sxw, syh);
+    }
+}
+
+// Whether the table pays. Every block makes it, bins / 256 of them a thread with
+// several searches each, and it saves most of a search per look-up: of a thread's
+// look-ups, 3 a pixel and sample (9 with crosstalk) for at least one pixel. 256
+// views to a panel of 256x256, one sample: 5.2 us a thread a pixel, 10.6 with the
+// table; of 32 samples 28.9 and 14.6. 96 views to 512x512: one sample 6.9 and 10.1,
+// four 13.4 and 11.9. near: every sample's angular offset lies within the table's
+// margin (beyond it the kernel would search as the plain one does, a fifth slower).
+bool gauss_table(const DispConst& c, int ns, bool near, int sms) {
+    if (!near || (uint64_t)c.nr * c.W * c.H * 4u > 0xffffffffull) return false;
+    const double pixels = std::max(1.0, double(c.Wp) * c.Hp / (4.0 * kGaussThreads * sms));
+    return pixels * ns * (c.xtalk > 0.0f ? 9.0 : 3.0) > 3.2 * gauss_bins(c.n_views) / kGaussThreads;
 }
 
 // The column stride between a warp's lanes: of the multiples of 8 (one warp
@@ -764,7 +799,7 @@ cudaError_t launch_view_mip(const uint8_t* views, int W, int H, int nr, int leve
 }
 
 cudaError_t launch_interleave(const DispConst& dc, const uint8_t* views, const float* pos, const float* samples,
-                              int n_samples, uint8_t* panel, cudaStream_t s) {
+                              int n_samples, bool near, uint8_t* panel, cudaStream_t s) {
     int dev = 0, sms = 0, smem_max = 0, smem_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -772,17 +807,16 @@ cudaError_t launch_interleave(const DispConst& dc, const uint8_t* views, const f
     cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     if (dc.recon == 2 || dc.recon == 3) {
         if (n_samples < 1 || n_samples > 32) return cudaErrorInvalidValue;
+        if (!gauss_table(dc, n_samples, near, sms))
+            return launch_after_previous(k_interleave_gauss_plain, dim3(sms * 16), dim3(kGaussThreads), 0, s, dc, views, pos,
+                                         samples, n_samples, panel);
         const int S = gauss_stride(dc);
-        // 32-bit byte offsets of the views' texels
-        const int table = (uint64_t)dc.nr * dc.W * dc.H * 4u <= 0xffffffffull;
-        const size_t bytes = (table ? sizeof(GaussBin) * gauss_bins(dc.n_views) : 0u) + 2u * 32u * S * 4u;
+        const int bins = gauss_bins(dc.n_views);
+        const size_t bytes = sizeof(GaussBin) * bins + 2u * 32u * S * 4u;
         const uint64_t rows = (uint64_t)((dc.Wp + 32 * S - 1) / (32 * S)) * dc.Hp;
         const int grid = int(std::min<uint64_t>(rows, uint64_t(sms) * 4u));
-        if (dc.xtalk > 0.0f)
-            return launch_after_previous(k_interleave_gauss<true>, dim3(grid), dim3(kGaussThreads), bytes, s, dc, views,
-                                         pos, samples, n_samples, panel, S, table);
-        return launch_after_previous(k_interleave_gauss<false>, dim3(grid), dim3(kGaussThreads), bytes, s, dc, views,
-                                     pos, samples, n_samples, panel, S, table);
+        return launch_after_previous(dc.xtalk > 0.0f ? k_interleave_gauss<true> : k_interleave_gauss<false>, dim3(grid),
+                                     dim3(kGaussThreads), bytes, s, dc, views, pos, samples, n_samples, panel, S, bins);
     }
     // the widest source segment of a strip: (cols - 1) W / Wp + 2 pixels
     const bool tent = dc.recon == 1;

@@ -424,9 +424,11 @@ constexpr int kMaxBatchScenes = 64;
 constexpr int kMaxBatchViews = 4096;   // rendered views summed over a batch
 cudaError_t launch_resolve(const FrameArgs& a, cudaStream_t s);
 // pos [nr] (views on the display-view axis) and samples [n_samples][3] are
-// read only for Gaussian reconstruction (recon 2, 3).
+// read only for Gaussian reconstruction (recon 2, 3); near: no sample's angular
+// offset is beyond kGaussMargin views.
+constexpr int kGaussMargin = 4;        // display views covered on either side of [0, N] by the Gaussian's table
 cudaError_t launch_interleave(const DispConst& dc, const uint8_t* views, const float* pos, const float* samples,
-                              int n_samples, uint8_t* panel, cudaStream_t s);
+                              int n_samples, bool near, uint8_t* panel, cudaStream_t s);
 // Mip level `level` (1 or 2) of nr views of W x H RGBA8 into out.
 cudaError_t launch_view_mip(const uint8_t* views, int W, int H, int nr, int level, uint8_t* out, cudaStream_t s);
 cudaError_t launch_mip_level(const uint8_t* src, uint32_t sw, uint32_t sh, uint8_t* dst,

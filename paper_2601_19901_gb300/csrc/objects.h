@@ -25,6 +25,7 @@ struct lfdpr_display {
     float* d_pos = nullptr;       // rendered views' positions on the display-view axis
     float* d_samples = nullptr;   // Gaussian reconstruction samples [32][3]
     int n_samples = 0;
+    bool near_samples = true;     // every angular offset within kGaussMargin views
     uint4* points = nullptr;
     uint32_t max_points = 0;
     lfdpr::WorkRec* work = nullptr;

@@ -199,7 +199,8 @@ lfdpr_status record_interleave(lfdpr_display* disp, uint8_t* panel, cudaStream_t
         dc.H >>= disp->ss_level;
         views = disp->views_mip;
     }
-    const cudaError_t e = launch_interleave(dc, views, disp->d_pos, disp->d_samples, disp->n_samples, panel, s);
+    const cudaError_t e = launch_interleave(dc, views, disp->d_pos, disp->d_samples, disp->n_samples, disp->near_samples,
+                                            panel, s);
     if (e != cudaSuccess) return cuda_fail(e, "launch k_interleave");
     disp->launches += 1;
     return LFDPR_OK;
@@ -628,6 +629,8 @@ lfdpr_status lfdpr_set_recon_samples(lfdpr_display* disp, const float* samples, 
         if (!std::isfinite(samples[k])) return fail(LFDPR_EINVAL, "set_recon_samples: non-finite offset");
     CK(cudaMemcpy(disp->d_samples, samples, sizeof(float) * 3 * n, cudaMemcpyHostToDevice), "set_recon_samples");
     disp->n_samples = n;
+    disp->near_samples = true;
+    for (int k = 0; k < n; k++) disp->near_samples &= std::fabs(samples[3 * k + 2]) <= float(kGaussMargin);
     return LFDPR_OK;
 }
 

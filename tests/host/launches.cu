@@ -49,7 +49,7 @@ static DispConst display(int recon, int n, int w, int h, int panel_w, int panel_
 }
 
 static cudaError_t interleave(int recon, int n, int w, int panel_w) {
-    return launch_interleave(display(recon, n, w, 64, panel_w, 640, 0.15f), nullptr, nullptr, nullptr, 0, nullptr, nullptr);
+    return launch_interleave(display(recon, n, w, 64, panel_w, 640, 0.15f), nullptr, nullptr, nullptr, 0, true, nullptr, nullptr);
 }
 
 // which form a tent interleave takes: tiles (dynamic shared memory) or the gather
@@ -71,9 +71,30 @@ static void tent() {
     for (const auto& k : cases) {
         char what[96];
         snprintf(what, sizeof what, "%d views of %dx%d to %dx%d, crosstalk %g", k.n, k.w, k.h, k.pw, k.ph, k.xtalk);
-        check(launch_interleave(display(1, k.n, k.w, k.h, k.pw, k.ph, k.xtalk), nullptr, nullptr, nullptr, 0, nullptr,
+        check(launch_interleave(display(1, k.n, k.w, k.h, k.pw, k.ph, k.xtalk), nullptr, nullptr, nullptr, 0, true, nullptr,
                                 nullptr) == cudaSuccess &&
                   (g_last_smem > 0) == k.tiles,
+              what);
+    }
+}
+
+// which form a Gaussian interleave takes: with the table (dynamic shared memory) or plain
+static void gauss() {
+    const struct {
+        int n, w, h, pw, ph, ns;
+        float xtalk;
+        bool near, table;
+    } cases[] = {{48, 420, 560, 2560, 1600, 8, 0.15f, true, true},   {48, 420, 560, 2560, 1600, 8, 0.15f, false, false},
+                 {48, 420, 560, 2560, 1600, 1, 0.0f, true, true},    {256, 64, 64, 256, 256, 1, 0.0f, true, false},
+                 {256, 64, 64, 256, 256, 4, 0.0f, true, false},      {256, 64, 64, 256, 256, 32, 0.0f, true, true},
+                 {96, 128, 128, 512, 512, 1, 0.0f, true, false},     {96, 128, 128, 512, 512, 4, 0.0f, true, true},
+                 {256, 1000, 2200, 2560, 1600, 8, 0.15f, true, false}};   // beyond 32-bit offsets
+    for (const auto& k : cases) {
+        char what[96];
+        snprintf(what, sizeof what, "%d views of %dx%d to %dx%d, %d samples", k.n, k.w, k.h, k.pw, k.ph, k.ns);
+        check(launch_interleave(display(2, k.n, k.w, k.h, k.pw, k.ph, k.xtalk), nullptr, nullptr, nullptr, k.ns, k.near,
+                                nullptr, nullptr) == cudaSuccess &&
+                  (g_last_smem > 0) == k.table,
               what);
     }
 }
@@ -81,9 +102,9 @@ static void tent() {
 // a lens pitch whose reciprocal overflows: the lens phase is no number
 static void tiny_pitch() {
     for (int recon : {2, 3}) {
-        DispConst c = display(recon, 8, 64, 64, 200, 200, 0.0f);
+        DispConst c = display(recon, 8, 64, 64, 200, 200, 0.15f);   // (with the table)
         c.inv_pitch = INFINITY;
-        check(launch_interleave(c, nullptr, nullptr, nullptr, 1, nullptr, nullptr) == cudaSuccess, "tiny pitch");
+        check(launch_interleave(c, nullptr, nullptr, nullptr, 1, true, nullptr, nullptr) == cudaSuccess, "tiny pitch");
     }
 }
 
@@ -129,6 +150,7 @@ int main(int, char** argv) {
     if (!strcmp(argv[1], "threads")) threads();
     if (!strcmp(argv[1], "tiny_pitch")) tiny_pitch();
     if (!strcmp(argv[1], "tent")) tent();
+    if (!strcmp(argv[1], "gauss")) gauss();
     check(g_launched > 0, "something was launched");
     return g_failed;
 }

@@ -1,6 +1,7 @@
 """The interleave's forms on either side of the rules that choose between them,
 byte for byte against the oracle on views of random bytes: the tent's tiles
-(panels of many rows a view row) and the gather, with and without crosstalk.
+(panels of many rows a view row) and the gather, with and without crosstalk;
+the Gaussian with and without its table.
 """
 import numpy as np
 import pytest
@@ -34,3 +35,26 @@ def test_tent_matches_oracle(case):
     d = _display(*TENT[case])
     views = _views(d, 80 + case)
     assert np.array_equal(_panel(d, views), O.interleave(d, views))
+
+
+# (views, view w, h, panel w, h, pitch, slant, recon, crosstalk, samples, largest dphi)
+GAUSS = [(48, 21, 28, 64, 64, 8.0, 0.2, 2, 0.0, 1, None),         # too little for a table
+         (96, 21, 28, 65, 63, 8.0, 0.2, 3, 0.0, 2, None),
+         (256, 8, 9, 130, 20, 11.0, 0.3, 2, 0.15, 2, None),
+         (256, 8, 9, 130, 20, 11.0, 0.3, 2, 0.15, 3, None),       # enough for one
+         (1, 9, 9, 1, 1, 8.0, 0.2, 2, 0.2, 1, None),
+         (16, 12, 12, 700, 300, 8.0, 0.2, 2, 0.15, 7, 4.01),      # beyond the table
+         (16, 12, 12, 700, 300, 8.0, 0.2, 3, 0.0, 8, -9.0)]
+
+
+@pytest.mark.parametrize("case", range(len(GAUSS)))
+def test_gaussian_matches_oracle(case):
+    *size, ns, dphi = GAUSS[case]
+    d = _display(*size)
+    rng = np.random.default_rng(200 + case)
+    u = rng.random(d.n_render_views).astype(np.float32)
+    smp = (rng.normal(0.0, 1.0, (ns, 3)) * [0.5625, 0.5625, 0.5]).astype(np.float32)
+    if dphi is not None:
+        smp[-1, 2] = dphi
+    views = _views(d, 120 + case)
+    assert np.array_equal(_panel(d, views, u, smp), O.interleave(d, views, jitter=u, samples=smp))
