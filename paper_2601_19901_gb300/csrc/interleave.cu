@@ -141,6 +141,12 @@ constexpr int kTileCols = 4 * kTileThreads;   // panel columns per tile
 constexpr int kTentCols = 4 * kTentThreads;
 constexpr int kStageCols = 4;                 // 32-column runs of a row segment loaded together
 
+// Rendered views from which a tile is staged run after run of all views, two
+// views' loads in flight a warp; fewer leave a warp one view, and its whole segment
+// is loaded in turn (48 views of 1024x768 to 1920x1080: 62.8 us run after run, 71.2
+// view after view; 5 of 4000x1000 to 1000x500: 21.8 and 13.8).
+constexpr int kTileManyViews = 16;
+
 // The first panel row sampling view row sy; false if none does.
 __device__ __forceinline__ bool first_row_of(const DispConst& c, int sy, int& y) {
     y = max(0, int(uint32_t(sy) * uint32_t(c.Hp) / uint32_t(c.H)) - 1);
@@ -164,17 +170,27 @@ __global__ void __launch_bounds__(kTileThreads) k_interleave_tile(DispConst c, c
     const uint64_t npix = (uint64_t)c.W * c.H;
     const uint32_t* v32 = reinterpret_cast<const uint32_t*>(views);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i0 = lane; i0 < n; i0 += 32 * kStageCols)
-#pragma unroll 2
-        for (int m = warp; m < c.nr; m += kTileThreads / 32) {
+    constexpr int kWarps = kTileThreads / 32;
+    if (c.nr < kTileManyViews) {
+        for (int m = warp; m < c.nr; m += kWarps) {
             const uint32_t* src = v32 + (uint64_t)m * npix + (uint64_t)sy * c.W + sx_lo;
-#pragma unroll
-            for (int q = 0; q < kStageCols; q++) {
-                const int i = i0 + 32 * q;
-                if (i < n && LFDPR_IN_BOUNDS(uint32_t(sx_lo + i), uint32_t(c.W), 20) && LFDPR_IN_BOUNDS(i, stride, 20))
+            for (int i = lane; i < n; i += 32)
+                if (LFDPR_IN_BOUNDS(uint32_t(sx_lo + i), uint32_t(c.W), 20) && LFDPR_IN_BOUNDS(i, stride, 20))
                     s_row[m * stride + i] = __ldg(src + i);
-            }
         }
+    } else {
+        for (int i0 = lane; i0 < n; i0 += 32 * kStageCols)
+#pragma unroll 2
+            for (int m = warp; m < c.nr; m += kWarps) {
+                const uint32_t* src = v32 + (uint64_t)m * npix + (uint64_t)sy * c.W + sx_lo;
+#pragma unroll
+                for (int q = 0; q < kStageCols; q++) {
+                    const int i = i0 + 32 * q;
+                    if (i < n && LFDPR_IN_BOUNDS(uint32_t(sx_lo + i), uint32_t(c.W), 20) && LFDPR_IN_BOUNDS(i, stride, 20))
+                        s_row[m * stride + i] = __ldg(src + i);
+                }
+            }
+    }
     __syncthreads();
     const int xg = x0 + 4 * threadIdx.x;
     if (xg >= x1) return;
