@@ -436,7 +436,12 @@ lfdpr_status upload_geometry(lfdpr_display* disp, const float* xyz, const float*
 // most 64 views: 96 views, keys of 321 MB 1.42 against 1.48 ms, 361 MB 1.90
 // against 1.74, 501 MB 2.83 against 2.27, 723 MB 4.44 against 3.38; 128 views,
 // 595 MB 3.04 against 2.32. Up to 64 views a second band costs more than it
-// saves (64 views, 394 MB 1.82 against 1.93).
+// saves (64 views, 394 MB 1.82 against 1.93). The line does not look at the mesh,
+// and what bands save follows its depth tests: they lose on smaller ones (100,000
+// triangles: 80 views, 454 MB 0.91 against 1.00, 96 views, 722 MB 1.64 against 1.42;
+// 10,000 triangles: 96 views, 483 MB 0.365 against 0.380, 256 views, 481 MB 0.36
+// against 0.44) and near the line (10^6 triangles, 65 views, 374 MB 1.48 against
+// 1.57). A caller with such frames sets one band.
 int view_band(const lfdpr_display* d) {
     const int nr = d->dc.nr;
     if (d->view_band > 0) return std::min(d->view_band, nr);
