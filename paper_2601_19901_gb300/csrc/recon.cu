@@ -1180,26 +1180,35 @@ lfdpr_status lfdpr_create_recon(int32_t view_w, int32_t view_h, int32_t in_views
     for (int o = 0; o < no3; o++) bout[o] = biases[nb3 + o];
     // layer geometry and packed weights; the layers leave each SM the shared
     // memory of two blocks of the warp (and 1 KB of the system's for each),
-    // which runs beside them
-    const uint32_t reserve = kWarpsBeside * (uint32_t(warp_smem(r->nin, r->nout, r->W)) + 1024u);
-    for (int l = 0; l < 14; l++) {
+    // which runs beside them. Views so wide that some layer's tiles leave no
+    // room keep no room in any: small tiles in the others would not be made up
+    // for (900x500, 2 to 16 input views: 432..706 us with room where it can be
+    // left, 360..615 without; 1024x768 714..1136 and 574..994).
+    auto tile = [&](int l, uint32_t reserve) {
         const ConvSpec& L = kLayers[l];
-        const int Hl = r->Hp >> L.level, Wl = r->Wp >> L.level;
         // layers 8, 10, 12 read [upsampled (map a) | skip (map b)]
         const int cin_b = (l == 8 || l == 10 || l == 12) ? L.cin / 3 : 0;
         const int up = l == 7 || l == 9 || l == 11;   // write 2x upsampled into the next level's tensor
-        r->geom[l] = pick_tile(Hl, Wl, L.cin - cin_b, cin_b, L.cout, up, r->sm_count, reserve);
+        return pick_tile(r->Hp >> L.level, r->Wp >> L.level, L.cin - cin_b, cin_b, L.cout, up, r->sm_count, reserve);
+    };
+    uint32_t reserve = kWarpsBeside * (uint32_t(warp_smem(r->nin, r->nout, r->W)) + 1024u);
+    for (int l = 0; l < 14; l++)
+        if (!tile(l, reserve).beside) {
+            reserve = 0;
+            break;
+        }
+    for (int l = 0; l < 14; l++) {
+        r->geom[l] = tile(l, reserve);
         r->geom[l].early = 1;
-        if (up) {
+        if (r->geom[l].up) {
+            const int Hl = r->Hp >> kLayers[l].level, Wl = r->Wp >> kLayers[l].level;
             r->geom[l].Wbo = 2 * Wl + 2;
             r->geom[l].Qpo = int(qpad(2 * Hl, 2 * Wl));
         }
     }
-    // as many blocks of the warp as the layers leave room for; where one does
-    // not, a block per row and interval
-    r->warp_grid = kWarpsBeside * r->sm_count;
-    for (const TcGeom& g : r->geom)
-        if (!g.beside) r->warp_grid = r->H * (r->nin - 1);
+    // as many blocks of the warp as the layers leave room for; where they leave
+    // none, a block per row and interval
+    r->warp_grid = reserve ? kWarpsBeside * r->sm_count : r->H * (r->nin - 1);
     r->geom_out = out_geom(r->Hp, r->Wp, r->H, r->W, r->nout, ntout);
     const __nv_bfloat16* conv_in[14] = {r->x0, r->e0a, r->p1, r->e1a, r->p2, r->e2a, r->p3,
                                         r->ba, r->U2,  r->d2a, r->U1, r->d1a, r->U0, r->d0a};
