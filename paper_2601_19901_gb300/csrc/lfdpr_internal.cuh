@@ -407,12 +407,13 @@ cudaError_t launch_after_previous(void (*kernel)(P...), dim3 grid, dim3 block, s
 cudaError_t launch_setup(const FrameArgs& a, cudaStream_t s);
 // The depth-guided warp of nin rendered views (RGBA8 and depth keys) to nout
 // eyes on the same eye line (warp.cu); views at most kMaxWarpWidth wide.
-// grid: blocks, each taking (row, input interval) pairs in turn.
+// grid: blocks, each taking (row, input interval) pairs in turn; beside: the call
+// runs beside the network's layers.
 constexpr int kMaxWarpWidth = 4032;   // the warp block's shared memory: 48 bytes a pixel at the widest
 size_t warp_smem(int nin, int nout, int W);   // bytes of dynamic shared memory of a block
 cudaError_t launch_warp_views(const uint8_t* views, const uint64_t* keys, const float* in_eyes, int nin,
                               const float* out_eyes, int nout, int W, int H, float ipw, uint8_t* out, int grid,
-                              cudaStream_t s);
+                              bool beside, cudaStream_t s);
 cudaError_t launch_scan(const FrameArgs& a, cudaStream_t s);
 cudaError_t launch_emit(const FrameArgs& a, cudaStream_t s);
 cudaError_t launch_fetch(const FrameArgs& a, cudaStream_t s);

@@ -1298,7 +1298,7 @@ lfdpr_status lfdpr_recon_forward(lfdpr_recon* r, const uint8_t* in_views, const 
     CKR(conv(0), "conv 0");
     CKR(cudaStreamWaitEvent(r->side, r->fork, 0), "recon_forward: fork");
     CKR(launch_warp_views(in_views, in_keys, in_eyes, r->nin, out_eyes, r->nout, r->W, r->H, pixels_per_unit,
-                          r->warp, r->warp_grid, r->side),
+                          r->warp, r->warp_grid, true, r->side),
         "launch k_warp_views");
     CKR(cudaEventRecord(r->join, r->side), "recon_forward: join");
     CKR(conv(1), "conv 1");

@@ -108,7 +108,7 @@ static void tiny_pitch() {
     }
 }
 
-static cudaError_t warp(int w) { return launch_warp_views(nullptr, nullptr, nullptr, 2, nullptr, 4, w, 64, 1.0f, nullptr, 1, nullptr); }
+static cudaError_t warp(int w) { return launch_warp_views(nullptr, nullptr, nullptr, 2, nullptr, 4, w, 64, 1.0f, nullptr, 1, false, nullptr); }
 
 // every number of view slots a lane, and both unit sizes, on one device and then another
 static void devices() {
@@ -140,7 +140,7 @@ static void threads() {
     check(interleave(0, 48, 420, 1000) == cudaSuccess, "large tile beside a small one");
     g_meanwhile = [] { check(interleave(1, 4, 420, 2560) == cudaSuccess, "small tent tile"); };
     check(interleave(1, 100, 240, 1000) == cudaSuccess, "large tent tile beside a small one");
-    g_meanwhile = [] { check(warp(1200) == cudaSuccess, "narrow warp"); };
+    g_meanwhile = [] { check(warp(1200) == cudaSuccess, "narrower warp"); };
     check(warp(4000) == cudaSuccess, "wide warp beside a narrow one");
 }
 
