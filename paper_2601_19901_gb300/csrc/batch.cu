@@ -1,7 +1,9 @@
 // Batched frames (lfdpr_create_batch ... lfdpr_batch_panel in include/lfdpr.h):
 // several (display, mesh) scenes of uneven size rendered and interleaved by
 // one CUDA graph: each scene's frame, from set-up (Sec. 3.1) to interleave
-// (Sec. 4), on one of the concurrent branches. Each scene runs exactly the kernels and
+// (Sec. 4), on one of the concurrent branches. With more scenes than branches a
+// branch is two streams, so that a scene's point generation runs beside the splat
+// of the scene before it. Each scene runs exactly the kernels and
 // arithmetic of lfdpr_render_frame + lfdpr_interleave, so its keys, views and
 // panel are bit-identical to rendering it alone; the model matrices come from
 // device memory so one captured graph replays every frame.
@@ -26,8 +28,8 @@ struct lfdpr_batch {
     float* h_models = nullptr;       // pinned staging of the same
     cudaEvent_t staged = nullptr;    // the last copy out of h_models has run
     cudaStream_t cap = nullptr;      // the stream the graph is captured on
-    std::vector<cudaStream_t> br;    // branch streams
-    std::vector<cudaEvent_t> ev;     // fork, joins
+    std::vector<cudaStream_t> br;    // branch streams; with more scenes than branches, their second ones after them
+    std::vector<cudaEvent_t> ev;     // fork, joins, then a branch's fetch done
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     bool stale = true;               // capture again before the next replay
@@ -89,31 +91,48 @@ void free_batch(lfdpr_batch* b) {
     delete b;
 }
 
+// Streams of the batch's branches.
+int branch_streams(const lfdpr_batch* b) { return b->n > b->cfg.branches ? 2 * b->cfg.branches : b->cfg.branches; }
+
 // Record the whole batch on b->cap (which is capturing).
 lfdpr_status record_batch(lfdpr_batch* b) {
-    const int K = b->cfg.branches;
+    const int K = b->cfg.branches, n_streams = branch_streams(b);
     cudaStream_t s = b->cap;
-    cudaEvent_t fork = b->ev[0];   // then the branches' joins
+    cudaEvent_t fork = b->ev[0];   // then the streams' joins
     // timing events as event-record nodes of the graph (a plain record during
     // capture would only join streams)
     CK(cudaEventRecordWithFlags(b->tev[0], s, cudaEventRecordExternal), "batch: start event");
     CK(cudaEventRecord(fork, s), "batch: fork");
-    for (int j = 0; j < K; j++) CK(cudaStreamWaitEvent(b->br[j], fork, 0), "batch: branch wait");
+    for (int j = 0; j < n_streams; j++) CK(cudaStreamWaitEvent(b->br[j], fork, 0), "batch: branch wait");
+    // A wave of the splat's blocks, whatever the configuration asks for beyond it: a
+    // splat of few points ends with the blocks it has no units for, and beside other
+    // scenes one wave is enough for many. 32 scenes of 5,000 triangles, 24 views: 768
+    // us with 16 blocks per SM and one stream a branch, 678 with four blocks, 662 with
+    // two streams as well (620 with one splat over all scenes, which took 1145
+    // against 941 for 12 scenes of 20,000 at 96 views); 64 of 1,000, 4 views 1144, 956
+    // and 699; 12 of 5,000 to 200,000 triangles, 24 to 96 views 2766, 2724 and 2685.
+    const int splat_blocks = std::min(b->cfg.splat_blocks_per_sm, 4);
     for (int i = 0; i < b->n; i++) {
+        cudaStream_t front = b->br[i % K], back = b->br[n_streams - K + i % K];
         FrameArgs a = frame_args(b->disp[i], b->mesh[i]);
         a.model_dev = b->d_models + 12 * i;
-        const lfdpr_status st = record_frame_front(b->disp[i], b->mesh[i], a, b->br[i % K], false);
+        const lfdpr_status st = record_frame_front(b->disp[i], b->mesh[i], a, front, false);
         if (st != LFDPR_OK) return st;
-        CK(launch_splat(a, b->br[i % K], b->cfg.splat_blocks_per_sm, b->cfg.splat_slots), "launch k_splat");
-        CK(launch_resolve(a, b->br[i % K]), "launch k_resolve");
+        if (back != front) {
+            cudaEvent_t fetched = b->ev[1 + n_streams + i % K];
+            CK(cudaEventRecord(fetched, front), "batch: fetched");
+            CK(cudaStreamWaitEvent(back, fetched, 0), "batch: splat wait");
+        }
+        CK(launch_splat(a, back, splat_blocks, b->cfg.splat_slots), "launch k_splat");
+        CK(launch_resolve(a, back), "launch k_resolve");
         lfdpr_display* d = b->disp[i];
         if ((d->desc.recon == 2 || d->desc.recon == 3) && d->n_samples == 0)
             return fail(LFDPR_EINVAL, "batch: scene %d needs lfdpr_set_recon_samples", i);
-        const lfdpr_status sti = record_interleave(b->disp[i], d->panel, b->br[i % K]);
+        const lfdpr_status sti = record_interleave(b->disp[i], d->panel, back);
         if (sti != LFDPR_OK) return sti;
-        CK(cudaEventRecordWithFlags(b->tev[1 + i], b->br[i % K], cudaEventRecordExternal), "batch: scene event");
+        CK(cudaEventRecordWithFlags(b->tev[1 + i], back, cudaEventRecordExternal), "batch: scene event");
     }
-    for (int j = 0; j < K; j++) {
+    for (int j = 0; j < n_streams; j++) {
         CK(cudaEventRecord(b->ev[1 + j], b->br[j]), "batch: join");
         CK(cudaStreamWaitEvent(s, b->ev[1 + j], 0), "batch: join wait");
     }
@@ -122,11 +141,11 @@ lfdpr_status record_batch(lfdpr_batch* b) {
 
 lfdpr_status capture(lfdpr_batch* b) {
     drop_graph(b);
-    const int K = b->cfg.branches;
-    if ((int)b->br.size() != K) {
+    const int n_streams = branch_streams(b);
+    if ((int)b->br.size() != n_streams) {
         drop_branches(b);
-        b->br.resize(K, nullptr);
-        b->ev.resize(1 + K, nullptr);
+        b->br.resize(n_streams, nullptr);
+        b->ev.resize(1 + n_streams + b->cfg.branches, nullptr);
         for (auto& s : b->br) CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking), "batch: stream");
         for (auto& e : b->ev) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "batch: event");
     }
@@ -273,7 +292,7 @@ lfdpr_status lfdpr_batch_autotune(lfdpr_batch* b, const float* models, int32_t r
     g_err[0] = 0;
     if (!b || !models || reps < 1) return fail(LFDPR_EINVAL, "batch_autotune: null argument or reps < 1");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // Candidates: branch counts, persistent-splat grid sizes, and view slots
+    // Candidates: branch counts, splat grid sizes, and view slots
     // per lane (the fewest that hold the largest view count, and half that
     // where the scenes' view counts make two groups of it fit).
     std::vector<int> ks, gs = {4, 8, 16}, ss;
