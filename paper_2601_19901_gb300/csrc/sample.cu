@@ -626,7 +626,10 @@ __device__ __forceinline__ int last_at_most(const uint32_t* s_num, uint32_t k) {
 // columns, and its stores are contiguous.
 //
 // Meshes whose 256-triangle blocks do not fill the SMs spread each over `split`
-// blocks (each scans all 256 counts and emits its share of the triangles).
+// blocks (each scans all 256 counts and emits its share of the triangles: of those
+// emitted by a thread neighbours, in whole warps, of the others every split-th where
+// that is more than every second, so that a few large triangles are shared out too:
+// eight of 28,000 points each 184 us in one block, 32 in eight).
 // Bound by the dependent chain of a block's largest triangle while one thread or
 // one warp emits it; shared out, by the searches and stores of its points.
 // Measured on twelve meshes of 61 k to 1.2 M points (24 to 96 views): 608 us
@@ -654,9 +657,10 @@ __global__ void __launch_bounds__(kSetupThreads) k_emit(FrameArgs a, uint32_t sp
     // meshes a block's chain of loads is the kernel's time: 2,048 triangles 8.0 ->
     // 6.3 us, 10^6 31.7 -> 30.7)
     const uint32_t cnt = t < a.n_tris ? a.counts[t] : 0u;
-    const bool mine = t < a.n_tris && threadIdx.x / width == part;
+    const uint32_t near = threadIdx.x / width, far = split > 2u ? threadIdx.x % split : near;
     uint4 cs = make_uint4(kColSumWalk, 0u, 0u, 0u);
-    if (mine && a.colsum) cs = __ldcg(a.colsum + t);
+    if (t < a.n_tris && (near == part || far == part) && a.colsum) cs = __ldcg(a.colsum + t);
+    const bool big = cnt > kEmitOwn, mine = t < a.n_tris && (big ? far : near) == part;
     uint32_t first;
     bool overflow;
     if constexpr (kScanned) {
@@ -706,7 +710,7 @@ __global__ void __launch_bounds__(kSetupThreads) k_emit(FrameArgs a, uint32_t sp
     if (mine) a.offsets[t] = first;
     if (overflow) return;
     const bool live = mine && cnt > 0u;
-    const bool walk = cs.x == kColSumWalk, together = live && cnt > kEmitOwn;
+    const bool walk = cs.x == kColSumWalk, together = live && big;
     const uint32_t w[4] = {cs.x, cs.y, cs.z, cs.w};
     if (live && !together) {
         uint32_t p = first;
