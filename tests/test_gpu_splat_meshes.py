@@ -1,0 +1,53 @@
+"""The splat's kernels by the size of the mesh: with four and six view slots a
+lane, units of two points below 50,000 and 150,000 triangles and of four from
+there on. Sampling and the views looked at equal the oracle's on either side, and
+the walk of segments (a low lane limit) gives the pooled passes' keys."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2601_19901_gb300 import lfdpr, scenes as S
+from parity import check_sampling, check_views, gpu_frame
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2601_19901_gb300 import build
+    build.build()
+    lfdpr.lib()
+
+
+def _mesh(triangles):
+    """Displaced surfaces of 5,000 triangles each, cut to the number asked for."""
+    sc = S.geometry_paper(n_instances=-(-triangles // 5000), res=50, n_textures=2, seed=5, r_max=0.5)
+    return replace(sc, idx=sc.idx[:triangles], tri_tex=sc.tri_tex[:triangles],
+                   textures=[S.value_noise_texture(64, 64, 7), S.value_noise_texture(256, 256, 8)])
+
+
+def _check(views, triangles, bias_h=1.0, bias_v=1.0, size=96):
+    d = replace(S.display_paper(), n_views=views, view_w=size, view_h=size + 8, focal_w=2.4 * size / (size + 8),
+                bias_h=bias_h, bias_v=bias_v)
+    sc, m = _mesh(triangles), S.model_matrix(4)
+    looked_at = sorted({0, views // 2, views - 1})
+    o = O.render(d, sc, m, views=looked_at, panel=False)
+    with lfdpr.Renderer(d, sc, len(o.points) + 1) as R:
+        g = gpu_frame(d, sc, m, renderer=R, panel=False)
+        lfdpr.lfdpr_set_splat_lane_limit(R.disp, 3)
+        walked = gpu_frame(d, sc, m, renderer=R, panel=False)
+    assert g.stats.n_splat_writes > 0
+    check_sampling(g, o)
+    check_views(g, o, views=looked_at)
+    assert walked.stats.n_splat_writes == g.stats.n_splat_writes
+    assert np.array_equal(walked.keys, g.keys)
+
+
+@pytest.mark.parametrize("views,triangles", [(49, 49999), (49, 50000), (64, 49999), (64, 50000), (65, 149999),
+                                             (65, 150000), (96, 149999), (96, 150000)])
+def test_meshes_on_either_side_of_a_line(views, triangles):
+    _check(views, triangles)
