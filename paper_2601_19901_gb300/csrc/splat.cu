@@ -314,6 +314,9 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
     add_writes(a.ctr, writes);
 }
 
+// Cells of a sampling bias of eight pixels and more.
+__host__ __device__ __forceinline__ bool coarse_cells(const DispConst& c) { return c.bias_h * c.bias_v >= 8.0f; }
+
 template <int S, int P>
 __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     // With more than two slots the resolve is let in only when this block is
@@ -331,6 +334,7 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     // registers one more for the warps costs 96 views 3 %)
     const uint32_t n = __reduce_max_sync(0xffffffffu, a.ctr->n_work);
     const uint32_t wave = 4u * uint32_t(a.sm_count);
+    const bool coarse = coarse_cells(a.dc);
     uint32_t unit = 2u * P;
     // few points (often large cells, whose units are long): a unit for every warp
     // (2,048 points of 18,000 pixels over 48 views: 8.2 -> 1.9 ms a frame; of small
@@ -345,7 +349,7 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     // 48 views 572 us with neighbours, 587 with points from all over.)
     const bool spread = S <= 3 && units <= wave * kSplatWarps * kSpreadUnits;
     uint32_t blocks = gridDim.x;
-    if (P == unit_pairs(S)) blocks = min(blocks, wave * (1u + units / (wave * kSplatWarps * kUnitsPerWarp)));
+    if (P == unit_pairs(S) && !(S == 8 && coarse)) blocks = min(blocks, wave * (1u + units / (wave * kSplatWarps * kUnitsPerWarp)));
     if (blockIdx.x >= blocks) return;
     __syncthreads();
     const uint32_t n_warps = __reduce_max_sync(0xffffffffu, blocks * kSplatWarps);
@@ -539,10 +543,11 @@ cudaError_t splat_as(const FrameArgs& a, int grid, cudaStream_t s) {
     return launch_after_previous(k_splat<S, P>, dim3(grid), dim3(kSplatWarps * 32), bytes, s, a);
 }
 
-// Coarse cells, of a sampling bias of eight pixels and more, fill the passes of
-// small units and make large ones uneven: two pairs (one with more slots) and every
-// block, as 48 views of 420x560 at bias 16: 50,000 points 178 -> 158 us a frame,
-// 310,000 points 369 -> 336. Up to 16 views the large units are as good.
+// Coarse cells fill the passes of small units and make large ones uneven: two pairs
+// (one with more slots) and every block, as 48 views of 420x560 at bias 16: 50,000
+// points 178 -> 158 us a frame, 310,000 points 369 -> 336; 128 views, whose units are
+// of one pair anyway, 73,000 points 373 -> 338 with every block, 276,000 825 -> 788. Up
+// to 16 views the large units are as good.
 // With six slots so do those of meshes below 150,000 triangles, where the points
 // of a unit are too unlike for one of two pairs (82 and 96 views; 110,000 triangles,
 // textures of 256 texels 413 -> 367 and 458 -> 406 us a frame, of up to 4,096 423 ->
@@ -551,7 +556,7 @@ cudaError_t splat_as(const FrameArgs& a, int grid, cudaStream_t s) {
 template <int S>
 cudaError_t splat_one(const FrameArgs& a, int grid, cudaStream_t s) {
     constexpr int kFew = S <= 3 ? 2 : 1;
-    if (S > 1 && a.dc.bias_h * a.dc.bias_v >= 8.0f) return splat_as<S, (S == 1 ? unit_pairs(S) : kFew)>(a, grid, s);
+    if (S > 1 && coarse_cells(a.dc)) return splat_as<S, (S == 1 ? unit_pairs(S) : kFew)>(a, grid, s);
     if ((S == 6 && a.n_tris < 150000u) || (S == 4 && a.n_tris < 50000u))
         return splat_as<S, (S == 4 || S == 6 ? kFew : unit_pairs(S))>(a, grid, s);
     return splat_as<S, unit_pairs(S)>(a, grid, s);

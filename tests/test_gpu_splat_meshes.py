@@ -51,3 +51,10 @@ def _check(views, triangles, bias_h=1.0, bias_v=1.0, size=96):
                                              (65, 150000), (96, 149999), (96, 150000)])
 def test_meshes_on_either_side_of_a_line(views, triangles):
     _check(views, triangles)
+
+
+# views, triangles, bias: coarse cells with eight slots
+@pytest.mark.parametrize("views,triangles,bias_h,bias_v", [(97, 20000, 4.0, 2.0), (128, 20000, 4.0, 4.0),
+                                                           (130, 600, 8.0, 2.0)])
+def test_coarse_cells_of_many_views(views, triangles, bias_h, bias_v):
+    _check(views, triangles, bias_h, bias_v)
