@@ -336,10 +336,14 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     const uint32_t wave = 4u * uint32_t(a.sm_count);
     const bool coarse = coarse_cells(a.dc);
     uint32_t unit = 2u * P;
-    // few points (often large cells, whose units are long): a unit for every warp
-    // (2,048 points of 18,000 pixels over 48 views: 8.2 -> 1.9 ms a frame; of small
-    // cells, 7,000 points at 8 views, 44 -> 47 us)
-    if (S <= 3 && n < 2u * wave * kSplatWarps) unit = min(unit, max(1u, n / (wave * kSplatWarps)));
+    // few points, often of large cells, whose units are long, and coarse cells: a unit
+    // for every warp (2,048 points of 18,000 pixels over 48 views: 8.2 -> 1.9 ms a
+    // frame; 11,000 points at bias 32 over 8 and 48 views: 49 -> 38 and 97 -> 78 us).
+    // The units of small cells are cheap, and with one slot shorter than the passes
+    // that they fill: four points at least (15,000 points of two pixels at 8 views: 35
+    // us a frame with units of one, 31 so, 34 with units of twelve).
+    if (S <= 3 && (coarse || n < 2u * wave * kSplatWarps))
+        unit = min(unit, max(S == 1 && !coarse ? 4u : 1u, n / (wave * kSplatWarps)));
     const uint32_t units = (n + unit - 1u) / unit;
     // Neighbouring points are alike, and a unit of the coarse ones of a mesh is much
     // longer than the others: of few units, each takes its points from all over the

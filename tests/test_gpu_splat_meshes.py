@@ -58,3 +58,12 @@ def test_meshes_on_either_side_of_a_line(views, triangles):
                                                            (130, 600, 8.0, 2.0)])
 def test_coarse_cells_of_many_views(views, triangles, bias_h, bias_v):
     _check(views, triangles, bias_h, bias_v)
+
+
+# views, triangles, bias, view size: up to 48 views, units by the points a warp has
+@pytest.mark.parametrize("views,triangles,bias_h,bias_v,size", [(8, 10000, 4.0, 2.0, 160), (16, 20000, 8.0, 4.0, 200),
+                                                                (8, 5000, 6.0, 1.0, 96), (4, 300, 1.0, 1.0, 64),
+                                                                (24, 10000, 4.0, 2.0, 160), (48, 10000, 8.0, 4.0, 160),
+                                                                (48, 50000, 4.0, 4.0, 96)])
+def test_units_by_the_points(views, triangles, bias_h, bias_v, size):
+    _check(views, triangles, bias_h, bias_v, size)
