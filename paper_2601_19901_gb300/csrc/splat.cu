@@ -58,7 +58,8 @@ constexpr int kSplatWarps = 8;
 // 5,000 triangles at 48 views 125 -> 116 us a frame, at 96 views 201 -> 182; twelve
 // scenes of a batch 2.88 -> 2.77 ms; from 300,000 triangles on the same.
 constexpr uint32_t kUnitsPerWarp = 14;
-constexpr uint32_t kSpreadUnits = 20;   // units a warp of a wave up to which they are spread over the list
+// Units a warp of a wave up to which they are spread over the list (see k_splat).
+__host__ __device__ constexpr uint32_t spread_units(int S) { return S == 3 ? 40u : 20u; }
 
 // The per-pixel test; every condition is evaluated (no early exits), so the
 // lanes' different candidates do not diverge.
@@ -349,9 +350,11 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     // longer than the others: of few units, each takes its points from all over the
     // list. Of many it takes neighbours, which share triangles. (Meshes of 20,000 and
     // 110,000 triangles with textures of 256 texels a side: at 16 views 98 -> 72 and
-    // 160 -> 144 us a frame, at 48 views 182 -> 146 and 284 -> 258; 10^6 triangles at
-    // 48 views 572 us with neighbours, 587 with points from all over.)
-    const bool spread = S <= 3 && units <= wave * kSplatWarps * kSpreadUnits;
+    // 160 -> 144 us a frame, at 48 views 182 -> 146 and 284 -> 258; 200,000 triangles,
+    // 10^6 points, 40 and 48 views 357 -> 340 and 394 -> 374, the line at 40 units a warp
+    // instead of 20; 10^6 triangles at 48 views 572 us with neighbours, 587 with points
+    // from all over, at 24 views 443 and 455.)
+    const bool spread = S <= 3 && units <= wave * kSplatWarps * spread_units(S);
     uint32_t blocks = gridDim.x;
     if (P == unit_pairs(S) && !(S == 8 && coarse)) blocks = min(blocks, wave * (1u + units / (wave * kSplatWarps * kUnitsPerWarp)));
     if (blockIdx.x >= blocks) return;

@@ -23,20 +23,21 @@ def _lib():
     lfdpr.lib()
 
 
-def _mesh(triangles):
+def _mesh(triangles, texels=256):
     """Displaced surfaces of 5,000 triangles each, cut to the number asked for."""
     sc = S.geometry_paper(n_instances=-(-triangles // 5000), res=50, n_textures=2, seed=5, r_max=0.5)
     return replace(sc, idx=sc.idx[:triangles], tri_tex=sc.tri_tex[:triangles],
-                   textures=[S.value_noise_texture(64, 64, 7), S.value_noise_texture(256, 256, 8)])
+                   textures=[S.value_noise_texture(max(64, texels // 4), max(64, texels // 4), 7), S.value_noise_texture(texels, texels, 8)])
 
 
-def _check(views, triangles, bias_h=1.0, bias_v=1.0, size=96):
+def _check(views, triangles, bias_h=1.0, bias_v=1.0, size=96, texels=256):
     d = replace(S.display_paper(), n_views=views, view_w=size, view_h=size + 8, focal_w=2.4 * size / (size + 8),
                 bias_h=bias_h, bias_v=bias_v)
-    sc, m = _mesh(triangles), S.model_matrix(4)
+    sc, m = _mesh(triangles, texels), S.model_matrix(4)
     looked_at = sorted({0, views // 2, views - 1})
     o = O.render(d, sc, m, views=looked_at, panel=False)
-    with lfdpr.Renderer(d, sc, len(o.points) + 1) as R:
+    n = len(o.points)
+    with lfdpr.Renderer(d, sc, n + 1) as R:
         g = gpu_frame(d, sc, m, renderer=R, panel=False)
         lfdpr.lfdpr_set_splat_lane_limit(R.disp, 3)
         walked = gpu_frame(d, sc, m, renderer=R, panel=False)
@@ -45,6 +46,7 @@ def _check(views, triangles, bias_h=1.0, bias_v=1.0, size=96):
     check_views(g, o, views=looked_at)
     assert walked.stats.n_splat_writes == g.stats.n_splat_writes
     assert np.array_equal(walked.keys, g.keys)
+    return n
 
 
 @pytest.mark.parametrize("views,triangles", [(49, 49999), (49, 50000), (64, 49999), (64, 50000), (65, 149999),
@@ -67,3 +69,12 @@ def test_coarse_cells_of_many_views(views, triangles, bias_h, bias_v):
                                                                 (48, 50000, 4.0, 4.0, 96)])
 def test_units_by_the_points(views, triangles, bias_h, bias_v, size):
     _check(views, triangles, bias_h, bias_v, size)
+
+
+# views, view size: points on either side of the line between units of points
+# from all over the list and of neighbours (1.2, 0.8 and 1.2 million points for one, two
+# and three slots)
+@pytest.mark.parametrize("views,size,least,most", [(48, 140, 3e5, 1.2e6), (40, 300, 2.4e6, 6e6), (24, 120, 3e5, 8e5),
+                                                   (24, 300, 2.4e6, 6e6), (8, 140, 3e5, 1.2e6), (8, 300, 2.4e6, 6e6)])
+def test_many_points(views, size, least, most):
+    assert least < _check(views, 100000, 0.2, 0.2, size, 2048) < most
