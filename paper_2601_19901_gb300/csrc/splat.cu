@@ -559,12 +559,17 @@ cudaError_t splat_as(const FrameArgs& a, int grid, cudaStream_t s) {
 // of a unit are too unlike for one of two pairs (82 and 96 views; 110,000 triangles,
 // textures of 256 texels 413 -> 367 and 458 -> 406 us a frame, of up to 4,096 423 ->
 // 447; from 200,000 on two pairs gain: 10^6 triangles 912 -> 836), and with four
-// below 50,000 (60 views, 20,000 triangles: 148 -> 139 and 193 -> 170).
+// below 50,000 (60 views, 20,000 triangles: 148 -> 139 and 193 -> 170). A sampling
+// bias leaves fewer and coarser points to the same triangles: with six slots the
+// line is their number over the root of the bias (200,000 triangles at 96 views,
+// bias 2, 4 and 6: 568, 603 and 546 us with one pair, 573, 627 and 556 with two
+// whatever the bias, 550, 587 and 533 now; 10^6 at bias 6 784 and 721).
 template <int S>
 cudaError_t splat_one(const FrameArgs& a, int grid, cudaStream_t s) {
     constexpr int kFew = S <= 3 ? 2 : 1;
     if (S > 1 && coarse_cells(a.dc)) return splat_as<S, (S == 1 ? unit_pairs(S) : kFew)>(a, grid, s);
-    if ((S == 6 && a.n_tris < 150000u) || (S == 4 && a.n_tris < 50000u))
+    const double tris = double(a.n_tris), bias = double(a.dc.bias_h) * a.dc.bias_v;
+    if ((S == 6 && tris * tris < 150000.0 * 150000.0 * bias) || (S == 4 && a.n_tris < 50000u))
         return splat_as<S, (S == 4 || S == 6 ? kFew : unit_pairs(S))>(a, grid, s);
     return splat_as<S, unit_pairs(S)>(a, grid, s);
 }

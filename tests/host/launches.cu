@@ -25,11 +25,12 @@ lfdpr_status cuda_fail(cudaError_t, const char*) { return LFDPR_ECUDA; }
 
 using namespace lfdpr;
 
-static cudaError_t splat(int views, uint32_t tris) {
+static cudaError_t splat(int views, uint32_t tris, float bias = 1.0f) {
     FrameArgs a{};
     a.n_tris = tris;
     a.sm_count = 152;
-    a.dc.bias_h = a.dc.bias_v = 1.0f;
+    a.dc.bias_h = bias;
+    a.dc.bias_v = 1.0f;
     a.dc.nr = a.view_hi = views;
     return launch_splat(a, nullptr);
 }
@@ -99,6 +100,25 @@ static void gauss() {
     }
 }
 
+// units of one or two pairs of points (shared memory) with four and six slots
+static void units() {
+    const struct {
+        int views;
+        uint32_t tris;
+        float bias;
+        bool two;
+    } cases[] = {{49, 49999, 1.0f, false},   {49, 50000, 1.0f, true},   {64, 50000, 4.0f, true},   {64, 50000, 8.0f, false},
+                 {65, 149999, 1.0f, false},  {65, 150000, 1.0f, true},  {96, 200000, 1.0f, true},  {96, 200000, 2.0f, false},
+                 {96, 200000, 6.0f, false},  {96, 300000, 3.9f, true},  {82, 1000000, 6.0f, true}, {82, 1000000, 8.0f, false},
+                 {96, 100000, 0.25f, true}};
+    for (const auto& k : cases) {
+        char what[96];
+        snprintf(what, sizeof what, "units of %d views, %u triangles, bias %g", k.views, k.tris, k.bias);
+        const int slots = k.views <= 64 ? 4 : 6;
+        check(splat(k.views, k.tris, k.bias) == cudaSuccess && (g_last_smem >= 8u * 2u * 32u * slots * 16u) == k.two, what);
+    }
+}
+
 // a lens pitch whose reciprocal overflows: the lens phase is no number
 static void tiny_pitch() {
     for (int recon : {2, 3}) {
@@ -151,6 +171,7 @@ int main(int, char** argv) {
     if (!strcmp(argv[1], "tiny_pitch")) tiny_pitch();
     if (!strcmp(argv[1], "tent")) tent();
     if (!strcmp(argv[1], "gauss")) gauss();
+    if (!strcmp(argv[1], "units")) units();
     check(g_launched > 0, "something was launched");
     return g_failed;
 }

@@ -55,6 +55,11 @@ def test_meshes_on_either_side_of_a_line(views, triangles):
     _check(views, triangles)
 
 
+@pytest.mark.parametrize("triangles,bias_h,bias_v", [(150000, 2.0, 1.0), (220000, 2.0, 1.0), (120000, 0.5, 1.0)])
+def test_the_line_moves_with_the_bias(triangles, bias_h, bias_v):
+    _check(70, triangles, bias_h, bias_v)
+
+
 # views, triangles, bias: coarse cells with eight slots
 @pytest.mark.parametrize("views,triangles,bias_h,bias_v", [(97, 20000, 4.0, 2.0), (128, 20000, 4.0, 4.0),
                                                            (130, 600, 8.0, 2.0)])
