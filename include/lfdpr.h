@@ -17,10 +17,11 @@
  *  - Output buffers are owned by the caller.
  *  - `stream` is a cudaStream_t (NULL = the legacy default stream). Calls that
  *    launch work are asynchronous with respect to the host on that stream.
- *    A frame's kernels after the first are launched as programmatic
- *    dependents of the kernel before them (their launch overlaps its last
- *    blocks) and wait for it before touching memory, so stream order holds
- *    for the caller's own work as for plain launches. Each of them lets the
+ *    A frame's kernels are launched as programmatic dependents of the kernel
+ *    before them on the stream, the first one of the caller's own last kernel
+ *    (their launch overlaps its last blocks), and wait for it before touching
+ *    memory, so stream order holds for the caller's own work as for plain
+ *    launches. Each of them lets the
  *    next kernel start early, so a kernel of the caller's that is itself
  *    launched with programmatic stream serialization right after a call must
  *    wait for its predecessor (griddepcontrol.wait) before reading the
@@ -160,7 +161,8 @@ enum {
  *                                            metallic tv_min, tv_max bytes (R channels; meshes of
  *                                            materials)
  *  resolve_mat u32 [max_points][2]           normal-map tv_min, tv_max RGBA8 (meshes of materials;
- *                                            NULL before the display's first such mesh)
+ *                                            NULL before the display's first such mesh; written for
+ *                                            this inspection alone: the resolve reads a copy)
  */
 typedef struct {
     const uint32_t *counts, *offsets, *points;
@@ -291,7 +293,7 @@ lfdpr_status lfdpr_set_stage_timing(lfdpr_display *disp, int32_t enable);
 
 /*
  * lfdpr_set_splat_lane_limit: the splat (Sec. 3.2) pools the candidate
- * pixels of four points per warp into 32-lane passes numbered with 32-bit
+ * pixels of a unit of one to twelve points per warp into 32-lane passes numbered with 32-bit
  * integers; a unit in which some lane's views hold `limit` or more candidates
  * (huge cells) is instead walked segment by segment, one lane per (point,
  * view). The default, and the largest value, 2^24, keeps every number below
@@ -456,7 +458,8 @@ lfdpr_status lfdpr_set_shading(lfdpr_display *disp, const lfdpr_shading *shading
  * count, view size, panel), rendered and interleaved together. One call runs
  * every scene's frame, Sec. 3.1-4 as lfdpr_render_frame followed by
  * lfdpr_interleave, as one CUDA graph: the scenes' frames on `branches`
- * concurrent graph branches (scene i on branch i mod branches), each
+ * concurrent graph branches (scene i on branch i mod branches; of more scenes
+ * than branches, a branch samples one while it splats the one before), each
  * interleaved into its display's own panel buffer (lfdpr_batch_panel). The
  * graph is captured on the first lfdpr_render_batch after creation or a
  * configuration change; later calls replay it with new model matrices. Each

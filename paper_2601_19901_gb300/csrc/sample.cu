@@ -1332,8 +1332,8 @@ __global__ void __launch_bounds__(256) k_near_work(FrameArgs a) {
 // The normal, roughness and metallic maps of every point of a mesh of
 // materials (run after k_fetch): each texture at its own Eq. 6-7 LOD pair
 // (the record's size_vpuv bounds and its resolution), at the cell centre's
-// texture coordinate (as k_fetch); the normal map's two RGBA8 values go to
-// rmat, the roughness and metallic R channels to the resolve record's b.w as
+// texture coordinate (as k_fetch); the normal map's two RGBA8 values go to the
+// shading record (and to rmat, for inspection alone), the roughness and metallic R channels to the resolve record's b.w as
 // bytes (min, max, min, max).
 // Bound by issue and the texel gathers. 2.6 M points, maps of three sizes: 146 us
 // with two logarithms a map, an unconditional third level and a 16-byte record;
