@@ -626,10 +626,10 @@ __device__ __forceinline__ int last_at_most(const uint32_t* s_num, uint32_t k) {
 // columns, and its stores are contiguous.
 //
 // Meshes whose 256-triangle blocks do not fill the SMs spread each over `split`
-// blocks (each scans all 256 counts and emits its share of the triangles: of those
-// emitted by a thread neighbours, in whole warps, of the others every split-th where
-// that is more than every second, so that a few large triangles are shared out too:
-// eight of 28,000 points each 184 us in one block, 32 in eight).
+// blocks (each scans all 256 counts and emits its share of the triangles: neighbours,
+// in whole warps; of a mesh of one block every split-th of those that are not a
+// thread's own, so that a few large triangles are shared out too: eight of 28,000
+// points each 184 us in one block, 32 in eight).
 // Bound by the dependent chain of a block's largest triangle while one thread or
 // one warp emits it; shared out, by the searches and stores of its points.
 // Measured on twelve meshes of 61 k to 1.2 M points (24 to 96 views): 608 us
@@ -657,7 +657,7 @@ __global__ void __launch_bounds__(kSetupThreads) k_emit(FrameArgs a, uint32_t sp
     // meshes a block's chain of loads is the kernel's time: 2,048 triangles 8.0 ->
     // 6.3 us, 10^6 31.7 -> 30.7)
     const uint32_t cnt = t < a.n_tris ? a.counts[t] : 0u;
-    const uint32_t near = threadIdx.x / width, far = split > 2u ? threadIdx.x % split : near;
+    const uint32_t near = threadIdx.x / width, far = a.n_blocks == 1u ? threadIdx.x % split : near;
     uint4 cs = make_uint4(kColSumWalk, 0u, 0u, 0u);
     if (t < a.n_tris && (near == part || far == part) && a.colsum) cs = __ldcg(a.colsum + t);
     const bool big = cnt > kEmitOwn, mine = t < a.n_tris && (big ? far : near) == part;
