@@ -341,10 +341,11 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     // for every warp (2,048 points of 18,000 pixels over 48 views: 8.2 -> 1.9 ms a
     // frame; 11,000 points at bias 32 over 8 and 48 views: 49 -> 38 and 97 -> 78 us).
     // The units of small cells are cheap, and with one slot shorter than the passes
-    // that they fill: four points at least (15,000 points of two pixels at 8 views: 35
-    // us a frame with units of one, 31 so, 34 with units of twelve).
+    // that they fill: two points at least (15,000 points of two pixels at 8 views: 35
+    // us a frame with units of one, 33 so; four would be better there, 31, and worse
+    // where textures of few texels leave large cells, 69 -> 70).
     if (S <= 3 && (coarse || n < 2u * wave * kSplatWarps))
-        unit = min(unit, max(S == 1 && !coarse ? 4u : 1u, n / (wave * kSplatWarps)));
+        unit = min(unit, max(S == 1 && !coarse ? 2u : 1u, n / (wave * kSplatWarps)));
     const uint32_t units = (n + unit - 1u) / unit;
     // Neighbouring points are alike, and a unit of the coarse ones of a mesh is much
     // longer than the others: of few units, each takes its points from all over the
