@@ -468,7 +468,7 @@ lfdpr_status lfdpr_set_shading(lfdpr_display *disp, const lfdpr_shading *shading
 typedef struct {
     int32_t branches;             /* concurrent graph branches, 1..32 */
     int32_t splat_blocks_per_sm;  /* splat grid: at most this many blocks of 256 threads per SM, 1..64
-                                     (of which an SM holds four at once; no more are launched) */
+                                     (an SM holds four at once; more only where a scene gains by them) */
     int32_t splat_slots;          /* most views per lane in the splat: 1, 2, 3, 4, 6 or 8 */
 } lfdpr_batch_config;
 

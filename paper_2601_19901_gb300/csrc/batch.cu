@@ -104,14 +104,18 @@ lfdpr_status record_batch(lfdpr_batch* b) {
     CK(cudaEventRecordWithFlags(b->tev[0], s, cudaEventRecordExternal), "batch: start event");
     CK(cudaEventRecord(fork, s), "batch: fork");
     for (int j = 0; j < n_streams; j++) CK(cudaStreamWaitEvent(b->br[j], fork, 0), "batch: branch wait");
-    // A wave of the splat's blocks, whatever the configuration asks for beyond it: a
-    // splat of few points ends with the blocks it has no units for, and beside other
-    // scenes one wave is enough for many. 32 scenes of 5,000 triangles, 24 views: 768
-    // us with 16 blocks per SM and one stream a branch, 678 with four blocks, 662 with
-    // two streams as well (620 with one splat over all scenes, which took 1145
-    // against 941 for 12 scenes of 20,000 at 96 views); 64 of 1,000, 4 views 1144, 956
-    // and 699; 12 of 5,000 to 200,000 triangles, 24 to 96 views 2766, 2724 and 2685.
-    const int splat_blocks = std::min(b->cfg.splat_blocks_per_sm, 4);
+    // No more than a wave of the splat's blocks where they only take as many as their
+    // units fill, or where scenes wait for branches: a splat of few points ends with
+    // the blocks it has no units for, and beside other scenes one wave is enough for
+    // many. 32 scenes of 5,000 triangles, 24 views: 768 us with 16 blocks per SM and one
+    // stream a branch, 678 with four blocks, 662 with two streams as well (620 with one
+    // splat over all scenes, which took 1145 against 941 for 12 scenes of 20,000 at 96
+    // views); 64 of 1,000, 4 views 1144, 956 and 699; 12 of 5,000 to 200,000 triangles,
+    // 24 to 96 views 2766, 2724 and 2685. Scenes that wait for none keep every block
+    // where units are few and long (three of 4,000 to 15,000 triangles, 24 to 96 views
+    // 567 us, 621 with a wave).
+    const int wave = std::min(b->cfg.splat_blocks_per_sm, 4);
+    const int splat_blocks = b->n > K ? wave : b->cfg.splat_blocks_per_sm;
     for (int i = 0; i < b->n; i++) {
         cudaStream_t front = b->br[i % K], back = b->br[n_streams - K + i % K];
         FrameArgs a = frame_args(b->disp[i], b->mesh[i]);
@@ -123,7 +127,7 @@ lfdpr_status record_batch(lfdpr_batch* b) {
             CK(cudaEventRecord(fetched, front), "batch: fetched");
             CK(cudaStreamWaitEvent(back, fetched, 0), "batch: splat wait");
         }
-        CK(launch_splat(a, back, splat_blocks, b->cfg.splat_slots), "launch k_splat");
+        CK(launch_splat(a, back, splat_blocks, wave, b->cfg.splat_slots), "launch k_splat");
         CK(launch_resolve(a, back), "launch k_resolve");
         lfdpr_display* d = b->disp[i];
         if ((d->desc.recon == 2 || d->desc.recon == 3) && d->n_samples == 0)

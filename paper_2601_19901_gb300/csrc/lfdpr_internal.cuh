@@ -419,8 +419,10 @@ cudaError_t launch_emit(const FrameArgs& a, cudaStream_t s);
 cudaError_t launch_fetch(const FrameArgs& a, cudaStream_t s);
 cudaError_t launch_fetch_mat(const FrameArgs& a, cudaStream_t s);   // meshes of materials, after launch_fetch
 cudaError_t launch_near_work(const FrameArgs& a, cudaStream_t s);   // after launch_fetch
-// blocks_per_sm blocks per SM, at most max_slots views per lane (1, 2, 3, 4, 6 or 8).
-cudaError_t launch_splat(const FrameArgs& a, cudaStream_t s, int blocks_per_sm = 16, int max_slots = 8);
+// blocks_per_sm blocks per SM (at most filled_per_sm where the kernel takes as many as
+// its units fill), at most max_slots views per lane (1, 2, 3, 4, 6 or 8).
+cudaError_t launch_splat(const FrameArgs& a, cudaStream_t s, int blocks_per_sm = 16, int filled_per_sm = 16,
+                         int max_slots = 8);
 constexpr int kMaxBatchScenes = 64;    // the interface's limits (include/lfdpr.h)
 constexpr int kMaxBatchViews = 4096;   // rendered views summed over a batch
 cudaError_t launch_resolve(const FrameArgs& a, cudaStream_t s);

@@ -318,6 +318,12 @@ __device__ __forceinline__ void splat_units(const FrameArgs& a, uint32_t n, uint
 // Cells of a sampling bias of eight pixels and more.
 __host__ __device__ __forceinline__ bool coarse_cells(const DispConst& c) { return c.bias_h * c.bias_v >= 8.0f; }
 
+// Whether a splat takes no more blocks than its units fill (else every block).
+template <int S, int P>
+__host__ __device__ __forceinline__ bool fills_blocks(const DispConst& c) {
+    return P == unit_pairs(S) && !(S == 8 && coarse_cells(c));
+}
+
 template <int S, int P>
 __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     // With more than two slots the resolve is let in only when this block is
@@ -357,7 +363,7 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 4) k_splat(FrameArgs a) {
     // from all over, at 24 views 443 and 455.)
     const bool spread = S <= 3 && units <= wave * kSplatWarps * spread_units(S);
     uint32_t blocks = gridDim.x;
-    if (P == unit_pairs(S) && !(S == 8 && coarse)) blocks = min(blocks, wave * (1u + units / (wave * kSplatWarps * kUnitsPerWarp)));
+    if (fills_blocks<S, P>(a.dc)) blocks = min(blocks, wave * (1u + units / (wave * kSplatWarps * kUnitsPerWarp)));
     if (blockIdx.x >= blocks) return;
     __syncthreads();
     const uint32_t n_warps = __reduce_max_sync(0xffffffffu, blocks * kSplatWarps);
@@ -537,18 +543,25 @@ __global__ void __launch_bounds__(256) k_resolve_pbr(FrameArgs a) {
     reinterpret_cast<uint32_t*>(a.views)[o] = out;
 }
 
+// Blocks per SM of a splat: all of them, and at most where the kernel takes as many
+// as its units fill.
+struct SplatGrid {
+    int all, filled;
+};
+
 // Launch with the per-warp pooling buffers as dynamic shared memory. Beyond 48 KB
 // (with the kernel's eye positions) the launch needs the attribute, which holds for
 // the current device only: it is set at every such launch.
 template <int S, int P>
-cudaError_t splat_as(const FrameArgs& a, int grid, cudaStream_t s) {
+cudaError_t splat_as(const FrameArgs& a, const SplatGrid& grid, cudaStream_t s) {
     constexpr size_t bytes = kSplatWarps * sizeof(SplatWarpSmem<S, P>);
     if (bytes + sizeof(float) * kMaxRenderViews > 48u * 1024u) {
         const cudaError_t e =
             cudaFuncSetAttribute(k_splat<S, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
         if (e != cudaSuccess) return e;
     }
-    return launch_after_previous(k_splat<S, P>, dim3(grid), dim3(kSplatWarps * 32), bytes, s, a);
+    const int per_sm = fills_blocks<S, P>(a.dc) ? grid.filled : grid.all;
+    return launch_after_previous(k_splat<S, P>, dim3(a.sm_count * per_sm), dim3(kSplatWarps * 32), bytes, s, a);
 }
 
 // Coarse cells fill the passes of small units and make large ones uneven: two pairs
@@ -566,7 +579,7 @@ cudaError_t splat_as(const FrameArgs& a, int grid, cudaStream_t s) {
 // bias 2, 4 and 6: 568, 603 and 546 us with one pair, 573, 627 and 556 with two
 // whatever the bias, 550, 587 and 533 now; 10^6 at bias 6 784 and 721).
 template <int S>
-cudaError_t splat_one(const FrameArgs& a, int grid, cudaStream_t s) {
+cudaError_t splat_one(const FrameArgs& a, const SplatGrid& grid, cudaStream_t s) {
     constexpr int kFew = S <= 3 ? 2 : 1;
     if (S > 1 && coarse_cells(a.dc)) return splat_as<S, (S == 1 ? unit_pairs(S) : kFew)>(a, grid, s);
     const double tris = double(a.n_tris), bias = double(a.dc.bias_h) * a.dc.bias_v;
@@ -579,11 +592,12 @@ cudaError_t splat_one(const FrameArgs& a, int grid, cudaStream_t s) {
 
 LFDPR_CHECK_READER(checks_splat)
 
-cudaError_t launch_splat(const FrameArgs& a, cudaStream_t s, int blocks_per_sm, int max_slots) {
+cudaError_t launch_splat(const FrameArgs& a, cudaStream_t s, int blocks_per_sm, int filled_per_sm, int max_slots) {
     // the fewest view slots per lane that hold every view of the range
     // [view_lo, view_hi) in one group (more than 16 max_slots views take
     // several groups)
-    const int nr = a.view_hi - a.view_lo, grid = a.sm_count * blocks_per_sm;
+    const int nr = a.view_hi - a.view_lo;
+    const SplatGrid grid{blocks_per_sm, filled_per_sm};
     const int slots = min((nr + 15) / 16, max_slots);
     if (slots <= 1) return splat_one<1>(a, grid, s);
     if (slots <= 2) return splat_one<2>(a, grid, s);
