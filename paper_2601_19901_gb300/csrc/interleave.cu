@@ -142,8 +142,8 @@ constexpr int kTentCols = 4 * kTentThreads;
 constexpr int kStageCols = 4;                 // 32-column runs of a row segment loaded together
 
 // Rendered views from which a tile is staged run after run of all views, two
-// views' loads in flight a warp; fewer leave a warp one view, and its whole segment
-// is loaded in turn (48 views of 1024x768 to 1920x1080: 62.8 us run after run, 71.2
+// views' loads in flight a warp; fewer leave a warp one view, and its whole segment,
+// where it is longer than a run, is loaded in turn (48 views of 1024x768 to 1920x1080: 62.8 us run after run, 71.2
 // view after view; 5 of 4000x1000 to 1000x500: 21.8 and 13.8).
 constexpr int kTileManyViews = 16;
 
@@ -156,7 +156,9 @@ __device__ __forceinline__ bool first_row_of(const DispConst& c, int sy, int& y)
 
 // Block (strip bx, view row sy): view pixels sx_lo..sx_lo + n - 1 of row sy
 // for every rendered view, then the panel rows whose source row is sy.
-__global__ void __launch_bounds__(kTileThreads) k_interleave_tile(DispConst c, const uint8_t* __restrict__ views,
+// (Six blocks an SM, as before the two orders of staging: at five a frame of 61 views
+// of 341x143 takes 68.6 us instead of 65.5.)
+__global__ void __launch_bounds__(kTileThreads, 6) k_interleave_tile(DispConst c, const uint8_t* __restrict__ views,
                                                                   uint8_t* __restrict__ panel, int cols, int stride) {
     wait_previous_kernel();
     allow_next_kernel();
@@ -171,7 +173,7 @@ __global__ void __launch_bounds__(kTileThreads) k_interleave_tile(DispConst c, c
     const uint32_t* v32 = reinterpret_cast<const uint32_t*>(views);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr int kWarps = kTileThreads / 32;
-    if (c.nr < kTileManyViews) {
+    if (c.nr < kTileManyViews && n > 32 * kStageCols) {
         for (int m = warp; m < c.nr; m += kWarps) {
             const uint32_t* src = v32 + (uint64_t)m * npix + (uint64_t)sy * c.W + sx_lo;
             for (int i = lane; i < n; i += 32)
