@@ -803,6 +803,12 @@ __global__ void __launch_bounds__(256) k_view_mip(const uint8_t* __restrict__ sr
 
 LFDPR_CHECK_READER(checks_interleave)
 
+void prefer_view_mip_split() {
+    for (const void* k : {reinterpret_cast<const void*>(k_view_mip<1>), reinterpret_cast<const void*>(k_view_mip<2>)})
+        if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, kViewsSplit) != cudaSuccess)
+            cudaGetLastError();
+}
+
 cudaError_t launch_view_mip(const uint8_t* views, int W, int H, int nr, int level, uint8_t* out, cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);

@@ -423,6 +423,20 @@ cudaError_t launch_near_work(const FrameArgs& a, cudaStream_t s);   // after lau
 // its units fill), at most max_slots views per lane (1, 2, 3, 4, 6 or 8).
 cudaError_t launch_splat(const FrameArgs& a, cudaStream_t s, int blocks_per_sm = 16, int filled_per_sm = 16,
                          int max_slots = 8);
+// The split of an SM's memory between L1 and shared memory that the kernels
+// between the splat and the interleave ask for on the current device (a hint, in
+// per cent of the most shared memory: 100 of 228 KB). An SM changes its split only
+// while it is idle, which programmatic launches leave it no time for: without the
+// hint the resolve, the view mips and then the interleave ran under the splat's
+// split, of little L1, or under one too small for more than a block or two of the
+// interleave. 100 KB hold four blocks of the Gaussian interleave. Whole passes
+// without and with it: 88 views of 368x399, Gaussian, 855 -> 547 us, 86 of 138x253
+// 344 -> 240, 38 of 607x610, tent, 575 -> 557, 14 of 243x152 to a host panel 195 ->
+// 144, 96 of 420x560, Gaussian, 1060 -> 1041; at 25 to 70 per cent instead of 42 the
+// Gaussian ones are 0 to 14 % slower.
+constexpr int kViewsSplit = 42;
+void prefer_resolve_split();
+void prefer_view_mip_split();
 constexpr int kMaxBatchScenes = 64;    // the interface's limits (include/lfdpr.h)
 constexpr int kMaxBatchViews = 4096;   // rendered views summed over a batch
 cudaError_t launch_resolve(const FrameArgs& a, cudaStream_t s);

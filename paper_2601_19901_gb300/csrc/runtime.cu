@@ -542,6 +542,8 @@ lfdpr_status lfdpr_create_display(const lfdpr_display_desc* desc, lfdpr_display*
     d->max_points = uint32_t(d->desc.max_points);
     CK(cudaGetDevice(&d->device), "cudaGetDevice");
     CK(cudaDeviceGetAttribute(&d->sm_count, cudaDevAttrMultiProcessorCount, d->device), "sm count");
+    prefer_resolve_split();
+    prefer_view_mip_split();
 
     DispConst& c = d->dc;
     c.n_views = s.n_views;

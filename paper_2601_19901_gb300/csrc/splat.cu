@@ -607,6 +607,12 @@ cudaError_t launch_splat(const FrameArgs& a, cudaStream_t s, int blocks_per_sm, 
     return splat_one<8>(a, grid, s);
 }
 
+void prefer_resolve_split() {
+    for (const void* k : {reinterpret_cast<const void*>(k_resolve), reinterpret_cast<const void*>(k_resolve_pbr)})
+        if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, kViewsSplit) != cudaSuccess)
+            cudaGetLastError();
+}
+
 cudaError_t launch_resolve(const FrameArgs& a, cudaStream_t s) {
     const uint32_t npix = uint32_t(a.dc.W) * uint32_t(a.dc.H);
     const uint32_t nv = uint32_t(a.view_hi - a.view_lo);

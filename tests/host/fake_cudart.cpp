@@ -15,6 +15,7 @@ void (*g_meanwhile)() = nullptr;
 int g_launched = 0;
 size_t g_last_smem = 0;
 unsigned g_last_blocks = 0;
+int g_splits = 0;
 
 namespace {
 cudaError_t g_last = cudaSuccess;
@@ -53,6 +54,7 @@ cudaError_t cudaFuncSetAttribute(const void* kernel, cudaFuncAttribute a, int v)
         g_fail_attributes--;
         return cudaErrorMemoryAllocation;
     }
+    if (a == cudaFuncAttributePreferredSharedMemoryCarveout) g_splits++;
     if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) {
         g_limit[{kernel, g_device}] = v;
         if (void (*other)() = g_meanwhile) {

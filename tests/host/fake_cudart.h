@@ -7,3 +7,4 @@ extern void (*g_meanwhile)();      // another thread's call, right after an attr
 extern int g_launched;             // launches that were not refused
 extern size_t g_last_smem;         // the last one's dynamic shared memory
 extern unsigned g_last_blocks;     // and blocks
+extern int g_splits;               // kernels that were given a split of L1 and shared memory

@@ -145,6 +145,17 @@ static void devices() {
     }
 }
 
+// both resolves and both view mips ask for their split; a refusal is no error
+static void splits() {
+    prefer_resolve_split();
+    prefer_view_mip_split();
+    check(g_splits == 4, "splits of the kernels between splat and interleave");
+    g_fail_attributes = 4;
+    prefer_resolve_split();
+    prefer_view_mip_split();
+    check(splat(48, 1000u) == cudaSuccess && cudaGetLastError() == cudaSuccess, "a refused split");
+}
+
 // a call after a failed one
 static void retry() {
     g_fail_attributes = 1;
@@ -172,6 +183,7 @@ int main(int, char** argv) {
     if (!strcmp(argv[1], "tent")) tent();
     if (!strcmp(argv[1], "gauss")) gauss();
     if (!strcmp(argv[1], "units")) units();
+    if (!strcmp(argv[1], "splits")) splits();
     check(g_launched > 0, "something was launched");
     return g_failed;
 }

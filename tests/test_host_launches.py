@@ -34,7 +34,7 @@ def test_shared_memory_is_allowed_where_a_launch_needs_it(program, what):
     assert r.returncode == 0, r.stdout
 
 
-@pytest.mark.parametrize("what", ["tent", "gauss", "units"])
+@pytest.mark.parametrize("what", ["tent", "gauss", "units", "splits"])
 def test_a_launch_takes_the_form_that_is_faster(program, what):
     r = subprocess.run([program, what], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout
