@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kWarpThreads) k_warp_views(WarpArgs a) {
 // block per (row y, input interval j). Its 256 threads sweep (view, pixel) pairs
 // of a pass as one range, so that a short row leaves none idle, and it picks its
 // own interval's views out of all instead of sorting them.
-constexpr int kMaxRowsWidth = 512;   // 43 KB of shared memory
+constexpr int kMaxRowsWidth = 512;   // 39 KB of shared memory
 __global__ void __launch_bounds__(kWarpThreads) k_warp_rows(WarpArgs a) {
     extern __shared__ __align__(16) uint8_t s_raw[];
     const int y = blockIdx.x, j = blockIdx.y, W = a.W, V = views_per_pass(W);
