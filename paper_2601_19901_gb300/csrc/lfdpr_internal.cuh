@@ -432,9 +432,10 @@ cudaError_t launch_splat(const FrameArgs& a, cudaStream_t s, int blocks_per_sm =
 // interleave. 100 KB hold four blocks of the Gaussian interleave. Whole passes
 // without and with it: 88 views of 368x399, Gaussian, 855 -> 547 us, 86 of 138x253
 // 344 -> 240, 38 of 607x610, tent, 575 -> 557, 14 of 243x152 to a host panel 195 ->
-// 144, 96 of 420x560, Gaussian, 1060 -> 1041; small plain frames lose 1 to 2 (5 views of
-// 168x532 99.4 -> 101.8). At 25 to 70 per cent instead of 42 the Gaussian ones are 0 to
-// 14 % slower.
+// 144, 96 of 420x560, Gaussian, 1060 -> 1041; 122 frames of random
+// sizes: Gaussian 58 to 100 % of the time (93 in the mean), the others 91 to 106 (99.4;
+// the most that one loses is 8 views of 275x189 to 2202x1462, 47.3 -> 50.0). At 25 to
+// 70 per cent instead of 42 the Gaussian ones are 0 to 14 % slower.
 constexpr int kViewsSplit = 42;
 void prefer_resolve_split();
 void prefer_view_mip_split();
