@@ -156,9 +156,11 @@ __device__ __forceinline__ bool first_row_of(const DispConst& c, int sy, int& y)
 
 // Block (strip bx, view row sy): view pixels sx_lo..sx_lo + n - 1 of row sy
 // for every rendered view, then the panel rows whose source row is sy.
-// (Six blocks an SM, as before the two orders of staging: at five a frame of 61 views
-// of 341x143 takes 68.6 us instead of 65.5.)
-__global__ void __launch_bounds__(kTileThreads, 6) k_interleave_tile(DispConst c, const uint8_t* __restrict__ views,
+// InTurn: view after view. (A kernel for each order: with both in one, at five blocks
+// an SM a frame of 61 views of 341x143 took 68.6 us instead of 65.5, and held to six
+// one of 65 of 174x182 to a host panel 130.7 instead of 126.6.)
+template <bool InTurn>
+__global__ void __launch_bounds__(kTileThreads) k_interleave_tile(DispConst c, const uint8_t* __restrict__ views,
                                                                   uint8_t* __restrict__ panel, int cols, int stride) {
     wait_previous_kernel();
     allow_next_kernel();
@@ -173,7 +175,7 @@ __global__ void __launch_bounds__(kTileThreads, 6) k_interleave_tile(DispConst c
     const uint32_t* v32 = reinterpret_cast<const uint32_t*>(views);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr int kWarps = kTileThreads / 32;
-    if (c.nr < kTileManyViews && n > 32 * kStageCols) {
+    if constexpr (InTurn) {
         for (int m = warp; m < c.nr; m += kWarps) {
             const uint32_t* src = v32 + (uint64_t)m * npix + (uint64_t)sy * c.W + sx_lo;
             for (int i = lane; i < n; i += 32)
@@ -849,8 +851,10 @@ cudaError_t launch_interleave(const DispConst& dc, const uint8_t* views, const f
     const int64_t words = tent ? dc.n_views + 5 : dc.nr, bytes = words * seg * 4;
     const dim3 tiles((dc.Wp + cols - 1) / cols, dc.H);
     if (bytes <= smem_max / 2 && (!tent || tent_pays(dc, bytes, int64_t(tiles.x) * tiles.y, sms, smem_sm))) {
-        const auto kernel = !tent ? k_interleave_tile
-                            : dc.xtalk > 0.0f ? k_interleave_tent<true> : k_interleave_tent<false>;
+        const bool in_turn = dc.nr < kTileManyViews && seg > 32 * kStageCols + 1;
+        const auto kernel = !tent            ? in_turn ? k_interleave_tile<true> : k_interleave_tile<false>
+                            : dc.xtalk > 0.0f ? k_interleave_tent<true>
+                                              : k_interleave_tent<false>;
         // the most that a tile takes, not this one's: another thread's tile may need more
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max / 2);
         if (e != cudaSuccess) return e;

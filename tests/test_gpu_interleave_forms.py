@@ -1,7 +1,8 @@
 """The interleave's forms on either side of the rules that choose between them,
 byte for byte against the oracle on views of random bytes: the tent's tiles
 (panels of many rows a view row) and the gather, with and without crosstalk;
-the Gaussian with and without its table.
+the Gaussian with and without its table; the plain tiles staged run after run
+and view after view.
 """
 import numpy as np
 import pytest
@@ -34,6 +35,21 @@ TENT = [(48, 42, 9, 512, 33, 8.0, 0.2, 1, 0.15),          # tiles: one whole str
 def test_tent_matches_oracle(case):
     d = _display(*TENT[case])
     views = _views(d, 80 + case)
+    assert np.array_equal(_panel(d, views), O.interleave(d, views))
+
+
+TILE = [(15, 129, 7, 1024, 9, 8.0, 0.2, 0, 0.0),      # view after view: the first segment longer than a run
+        (15, 128, 7, 1024, 9, 8.0, 0.2, 0, 0.0),      # run after run
+        (16, 129, 7, 1024, 9, 8.0, 0.2, 0, 0.0),
+        (15, 300, 7, 1100, 9, 8.0, 0.2, 0, 0.3),      # a last strip of few columns
+        (2, 1000, 5, 400, 3, 2.5, -0.1, 0, 0.0),      # views wider than the panel
+        (1, 1000, 5, 1000, 5, 2.5, 0.1, 0, 0.4)]
+
+
+@pytest.mark.parametrize("case", range(len(TILE)))
+def test_tiles_match_oracle(case):
+    d = _display(*TILE[case])
+    views = _views(d, 160 + case)
     assert np.array_equal(_panel(d, views), O.interleave(d, views))
 
 
